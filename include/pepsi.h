@@ -106,13 +106,14 @@ typedef struct {
                               ciphertexts [B][ell][2][k][N], every server layer one block of
                               plaintexts per request block, and the response B ciphertexts
                               [B][2][r][N], block j answering bins j*N .. j*N + N - 1 */
-  uint32_t plaintext_bytes;/* storage of the resident server plaintexts (NTT form), bytes per
-                              word: 0 or 8 = 64-bit words; 7 = the reduced value in three
-                              planes of 4, 2 and 1 bytes (every q_i < 2^56, else PEPSI_E_PARAM):
-                              12.5% more layers stay resident in the same budget, but the
-                              multiply-accumulate runs slower on a fully resident table (its
-                              unpacking costs more than the saved traffic).  Results are the
-                              same either way */
+  uint32_t plaintext_bytes;/* most bytes per word the caller allows for the resident server
+                              plaintexts (NTT form): 0 or 8, or 7 (every q_i < 2^56, else
+                              PEPSI_E_PARAM).  The storage is the same for all of them: byte
+                              planes of ceil(bits(q_i) / 8) bytes per word (at least 4; 7 for
+                              55-bit primes) with the code bits padded to a multiple of 16,
+                              or 64-bit words for codes so short that the padding would make
+                              the planes more than an eighth larger than words.  Results do
+                              not depend on it */
   uint32_t gamma;          /* client maximum bin load (Table 2, Section 4): 0 or 1 = cuckoo
                               hashing with one item per bin (the paper's evaluation); 2..16 =
                               bins of gamma slots, so up to gamma * b client items.  The client
@@ -144,7 +145,7 @@ typedef struct {
   uint32_t rescale_cap;  /* most layers one rounding may cover (1: per-layer rounding only) */
   uint32_t response_primes; /* primes of the evaluation's response (k: not switched) */
   uint32_t bins, blocks;     /* b = blocks * N bins */
-  uint32_t plaintext_bytes;  /* 7 or 8: storage of the resident server plaintexts per word */
+  uint32_t plaintext_bytes;  /* 7 or 8: as pepsi_params.plaintext_bytes asked */
   uint32_t gamma;            /* client maximum bin load: client batches per block */
 } pepsi_info;
 
@@ -200,7 +201,7 @@ typedef struct {
                            extends u, and the relinearised product is never stored;
                            0: it is stored, then the affine step runs */
   uint32_t batch_points;/* points per block of the multiply-accumulate that serves several
-                           requests with one read of the plaintexts (pepsi_eval_batch):
+                           requests with one read of regenerated plaintexts (pepsi_eval_batch):
                            0 = the default (32), 32 (16 layers per block) or 64 (8 layers:
                            longer copy rows, more re-reads of the request tiles) */
   uint32_t batch_groups;/* warp groups of that multiply-accumulate: 0 = the default (2),
@@ -275,8 +276,8 @@ int pepsi_query(pepsi_ctx* ctx, const uint64_t* items, size_t m, uint64_t enc_se
  * the response is switched); ciphertext (j, i) of the response answers
  * client batch i of request block j, its mask drawn from
  * mask_seed + j * gamma + i.  With gamma > 1 the batches of a block are
- * evaluated as by pepsi_eval_batch (shared multiply-accumulates).  A host request is uploaded in two pieces of its code bits
- * (the first short), the copy of the second overlapping the first piece's
+ * evaluated as by pepsi_eval_batch (shared multiply-accumulates).  A host request of 128 code bits or more is uploaded in two pieces of its
+ * bits (the first short), the copy of the second overlapping the first piece's
  * transform and multiply-accumulate; the words do not depend on it.  Device
  * buffers need 8-byte alignment (16-byte aligned rows take wider accesses).
  * Errors: PEPSI_E_PARAM (bad set/mode), PEPSI_E_NOMEM, PEPSI_E_CUDA. */

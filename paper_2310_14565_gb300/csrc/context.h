@@ -32,24 +32,23 @@ struct ServerSet {
   std::vector<u64> hT;          // [mu][N] host copy of T_s
   u64* dT = nullptr;            // [mu][N]
   uint16_t* dpos = nullptr;     // [mu][N][h]
-  // resident plaintexts of a prefix of the layers, [mu_res][ell][k][N]: one
-  // device array holding either 64-bit words in the split operand format, or
-  // (p7) the three planes of the 7-byte format one after another
-  void* dP = nullptr;
-  bool p7 = false;
+  // resident plaintexts of a prefix of the layers, in byte planes (kernels.h, PlaneTab) or
+  // (words) as [mu_res][ell][k][N] in the split operand format
+  unsigned char* dP = nullptr;
+  bool words = false;
   u32 mu_res = 0;               // layers [0, mu_res) resident, the rest regenerated per chunk
   bool has_values = false;      // loaded with values (labelled PSI / PSI-Sum)
   std::vector<uint32_t> hV;     // [mu][N] host copy of the value table
   u64* dVP = nullptr;           // [mu][k+kb][N] value plaintexts val_s, NTT form over Q u B
-  // the resident plaintexts as a table for the multiply-accumulate, from layer l0
-  PlainTab plain(size_t kN, int ell, u32 l0 = 0) const {
-    const size_t words = (size_t)mu_res * ell * kN, off = (size_t)l0 * ell * kN;
-    if (!p7) return plain_words(static_cast<const u64*>(dP)).at(off);
-    PlainTab t;
-    t.a = static_cast<const u32*>(dP);
-    t.b = reinterpret_cast<const uint16_t*>(t.a + words);
-    t.c = reinterpret_cast<const uint8_t*>(t.b + words);
-    return t.at(off);
+  const u64* word_table(size_t kN, int ell, u32 l0) const {
+    return reinterpret_cast<const u64*>(dP) + (size_t)l0 * ell * kN;
+  }
+  PlaneTab planes(int npl) const {
+    PlaneTab t;
+    t.p = dP;
+    t.rows = mu_res;
+    t.npl = npl;
+    return t;
   }
 };
 
@@ -113,7 +112,8 @@ struct pepsi_ctx {
   u32 rescale_cap = 1;      // most layers one rounding of the last products may cover
   bool value_margin = false;  // B also holds the value products under lazy rescaling
   int resp = 0;               // primes of the evaluation's response (k: no switching)
-  bool p7 = false;            // resident plaintexts in the 7-byte format
+  u32 plaintext_bytes = 8;    // as asked for (7 or 8); the storage is npl bytes per word either way
+  int npl = 8;                // bytes per word of the resident plaintexts: ceil(bits(q)/8), at least 4
   // per prime count r < k: modulus-switching constants and the RNS
   // constants of Q_r for decryption, built on first use
   std::unique_ptr<ModSwitchArgs> ms_args[PEPSI_MAXQ + 1];
@@ -196,10 +196,10 @@ struct Prof {
 
 // Scratch layout of the evaluation pipeline for chunks of up to Lc layers.
 struct EvalBufs {
-  u64 *C, *H, *Hc, *XB, *YB, *T3, *D, *R, *U, *W, *X, *Y, *side, *acc, *Pc, *out, *zero;
+  u64 *H, *Hc, *XB, *YB, *T3, *D, *R, *U, *W, *X, *Y, *side, *acc, *Pc, *out, *zero;
 };
 enum ScratchId { S_C, S_H, S_HC, S_XB, S_YB, S_T3, S_D, S_R, S_U, S_W, S_X, S_Y, S_SIDE, S_ACC, S_PC, S_OUT, S_ZERO,
-                 S_IN, S_DEC_Z, S_DEC_M, S_DEC_SLOTS, S_DEC_MAX, S_CT, S_POS, S_TC, S_HALL, S_COUNT };
+                 S_IN, S_DEC_Z, S_DEC_M, S_DEC_SLOTS, S_DEC_MAX, S_CT, S_POS, S_TC, S_HALL, S_CP, S_CW, S_COUNT };
 cudaError_t eval_bufs(pepsi_ctx* c, int Lc, bool need_pc, EvalBufs* b);
 
 // Operands of the last ciphertext product of the equality circuit, for L
@@ -249,8 +249,12 @@ u32 rescale_run(const pepsi_ctx* c, u32 nl, int mode);
 bool take_error_flag(pepsi_ctx* c);
 cudaError_t mac_status(cudaError_t e);
 cudaError_t copy_any(void* dst, const void* src, size_t bytes, cudaStream_t st);
-// a4: request ciphertexts (host or device) to NTT form in the split operand format, into C.
-cudaError_t prepare_request(pepsi_ctx* c, const u64* cts, u64* C, cudaStream_t st);
+// a4: request ciphertexts (host or device) to NTT form, in the formats of the
+// multiply-accumulates that will read them: `split` (request_prepared_words:
+// split operand words and half sums, for regenerated chunks) and / or `planes`
+// (request_plane_words, for resident layers); either may be null.  With planes
+// alone the NTT words go through the scratch slot S_CW.
+cudaError_t prepare_request(pepsi_ctx* c, const u64* cts, u64* split, u64* planes, cudaStream_t st);
 // a7: relinearise the layer sum, times (h!)^-1, inverse NTT, mask, response switch, copy to out.
 cudaError_t finish_request(pepsi_ctx* c, EvalBufs& b, u64* acc, bool acc_ntt, int mode, u64 mask_seed, u64* out,
                            cudaStream_t st);

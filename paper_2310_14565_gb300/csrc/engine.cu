@@ -116,11 +116,20 @@ struct pepsi_graph {
 
 namespace {
 
+// A lane of a wholly resident set keeps its requests in byte planes; one with
+// regenerated layers keeps them as split words (and makes the byte planes of a
+// resident chunk in the lane's scratch).
+bool in_planes(const Lane& L) { return L.mu_res == L.mu && !L.c->sets[L.set].words; }
+size_t prepared_words(const Lane& L) {
+  const size_t kN = (size_t)L.c->k * L.c->N;
+  return in_planes(L) ? request_plane_words(L.c->ell, kN) : request_prepared_words(L.c->ell, kN);
+}
+
 // Bytes of a request's device state on a lane (lazy: with its run sum).
 size_t request_bytes(const Lane& L, bool lazy) {
   const pepsi_ctx* c = L.c;
   const size_t kN = (size_t)c->k * c->N;
-  size_t w = request_prepared_words(c->ell, kN) + (size_t)L.Lc * 2 * kN + 3 * kN;
+  size_t w = prepared_words(L) + (size_t)L.Lc * 2 * kN + 3 * kN;
   if (lazy) w += (size_t)3 * (c->k + c->kb) * c->N;
   return w * 8;
 }
@@ -148,11 +157,12 @@ int admit(pepsi_engine* e, Lane& L, int s, u64 ticket, const Request& r, size_t 
   S.out = r.out;
   S.bytes = bytes;
   const u32 G = rescale_run(c, L.mu, r.mode);
-  cudaError_t err = pool_alloc(e, &S.C, request_prepared_words(c->ell, kN), st);
+  cudaError_t err = pool_alloc(e, &S.C, prepared_words(L), st);
   if (err == cudaSuccess) err = pool_alloc(e, &S.H, (size_t)L.Lc * 2 * kN, st);
   if (err == cudaSuccess) err = pool_alloc(e, &S.acc, 3 * kN, st);
   if (err == cudaSuccess && G > 1) err = pool_alloc(e, &S.X, (size_t)3 * (c->k + c->kb) * c->N, st);
-  if (err == cudaSuccess) err = prepare_request(c, r.cts, S.C, st);
+  if (err == cudaSuccess)
+    err = in_planes(L) ? prepare_request(c, r.cts, nullptr, S.C, st) : prepare_request(c, r.cts, S.C, nullptr, st);
   if (err != cudaSuccess) return cuda_status(err);
   if (G > 1) {
     S.lr.X = S.X;
@@ -191,22 +201,38 @@ int enqueue_step(Lane& L, Step& step, bool capturing = false) {
       act[na++] = s;
     }
   if (!na) return PEPSI_OK;
-  PlainTab P;
-  if (L.pos < L.mu_res) {
-    P = S.plain(kN, c->ell, L.pos);
+  if (L.pos < L.mu_res && in_planes(L)) {
+    for (int q0 = 0; q0 < na; q0 += c->batch_requests) {  // launches of at most batch_requests requests
+      Prof p(c, PC_MAC, st);
+      const u32* planes[kMaxSlots];
+      const int nq = std::min(c->batch_requests, na - q0);
+      for (int q = 0; q < nq; ++q) planes[q] = reinterpret_cast<const u32*>(Cs[q0 + q]);
+      launch_mac_planes(c->V, nq, planes, S.planes(c->npl), Hs + q0, c->ell, (int)L.pos, nl, c->d_err, st);
+    }
+  } else if (L.pos < L.mu_res && !S.words) {  // split words: byte planes of one request at a time
+    for (int q = 0; q < na; ++q) {
+      Prof p(c, PC_MAC, st, 2);
+      u32* planes = reinterpret_cast<u32*>(c->scratch[S_CP].p);
+      launch_pack_request(c->V, Cs[q], true, c->ell, planes, st);
+      const u32* pc = planes;
+      launch_mac_planes(c->V, 1, &pc, S.planes(c->npl), Hs + q, c->ell, (int)L.pos, nl, c->d_err, st);
+    }
   } else {
-    {
+    const u64* P = L.b.Pc;
+    if (L.pos < L.mu_res) {
+      P = S.word_table(kN, c->ell, L.pos);
+    } else {
       Prof p(c, PC_PTGEN, st);
       launch_ptgen(c->V, S.dpos + (size_t)L.pos * c->N * c->h, nl, c->ell, c->h, L.b.Pc, st);
     }
-    P = plain_words(L.b.Pc);
-  }
-  for (int q0 = 0; q0 < na; q0 += c->batch_requests) {  // launches of at most batch_requests requests
-    Prof p(c, PC_MAC, st);
-    const int nq = std::min(c->batch_requests, na - q0);
-    const cudaError_t me = mac_status(launch_mac_requests(c->V, nq, Cs + q0, P, Hs + q0, c->ell, nl, c->mac_fold,
-                                                          c->d_err, st, c->batch_points, c->batch_groups));
-    if (me != cudaSuccess) return cuda_status(me);
+    for (int q0 = 0; q0 < na; q0 += c->batch_requests) {
+      Prof p(c, PC_MAC, st);
+      const int nq = std::min(c->batch_requests, na - q0);
+      const cudaError_t me = mac_status(launch_mac_requests(c->V, nq, Cs + q0, P, Hs + q0, c->ell, nl,
+                                                            c->mac_fold, c->d_err, st, c->batch_points,
+                                                            c->batch_groups));
+      if (me != cudaSuccess) return cuda_status(me);
+    }
   }
   for (int i = 0; i < na; ++i) {
     Slot& T = L.slot[act[i]];
@@ -437,6 +463,13 @@ int pepsi_engine_create(const pepsi_lane* lanes, int nlanes, uint64_t hbm_budget
     L.nslots = (int)lanes[i].slots;
     L.Lc = balanced_chunk(L.c->chunk, L.mu);
     err = eval_bufs(L.c, L.Lc, L.mu_res < L.mu, &L.b);
+    {  // scratch of the request's preparation, before any capture: NTT words, or byte planes
+      const size_t kN = (size_t)L.c->k * L.c->N;
+      if (in_planes(L))
+        scratch(L.c, S_CW, (size_t)L.c->ell * 2 * kN * 8, &err);
+      else if (L.mu_res && !S.words)
+        scratch(L.c, S_CP, request_plane_words(L.c->ell, kN) * 8, &err);
+    }
     if (err == cudaSuccess) err = cudaHostAlloc((void**)&L.err_ring, (kStepsAhead + 1) * sizeof(int), 0);
     if (err == cudaSuccess) memset(L.err_ring, 0, (kStepsAhead + 1) * sizeof(int));
     if (err != cudaSuccess) rc = cuda_status(err);

@@ -9,7 +9,17 @@
 #include <cstring>
 
 #include "kernels.h"
+#include "mbar.cuh"
 #include "ntt_block.cuh"
+
+// SMs of the current device (cached per device).
+int sm_count() {
+  static int cached[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!cached[dev]) cudaDeviceGetAttribute(&cached[dev], cudaDevAttrMultiProcessorCount, dev);
+  return cached[dev];
+}
 
 namespace {
 
@@ -29,14 +39,6 @@ inline int ntt_threads(int N) {
 // Threads of the hot-path transform kernels: the schedule's choice
 // (DevView::nt, picked by the autotuner), else the default above.
 inline int xform_threads(const DevView& V) { return V.nt > 0 ? V.nt : ntt_threads(V.N); }
-// SMs of the current device (cached per device).
-inline int sm_count() {
-  static int cached[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!cached[dev]) cudaDeviceGetAttribute(&cached[dev], cudaDevAttrMultiProcessorCount, dev);
-  return cached[dev];
-}
 // Threads of a transform launch of `rows` blocks: a launch that gives each
 // block an SM of its own (the output stage, the lazy rounding) runs its
 // rows with up to the largest blocks instead, which shortens each
@@ -263,10 +265,12 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_valgen(DevView V, const 
 // split format (x = hi 2^s + lo, both halves below 2^32): a 64-bit product
 // is three 32x32->64 multiply-adds in Karatsuba form into three 64-bit
 // partial sums, folded into the reduced accumulator before they can
-// overflow.  The plaintext tile may also come as 7-byte words in three
-// planes (P7), put back together on the load.  Every mbarrier
+// overflow.  Every mbarrier
 // wait is bounded (about one second); on expiry the block waits, again
 // bounded, for its own copies in flight, sets *err and returns.
+// It serves the plaintext chunks regenerated at evaluation, which come as
+// 64-bit words with the points innermost; resident tables are stored in byte
+// planes for k_mac_planes.
 // Five 44 KB stages (220 KB of the 227 KB a block may hold): at the paper
 // shape a fifth stage took the launch from 12.13 to 11.94 ms, while stages
 // of 2, 3, 5 or 6 bits, or 16 layers a block, were no faster.
@@ -278,54 +282,10 @@ constexpr int THREADS = (CONSUMER_WARPS + 1) * 32;
 constexpr int P_WORDS = LB * JS * TN, C_WORDS = 2 * JS * TN;
 // A stage holds the plaintext tile, then the request tile and the request's
 // half sums (4 bytes per word, read instead of added by every layer slice).
-// The plaintext tile is 8 bytes per word (split operand format), or 7 bytes
-// per word in three planes one after another: bits 0-31, 32-47 and 48-55 of
-// the value.
-template <bool P7>
-__host__ __device__ constexpr int p_bytes() {
-  return P_WORDS * (P7 ? 7 : 8);
-}
-template <bool P7>
-__host__ __device__ constexpr int stage_bytes() {
-  return p_bytes<P7>() + C_WORDS * 12;
-}
-template <bool P7>
-__host__ __device__ constexpr size_t smem() {
-  return (size_t)NST * stage_bytes<P7>() + 2 * NST * 8 + 16 + 128;
-}
+constexpr int PB = P_WORDS * 8, SB = PB + C_WORDS * 12;
+constexpr size_t SMEM = (size_t)NST * SB + 2 * NST * 8 + 16 + 128;
 }  // namespace mac
 
-__device__ __forceinline__ u64 globaltimer_ns() {
-  u64 t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(u32 addr, u32 count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(addr), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(u32 addr, u32 bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(addr), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(u32 addr) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(addr) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(u32 addr, u32 parity) {
-  u32 ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(addr), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Wait for phase `parity` of an mbarrier for at most about one second.
-__device__ __forceinline__ bool mbar_wait_bounded(u32 addr, u32 parity) {
-  if (mbar_try_wait(addr, parity)) return true;
-  const u64 t0 = globaltimer_ns();
-  while (!mbar_try_wait(addr, parity))
-    if (globaltimer_ns() - t0 > 1000000000ull) return false;
-  return true;
-}
 __device__ __forceinline__ void tma_load_3d(u32 dst, const CUtensorMap* tm, int c0, int c1, int c2, u32 bar) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
@@ -389,45 +349,10 @@ __device__ __forceinline__ void fold_into(u64& acc, u64& S0, u64& SM, u64& S2, u
   S0 = SM = S2 = 0;
 }
 
-// Plaintext word o of a stage's tile as split operands xl = x mod 2^s,
-// xh = x >> s.  P7: x is put together from its three planes.
-template <bool P7>
-__device__ __forceinline__ void tile_word(const unsigned char* stg, int o, u32 s, u32 lmask, u32& xl, u32& xh) {
-  if constexpr (P7) {
-    const u32 a = reinterpret_cast<const u32*>(stg)[o];
-    const u32 b = reinterpret_cast<const uint16_t*>(stg + mac::P_WORDS * 4)[o];
-    const u32 c = stg[mac::P_WORDS * 6 + o];
-    const u32 hi = __byte_perm(b, c, 0x2410);  // b | c << 16: bits 32-55 of x
-    xl = a & lmask;
-    xh = __funnelshift_r(a, hi, s);
-  } else {
-    const u64 x = reinterpret_cast<const u64*>(stg)[o];
-    xl = (u32)x;
-    xh = (u32)(x >> 32);
-  }
-}
-// The stage's plaintext copies: one tensor copy of the words, or one per plane.
-template <bool P7>
-__device__ __forceinline__ void tma_plain(u32 sb, const CUtensorMap* tmP, const CUtensorMap* tmPb,
-                                          const CUtensorMap* tmPc, int x, int j, int l, u32 bar) {
-  tma_load_3d(sb, tmP, x, j, l, bar);
-  if constexpr (P7) {
-    tma_load_3d(sb + mac::P_WORDS * 4, tmPb, x, j, l, bar);
-    tma_load_3d(sb + mac::P_WORDS * 6, tmPc, x, j, l, bar);
-  }
-}
-
-// One launch covers the codeword bits [j0, j0 + nj) (nj a multiple of JS
-// unless the range ends at ell); with acc_in it adds to the h' already in
-// H, so a request can be multiplied in pieces as it arrives.
-template <bool P7>
 __global__ void __launch_bounds__(mac::THREADS, 1)
-    k_mac(DevView V, const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmPb,
-          const __grid_constant__ CUtensorMap tmPc, const __grid_constant__ CUtensorMap tmC,
-          const __grid_constant__ CUtensorMap tmS, u64* __restrict__ H, int j0, int nj, int L, int fold_stages,
-          int acc_in, int* err) {
+    k_mac(DevView V, const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmC,
+          const __grid_constant__ CUtensorMap tmS, u64* __restrict__ H, int ell, int L, int fold_stages, int* err) {
   using namespace mac;
-  constexpr int SB = stage_bytes<P7>(), PB = p_bytes<P7>();
   extern __shared__ __align__(128) u64 sm_raw[];
   // 128-byte aligned stage buffers for the tensor copies, derived from the
   // shared array by pointer arithmetic so that its loads stay shared-memory
@@ -438,7 +363,7 @@ __global__ void __launch_bounds__(mac::THREADS, 1)
   const int nl = min(LB, L - l0);
   const size_t idx0 = (size_t)blockIdx.y * TN;
   const int cnt = (int)min((size_t)TN, kN - idx0);
-  const int nst = (nj + JS - 1) / JS;
+  const int nst = (ell + JS - 1) / JS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const u32 sbase = (u32)__cvta_generic_to_shared(sm);
   const u32 full0 = sbase + (u32)(NST * SB), empty0 = full0 + NST * 8;
@@ -470,9 +395,9 @@ __global__ void __launch_bounds__(mac::THREADS, 1)
         const u32 sb = sbase + (u32)(buf * SB);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_expect_tx(bar, (u32)SB);
-        tma_plain<P7>(sb, &tmP, &tmPb, &tmPc, (int)idx0, j0 + st * JS, l0, bar);
-        tma_load_3d(sb + (u32)PB, &tmC, (int)idx0, 0, j0 + st * JS, bar);
-        tma_load_3d(sb + (u32)(PB + C_WORDS * 8), &tmS, (int)idx0, 0, j0 + st * JS, bar);
+        tma_load_3d(sb, &tmP, (int)idx0, st * JS, l0, bar);
+        tma_load_3d(sb + (u32)PB, &tmC, (int)idx0, 0, st * JS, bar);
+        tma_load_3d(sb + (u32)(PB + C_WORDS * 8), &tmS, (int)idx0, 0, st * JS, bar);
         issued = st + 1;
       }
     }
@@ -484,16 +409,11 @@ __global__ void __launch_bounds__(mac::THREADS, 1)
     const size_t idx = idx0 + (active ? tp : 0);
     const DevPrime pr = V.pr[idx / V.N];
     const u64 sp = pr.split;
-    const u32 s32 = (u32)sp, lmask = (1u << s32) - 1;
     u64 S0[LPT][2], SM[LPT][2], S2[LPT][2], acc[LPT][2];
 #pragma unroll
     for (int l = 0; l < LPT; ++l)
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        S0[l][c] = SM[l][c] = S2[l][c] = acc[l][c] = 0;
-        const int layer = g * LPT + l;
-        if (acc_in && active && layer < nl) acc[l][c] = H[((size_t)(l0 + layer) * 2 + c) * kN + idx];
-      }
+      for (int c = 0; c < 2; ++c) S0[l][c] = SM[l][c] = S2[l][c] = acc[l][c] = 0;
     int since = 0;
     for (int st = 0; st < nst; ++st) {
       const int buf = st % NST;
@@ -502,7 +422,7 @@ __global__ void __launch_bounds__(mac::THREADS, 1)
         break;
       }
       const unsigned char* stg = sm + (size_t)buf * SB;
-      const int po = g * LPT * JS * TN + tp;  // word (slice, bit 0, point) of the tile
+      const u64* ps = reinterpret_cast<const u64*>(stg) + g * LPT * JS * TN + tp;  // (slice, bit 0, point)
       const u64* cs = reinterpret_cast<const u64*>(stg + PB) + tp;
       const u32* ss = reinterpret_cast<const u32*>(stg + PB + C_WORDS * 8) + tp;
 #pragma unroll
@@ -512,9 +432,8 @@ __global__ void __launch_bounds__(mac::THREADS, 1)
         const u32 c0s = ss[(jj * 2) * TN], c1s = ss[(jj * 2 + 1) * TN];
 #pragma unroll
         for (int l = 0; l < LPT; ++l) {
-          u32 xl, xh;
-          tile_word<P7>(stg, po + (l * JS + jj) * TN, s32, lmask, xl, xh);
-          const u32 xs = xl + xh;
+          const u64 x = ps[(l * JS + jj) * TN];
+          const u32 xl = (u32)x, xh = (u32)(x >> 32), xs = xl + xh;
           kmac(S0[l][0], SM[l][0], S2[l][0], c0l, c0h, c0s, xl, xh, xs);
           kmac(S0[l][1], SM[l][1], S2[l][1], c1l, c1h, c1s, xl, xh, xs);
         }
@@ -586,71 +505,31 @@ struct Tile {
   static constexpr int P_WORDS = LB * JS * TN;
   static_assert(LG * WPS == GROUP_WARPS, "whole layer slices");
 };
-template <int QB, int WPS, bool P7>
-__host__ __device__ constexpr int p_bytes() {
-  return Tile<WPS>::P_WORDS * (P7 ? 7 : 8);
-}
 // request q's tile of split words, then its tile of half sums
 template <int WPS>
 __host__ __device__ constexpr int req_bytes() {
   return 2 * JS * Tile<WPS>::TN * 12;
 }
-template <int QB, int WPS, bool P7>
+template <int QB, int WPS>
 __host__ __device__ constexpr int stage_bytes() {
-  return p_bytes<QB, WPS, P7>() + QB * req_bytes<WPS>();
+  return Tile<WPS>::P_WORDS * 8 + QB * req_bytes<WPS>();
 }
-template <int QB, int WPS, bool P7>
+template <int QB, int WPS>
 __host__ __device__ constexpr size_t smem() {
-  return (size_t)NST * stage_bytes<QB, WPS, P7>() + 2 * NST * 8 + 16 + 128;
+  return (size_t)NST * stage_bytes<QB, WPS>() + 2 * NST * 8 + 16 + 128;
 }
 }  // namespace macq
 
-__device__ __forceinline__ void tma_load_4d(u32 dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, u32 bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
-      "[%6];" ::"r"(dst),
-      "l"(reinterpret_cast<u64>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-      : "memory");
-}
-
-// Plaintext word o of a stage tile of PW words (see tile_word), and the
-// stage's plaintext copies for that tile size.
-template <bool P7, int PW>
-__device__ __forceinline__ void tile_word_pw(const unsigned char* stg, int o, u32 s, u32 lmask, u32& xl, u32& xh) {
-  if constexpr (P7) {
-    const u32 a = reinterpret_cast<const u32*>(stg)[o];
-    const u32 b = reinterpret_cast<const uint16_t*>(stg + PW * 4)[o];
-    const u32 c = stg[PW * 6 + o];
-    const u32 hi = __byte_perm(b, c, 0x2410);
-    xl = a & lmask;
-    xh = __funnelshift_r(a, hi, s);
-  } else {
-    const u64 x = reinterpret_cast<const u64*>(stg)[o];
-    xl = (u32)x;
-    xh = (u32)(x >> 32);
-  }
-}
-template <bool P7, int PW>
-__device__ __forceinline__ void tma_plain_pw(u32 sb, const CUtensorMap* tmP, const CUtensorMap* tmPb,
-                                             const CUtensorMap* tmPc, int x, int j, int l, u32 bar) {
-  tma_load_3d(sb, tmP, x, j, l, bar);
-  if constexpr (P7) {
-    tma_load_3d(sb + PW * 4, tmPb, x, j, l, bar);
-    tma_load_3d(sb + PW * 6, tmPc, x, j, l, bar);
-  }
-}
-
-template <int QB, int RG, int WPS, bool P7>
+template <int QB, int RG, int WPS>
 __global__ void __launch_bounds__(macq::threads(RG), 1)
-    k_mac_multi(DevView V, const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmPb,
-                const __grid_constant__ CUtensorMap tmPc, const __grid_constant__ MacRequests rq, int ell, int L,
-                int fold_stages, int* err) {
+    k_mac_multi(DevView V, const __grid_constant__ CUtensorMap tmP, const __grid_constant__ MacRequests rq, int ell,
+                int L, int fold_stages, int* err) {
   using namespace macq;
   using TL = Tile<WPS>;
   constexpr int CONSUMER_WARPS = GROUP_WARPS * RG, QT = QB / RG;  // QT requests per consumer thread
   static_assert(QT * RG == QB, "whole request groups");
   constexpr int TN = TL::TN, LB = TL::LB, PW = TL::P_WORDS;
-  constexpr int SB = stage_bytes<QB, WPS, P7>(), PB = p_bytes<QB, WPS, P7>();
+  constexpr int SB = stage_bytes<QB, WPS>(), PB = PW * 8;
   extern __shared__ __align__(128) u64 sm_raw[];
   unsigned char* sm = stage_base(sm_raw);
   const size_t kN = (size_t)V.k * V.N;
@@ -692,7 +571,7 @@ __global__ void __launch_bounds__(macq::threads(RG), 1)
         const u32 sb = sbase + (u32)(buf * SB);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_expect_tx(bar, (u32)SB);
-        tma_plain_pw<P7, PW>(sb, &tmP, &tmPb, &tmPc, (int)idx0, st * JS, l0, bar);
+        tma_load_3d(sb, &tmP, (int)idx0, st * JS, l0, bar);
 #pragma unroll
         for (int q = 0; q < QB; ++q) {
           const u32 rb = sb + (u32)(PB + q * req_bytes<WPS>());
@@ -710,7 +589,6 @@ __global__ void __launch_bounds__(macq::threads(RG), 1)
     const size_t idx = idx0 + (active ? tp : 0);
     const DevPrime pr = V.pr[idx / V.N];
     const u64 sp = pr.split;
-    const u32 s32 = (u32)sp, lmask = (1u << s32) - 1;
     u64 S0[LPT][QT][2], SM[LPT][QT][2], S2[LPT][QT][2];
 #pragma unroll
     for (int l = 0; l < LPT; ++l)
@@ -726,14 +604,16 @@ __global__ void __launch_bounds__(macq::threads(RG), 1)
         break;
       }
       const unsigned char* stg = sm + (size_t)buf * SB;
-      const int po = g * LPT * JS * TN + tp;  // word (slice, bit 0, point) of the plaintext tile
+      const u64* ps = reinterpret_cast<const u64*>(stg) + g * LPT * JS * TN + tp;  // (slice, bit 0, point)
       const unsigned char* rqt = stg + PB + rg * QT * req_bytes<WPS>();  // this group's request tiles
 #pragma unroll
       for (int jj = 0; jj < JS; ++jj) {
         u32 xl[LPT], xh[LPT], xs[LPT];
 #pragma unroll
         for (int l = 0; l < LPT; ++l) {
-          tile_word_pw<P7, PW>(stg, po + (l * JS + jj) * TN, s32, lmask, xl[l], xh[l]);
+          const u64 x = ps[(l * JS + jj) * TN];
+          xl[l] = (u32)x;
+          xh[l] = (u32)(x >> 32);
           xs[l] = xl[l] + xh[l];
         }
 #pragma unroll
@@ -790,25 +670,6 @@ __global__ void k_split(DevView V, u64* x, size_t total, int to) {
   if (i >= total) return;
   const u64 s = V.pr[(i / V.N) % V.k].split;
   x[i] = to ? to_split(x[i], s) : from_split(x[i], s);
-}
-
-// Split-format words of rows [..][k][N] (row r uses prime r % k) to the
-// three planes of the 7-byte format: bits 0-31, 32-47 and 48-55 of each
-// reduced value (every prime below 2^56).
-__global__ void k_pack7(DevView V, const u64* __restrict__ src, size_t count, u32* a, uint16_t* b, uint8_t* c) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  const u64 x = from_split(src[i], V.pr[(i / V.N) % V.k].split);
-  a[i] = (u32)x;
-  b[i] = (uint16_t)(x >> 32);
-  c[i] = (uint8_t)(x >> 48);
-}
-// The reduced values back from the three planes.
-__global__ void k_unpack7(const u32* __restrict__ a, const uint16_t* __restrict__ b, const uint8_t* __restrict__ c,
-                          size_t count, u64* out) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  out[i] = (u64)a[i] | ((u64)b[i] << 32) | ((u64)c[i] << 48);
 }
 
 // ---------------------------------------------------- RNS conversions
@@ -1572,70 +1433,45 @@ bool encode3d_t(CUtensorMap* tm, CUtensorMapDataType dt, int esz, const void* ba
 bool encode3d(CUtensorMap* tm, const u64* base, u64 d0, u64 d1, u64 d2, u64 s1, u64 s2, u32 b0, u32 b1, u32 b2) {
   return encode3d_t(tm, CU_TENSOR_MAP_DATA_TYPE_UINT64, 8, base, d0, d1, d2, s1, s2, b0, b1, b2);
 }
-// Tensor maps of the plaintext tiles of L layers [L][ell][kN]: tm[0] the words, or
-// tm[0..2] the three planes of the 7-byte format (tm[1], tm[2] copies of tm[0] otherwise).
-bool encode_plain(CUtensorMap tm[3], const PlainTab& P, u64 kN, int ell, int L, u32 tn, u32 js, u32 lb) {
-  const u64 s2 = (u64)ell * kN;
-  if (!P.packed()) {
-    if (!encode3d(&tm[0], P.w, kN, ell, L, kN, s2, tn, js, lb)) return false;
-    tm[1] = tm[2] = tm[0];
-    return true;
-  }
-  return encode3d_t(&tm[0], CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, P.a, kN, ell, L, kN, s2, tn, js, lb) &&
-         encode3d_t(&tm[1], CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, P.b, kN, ell, L, kN, s2, tn, js, lb) &&
-         encode3d_t(&tm[2], CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, P.c, kN, ell, L, kN, s2, tn, js, lb);
-}
-bool encode4d(CUtensorMap* tm, const u64* base, u64 d0, u64 d1, u64 d2, u64 d3, u64 s1, u64 s2, u64 s3, u32 b0,
-              u32 b1, u32 b2, u32 b3) {
-  auto enc = tensor_map_encoder();
-  if (!enc) return false;
-  const cuuint64_t dims[4] = {d0, d1, d2, d3};
-  const cuuint64_t strides[3] = {s1 * 8, s2 * 8, s3 * 8};
-  const cuuint32_t box[4] = {b0, b1, b2, b3};
-  const cuuint32_t estr[4] = {1, 1, 1, 1};
-  return enc(tm, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<u64*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 }  // namespace
 
 namespace {
-template <int QB, int RG, int WPS, bool P7>
-void mac_multi_go(const DevView& V, const CUtensorMap (&tmP)[3], const MacRequests& rq, int ell, int L,
-                  int fold_stages, int* err, cudaStream_t st) {
+template <int QB, int RG, int WPS>
+void mac_multi_go(const DevView& V, const CUtensorMap& tmP, const MacRequests& rq, int ell, int L, int fold_stages,
+                  int* err, cudaStream_t st) {
   using TL = macq::Tile<WPS>;
   const u64 kN = (u64)V.k * V.N;
   dim3 grid((L + TL::LB - 1) / TL::LB, (unsigned)((kN + TL::TN - 1) / TL::TN));
-  k_mac_multi<QB, RG, WPS, P7><<<grid, macq::threads(RG), macq::smem<QB, WPS, P7>(), st>>>(
-      V, tmP[0], tmP[1], tmP[2], rq, ell, L, fold_stages, err);
+  k_mac_multi<QB, RG, WPS><<<grid, macq::threads(RG), macq::smem<QB, WPS>(), st>>>(V, tmP, rq, ell, L, fold_stages,
+                                                                                   err);
 }
 // groups: 1 = every consumer thread serves all requests; 2 = two groups of
 // warps serve half of them each (2 or 4 requests)
-template <int WPS, bool P7>
-void mac_multi_q(int nq, int groups, const DevView& V, const CUtensorMap (&tmP)[3], const MacRequests& rq, int ell,
-                 int L, int fold_stages, int* err, cudaStream_t st) {
+template <int WPS>
+void mac_multi_q(int nq, int groups, const DevView& V, const CUtensorMap& tmP, const MacRequests& rq, int ell, int L,
+                 int fold_stages, int* err, cudaStream_t st) {
   switch (nq * 4 + (groups == 2 && nq != 3 ? 2 : 1)) {
-    case 2 * 4 + 1: mac_multi_go<2, 1, WPS, P7>(V, tmP, rq, ell, L, fold_stages, err, st); break;
-    case 2 * 4 + 2: mac_multi_go<2, 2, WPS, P7>(V, tmP, rq, ell, L, fold_stages, err, st); break;
-    case 3 * 4 + 1: mac_multi_go<3, 1, WPS, P7>(V, tmP, rq, ell, L, fold_stages, err, st); break;
-    case 4 * 4 + 1: mac_multi_go<4, 1, WPS, P7>(V, tmP, rq, ell, L, fold_stages, err, st); break;
-    default: mac_multi_go<4, 2, WPS, P7>(V, tmP, rq, ell, L, fold_stages, err, st); break;
+    case 2 * 4 + 1: mac_multi_go<2, 1, WPS>(V, tmP, rq, ell, L, fold_stages, err, st); break;
+    case 2 * 4 + 2: mac_multi_go<2, 2, WPS>(V, tmP, rq, ell, L, fold_stages, err, st); break;
+    case 3 * 4 + 1: mac_multi_go<3, 1, WPS>(V, tmP, rq, ell, L, fold_stages, err, st); break;
+    case 4 * 4 + 1: mac_multi_go<4, 1, WPS>(V, tmP, rq, ell, L, fold_stages, err, st); break;
+    default: mac_multi_go<4, 2, WPS>(V, tmP, rq, ell, L, fold_stages, err, st); break;
   }
 }
 }  // namespace
 
-cudaError_t launch_mac_requests(const DevView& V, int nq, const u64* const* C, const PlainTab& P, u64* const* H,
-                                int ell, int L, int fold, int* err, cudaStream_t st, int tile_points, int groups) {
+cudaError_t launch_mac_requests(const DevView& V, int nq, const u64* const* C, const u64* P, u64* const* H, int ell,
+                                int L, int fold, int* err, cudaStream_t st, int tile_points, int groups) {
   if (L <= 0 || nq <= 0) return cudaSuccess;
   if (nq > macq::QMAX || (tile_points != 32 && tile_points != 64)) return cudaErrorInvalidValue;
   if (nq == 1) return launch_mac(V, C[0], P, H[0], ell, L, fold, err, st);  // one request: the single-request kernel
   const u64 kN = (u64)V.k * V.N;
   const int wps = tile_points / 32;
   const u32 tn = (u32)tile_points, lb = (u32)(macq::GROUP_WARPS / wps * macq::LPT);
-  CUtensorMap tmP[3];
+  CUtensorMap tmP;
   MacRequests rq;
   memset(&rq, 0, sizeof(rq));
-  if (!encode_plain(tmP, P, kN, ell, L, tn, macq::JS, lb)) return cudaErrorInvalidValue;
+  if (!encode3d(&tmP, P, kN, ell, L, kN, (u64)ell * kN, tn, macq::JS, lb)) return cudaErrorInvalidValue;
   for (int q = 0; q < nq; ++q) {
     if (!encode3d(&rq.c[q], C[q], kN, 2, ell, kN, 2 * kN, tn, 2, macq::JS) ||
         !encode3d_t(&rq.s[q], CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, request_sums(C[q], ell, kN), kN, 2, ell, kN, 2 * kN, tn,
@@ -1644,63 +1480,27 @@ cudaError_t launch_mac_requests(const DevView& V, int nq, const u64* const* C, c
     rq.h[q] = H[q];
   }
   const int fold_stages = fold / macq::JS > 0 ? fold / macq::JS : 1;
-  if (wps == 1) {
-    if (P.packed())
-      mac_multi_q<1, true>(nq, groups, V, tmP, rq, ell, L, fold_stages, err, st);
-    else
-      mac_multi_q<1, false>(nq, groups, V, tmP, rq, ell, L, fold_stages, err, st);
-  } else {
-    if (P.packed())
-      mac_multi_q<2, true>(nq, groups, V, tmP, rq, ell, L, fold_stages, err, st);
-    else
-      mac_multi_q<2, false>(nq, groups, V, tmP, rq, ell, L, fold_stages, err, st);
-  }
+  if (wps == 1)
+    mac_multi_q<1>(nq, groups, V, tmP, rq, ell, L, fold_stages, err, st);
+  else
+    mac_multi_q<2>(nq, groups, V, tmP, rq, ell, L, fold_stages, err, st);
   return cudaSuccess;
 }
 
-cudaError_t launch_mac_multi(const DevView& V, const u64* C, int nq, const PlainTab& P, u64* H, size_t hq, int ell,
-                             int L, int fold, int* err, cudaStream_t st, int tile_points, int groups) {
-  if (nq <= 0 || nq > macq::QMAX) return nq <= 0 ? cudaSuccess : cudaErrorInvalidValue;
-  const u64* cq[macq::QMAX];
-  u64* hqv[macq::QMAX];
-  for (int q = 0; q < nq; ++q) {
-    cq[q] = C + (size_t)q * request_prepared_words(ell, (size_t)V.k * V.N);
-    hqv[q] = H + (size_t)q * hq;
-  }
-  return launch_mac_requests(V, nq, cq, P, hqv, ell, L, fold, err, st, tile_points, groups);
-}
-
-cudaError_t launch_mac(const DevView& V, const u64* C, const PlainTab& P, u64* H, int ell, int L, int fold, int* err,
-                       cudaStream_t st, int j0, int nj, bool acc_in) {
+cudaError_t launch_mac(const DevView& V, const u64* C, const u64* P, u64* H, int ell, int L, int fold, int* err,
+                       cudaStream_t st) {
   if (L <= 0) return cudaSuccess;
-  if (nj < 0) nj = ell - j0;
-  if (j0 < 0 || nj <= 0 || j0 + nj > ell || (j0 % mac::JS) || (j0 + nj < ell && nj % mac::JS))
-    return cudaErrorInvalidValue;
   const u64 kN = (u64)V.k * V.N;
-  CUtensorMap tmP[3], tmC, tmS;
-  if (!encode_plain(tmP, P, kN, ell, L, mac::TN, mac::JS, mac::LB) ||
+  CUtensorMap tmP, tmC, tmS;
+  if (!encode3d(&tmP, P, kN, ell, L, kN, (u64)ell * kN, mac::TN, mac::JS, mac::LB) ||
       !encode3d(&tmC, C, kN, 2, ell, kN, 2 * kN, mac::TN, 2, mac::JS) ||
       !encode3d_t(&tmS, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, request_sums(C, ell, kN), kN, 2, ell, kN, 2 * kN, mac::TN, 2,
                   mac::JS))
     return cudaErrorInvalidValue;
   const int fold_stages = fold / mac::JS > 0 ? fold / mac::JS : 1;
   dim3 grid((L + mac::LB - 1) / mac::LB, (unsigned)((kN + mac::TN - 1) / mac::TN));
-  if (P.packed())
-    k_mac<true><<<grid, mac::THREADS, mac::smem<true>(), st>>>(V, tmP[0], tmP[1], tmP[2], tmC, tmS, H, j0, nj, L,
-                                                               fold_stages, acc_in ? 1 : 0, err);
-  else
-    k_mac<false><<<grid, mac::THREADS, mac::smem<false>(), st>>>(V, tmP[0], tmP[1], tmP[2], tmC, tmS, H, j0, nj, L,
-                                                                 fold_stages, acc_in ? 1 : 0, err);
+  k_mac<<<grid, mac::THREADS, mac::SMEM, st>>>(V, tmP, tmC, tmS, H, ell, L, fold_stages, err);
   return cudaSuccess;
-}
-
-void launch_pack7(const DevView& V, const u64* src, size_t count, u32* a, uint16_t* b, uint8_t* c, cudaStream_t st) {
-  if (!count) return;
-  k_pack7<<<grid_for(count, 256), 256, 0, st>>>(V, src, count, a, b, c);
-}
-void launch_unpack7(const u32* a, const uint16_t* b, const uint8_t* c, size_t count, u64* out, cudaStream_t st) {
-  if (!count) return;
-  k_unpack7<<<grid_for(count, 256), 256, 0, st>>>(a, b, c, count, out);
 }
 
 void launch_split(const DevView& V, u64* x, size_t groups, bool to, cudaStream_t st) {
@@ -1900,13 +1700,10 @@ cudaError_t kernels_init(int N) {
   set((const void*)k_ntt<true, true>);
   set((const void*)k_ptgen);
   set((const void*)k_valgen);
-  set((const void*)k_mac<false>);
-  set((const void*)k_mac<true>);
-#define PEPSI_SET_MACQ(QB, RG)                         \
-  set((const void*)k_mac_multi<QB, RG, 1, false>);     \
-  set((const void*)k_mac_multi<QB, RG, 1, true>);      \
-  set((const void*)k_mac_multi<QB, RG, 2, false>);     \
-  set((const void*)k_mac_multi<QB, RG, 2, true>);
+  set((const void*)k_mac);
+#define PEPSI_SET_MACQ(QB, RG)               \
+  set((const void*)k_mac_multi<QB, RG, 1>);  \
+  set((const void*)k_mac_multi<QB, RG, 2>);
   PEPSI_SET_MACQ(2, 1)
   PEPSI_SET_MACQ(2, 2)
   PEPSI_SET_MACQ(3, 1)
@@ -1925,6 +1722,7 @@ cudaError_t kernels_init(int N) {
   set((const void*)k_dec_z);
   set((const void*)k_dec_slots);
   set((const void*)k_mask);
+  if (e == cudaSuccess) e = mac_planes_init();
   return e;
 }
 

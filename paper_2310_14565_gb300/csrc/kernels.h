@@ -38,58 +38,57 @@ void launch_cw_unrank(const u64* T, size_t count, const u64* binom, int ell, int
 // Server plaintexts pt_s[l][j] in NTT form for L layers: P[L][ell][k][N], split operand format.
 void launch_ptgen(const DevView& V, const uint16_t* pos, int L, int ell, int h, u64* P, cudaStream_t st);
 
-// Plaintexts of L layers [L][ell][k][N]: either 64-bit words in the split
-// operand format (w), or 7-byte words of the reduced values in three planes of
-// the same shape (a: bits 0-31, b: bits 32-47, c: bits 48-55; every prime below
-// 2^56).  Each base is 16-byte aligned.
-struct PlainTab {
-  const u64* w = nullptr;
-  const u32* a = nullptr;
-  const uint16_t* b = nullptr;
-  const uint8_t* c = nullptr;
-  bool packed() const { return a != nullptr; }
-  // the table from word `off` on (a whole number of layers)
-  PlainTab at(size_t off) const {
-    PlainTab r;
-    if (packed()) {
-      r.a = a + off;
-      r.b = b + off;
-      r.c = c + off;
-    } else {
-      r.w = w + off;
-    }
-    return r;
-  }
-};
-inline PlainTab plain_words(const u64* w) {
-  PlainTab r;
-  r.w = w;
-  return r;
-}
+// SMs of the current device.
+int sm_count();
 
-// Fused ct x pt multiply-accumulate: H[l][c][p][n] = sum_j C[j][c][p][n] * P[l][j][p][n] mod q_p.
-// C a prepared request (split operand format and half sums), H reduced.  fold: terms between folds of the
+// A resident server table in byte planes (mac_planes.cu): `rows` layers of npl
+// bytes per word (npl = ceil(bits(q) / 8) of the widest q_i, 4..8), code bits
+// padded to whole steps of 16.
+struct PlaneTab {
+  unsigned char* p = nullptr;  // 16-byte aligned
+  u32 rows = 0;
+  int npl = 0;
+};
+inline int plane_steps(int ell) { return (ell + 15) / 16; }
+inline size_t plane_layer_bytes(int ell, size_t kN, int npl) { return (size_t)plane_steps(ell) * kN * 16 * npl; }
+// Whether a resident table is kept in byte planes, else as 64-bit words: the
+// planes' steps of 16 bits make a short code's table larger (24 bits in 7 planes:
+// 224 bytes per point and layer against 192), and its few bits do not pay for
+// the sums and reductions of an item.  The line allows planes an eighth more
+// bytes.  At 24 bits, 526 layers, N = 8192, k = 4
+// the multiply-accumulate took 1.22 ms on planes and 0.77 ms on words.
+inline bool table_in_planes(int ell, int npl) { return 8 * (size_t)plane_steps(ell) * 16 * npl <= 9 * (size_t)ell * 8; }
+// 64-bit words of a request in byte planes
+inline size_t request_plane_words(int ell, size_t kN) { return (size_t)plane_steps(ell) * kN * 32; }
+// H[q][l][c][p][n] = sum_j C[q][j][c][p][n] * P[l0 + l][j][p][n] mod q_p for nl layers of the table
+// and nq <= PEPSI_MAC_MAX_REQUESTS requests in byte planes, over the steps [ks0, ks1) (-1: all);
+// acc_in adds to the h' already in H.  *err is set when a bounded wait for a copy expires.
+void launch_mac_planes(const DevView& V, int nq, const u32* const* C, const PlaneTab& P, u64* const* H, int ell, int l0,
+                       int nl, int* err, cudaStream_t st, int ks0 = 0, int ks1 = -1, bool acc_in = false);
+// Split-format words [nl][ell][k][N] of layers l0.. into the table, and reduced values back from it.
+void launch_pack_planes(const DevView& V, const u64* words, int ell, int l0, int nl, const PlaneTab& P, cudaStream_t st);
+void launch_unpack_planes(const DevView& V, const PlaneTab& P, int ell, int l0, int nl, u64* out, cudaStream_t st);
+// Request words [ell][2][k][N] (reduced, or split format) to byte planes, steps [ks0, ks1) (-1: all).
+void launch_pack_request(const DevView& V, const u64* words, bool split, int ell, u32* C, cudaStream_t st, int ks0 = 0,
+                         int ks1 = -1);
+// Shared-memory limits of the kernels above (called by kernels_init).
+cudaError_t mac_planes_init();
+
+// Fused ct x pt multiply-accumulate of a regenerated chunk: H[l][c][p][n] = sum_j C[j][c][p][n] *
+// P[l][j][p][n] mod q_p.  C a prepared request (split operand format and half sums), P [L][ell][k][N] in the
+// split operand format, H reduced.  fold: terms between folds of the
 // 64-bit partial sums.  *err is set when a bounded wait for a TMA copy expires.
 // Returns cudaErrorInvalidValue when the tensor maps of the copies cannot be encoded.
-cudaError_t launch_mac(const DevView& V, const u64* C, const PlainTab& P, u64* H, int ell, int L, int fold, int* err,
-                       cudaStream_t st, int j0 = 0, int nj = -1, bool acc_in = false);
+cudaError_t launch_mac(const DevView& V, const u64* C, const u64* P, u64* H, int ell, int L, int fold, int* err,
+                       cudaStream_t st);
 
 // The same for nq <= PEPSI_MAC_MAX_REQUESTS requests sharing the plaintexts: prepared request q
 // at C[q], its h' [L][2][k][N] to H[q].  tile_points: 32
 // or 64 points per block (16 or 8 layers); groups: 1 = each consumer thread serves every
 // request, 2 = two groups of warps serve half of them each (2 or 4 requests; 3 requests
 // always run in one group); one request runs launch_mac.
-cudaError_t launch_mac_requests(const DevView& V, int nq, const u64* const* C, const PlainTab& P, u64* const* H,
-                                int ell, int L, int fold, int* err, cudaStream_t st, int tile_points = 32,
-                                int groups = 2);
-// The same with the prepared requests back to back in C (request_prepared_words apart) and H[q]
-// at H + q * hq.
-cudaError_t launch_mac_multi(const DevView& V, const u64* C, int nq, const PlainTab& P, u64* H, size_t hq, int ell,
-                             int L, int fold, int* err, cudaStream_t st, int tile_points = 32, int groups = 2);
-// count split-format words (rows [..][k][N]) to the three planes of the 7-byte format, and back
-// (reduced values)
-void launch_pack7(const DevView& V, const u64* src, size_t count, u32* a, uint16_t* b, uint8_t* c, cudaStream_t st);
-void launch_unpack7(const u32* a, const uint16_t* b, const uint8_t* c, size_t count, u64* out, cudaStream_t st);
+cudaError_t launch_mac_requests(const DevView& V, int nq, const u64* const* C, const u64* P, u64* const* H, int ell,
+                                int L, int fold, int* err, cudaStream_t st, int tile_points = 32, int groups = 2);
 constexpr int PEPSI_MAC_MAX_REQUESTS = 4;
 // Per-request operands of the multi-request multiply-accumulate (passed by value).
 struct MacRequests {

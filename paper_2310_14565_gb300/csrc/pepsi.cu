@@ -185,7 +185,6 @@ cudaError_t eval_bufs(pepsi_ctx* c, int Lc, bool need_pc, EvalBufs* b) {
   cudaError_t e = cudaSuccess;
   const size_t N = c->N, k = c->k, kb = c->kb, np = k + kb;
   auto get = [&](int id, size_t words) { return (u64*)scratch(c, id, words * 8, &e); };
-  b->C = get(S_C, request_prepared_words(c->ell, k * N));
   b->H = get(S_H, Lc * 2 * k * N);
   b->Hc = get(S_HC, Lc * 2 * k * N);
   b->XB = get(S_XB, Lc * 2 * kb * N);
@@ -337,18 +336,20 @@ cudaError_t copy_any(void* dst, const void* src, size_t bytes, cudaStream_t st) 
   return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, st);
 }
 
-// a4: request ciphertexts (host or device) to NTT form, then to the split
-// operand format of the multiply-accumulate with the sums of the halves,
-// into C (request_prepared_words).
-cudaError_t prepare_request(pepsi_ctx* c, const u64* cts, u64* C, cudaStream_t st) {
+cudaError_t prepare_request(pepsi_ctx* c, const u64* cts, u64* split, u64* planes, cudaStream_t st) {
   const size_t kN = (size_t)c->k * c->N, words = (size_t)c->ell * 2 * kN;
+  cudaError_t e = cudaSuccess;
+  u64* C = split ? split : (u64*)scratch(c, S_CW, words * 8, &e);
+  if (!C) return e;
   const u64* src = cts;
   if (!is_device_ptr(cts)) {
     CK(copy_any(C, cts, words * 8, st));
     src = C;
   }
-  Prof p(c, PC_NTT, st);  // forward NTT, stored in the split operand format
-  launch_ntt(c->V, true, src, C, (size_t)c->ell * 2, c->k, 0, kN, kN, st, true, request_sums(C, c->ell, kN));
+  Prof p(c, PC_NTT, st, planes ? 2 : 1);
+  launch_ntt(c->V, true, src, C, (size_t)c->ell * 2, c->k, 0, kN, kN, st, split != nullptr,
+             split ? request_sums(C, c->ell, kN) : nullptr);
+  if (planes) launch_pack_request(c->V, C, split != nullptr, c->ell, reinterpret_cast<u32*>(planes), st);
   return cudaSuccess;
 }
 
@@ -463,54 +464,71 @@ int eval_core(pepsi_ctx* c, int set_id, const u64* cts, u32 layer0, u32 nl, int 
     lr.acc = b.acc;
     lr.G = G;
   }
+  // The request in the formats its multiply-accumulates read: byte planes for
+  // resident layers, split words for regenerated chunks.
+  const bool resident = res_end > layer0 && !S.words, streamed = res_end < end || S.words;
+  u64* const Cs = streamed ? (u64*)scratch(c, S_C, request_prepared_words(c->ell, kN) * 8, &e) : nullptr;
+  u64* const Cp = resident ? (u64*)scratch(c, S_CP, request_plane_words(c->ell, kN) * 8, &e) : nullptr;
+  if (e != cudaSuccess) return cuda_status(e);
   // A host request with resident layers arrives in pieces of its code bits:
   // the upload of piece p+1 overlaps the NTT and multiply-accumulate of
   // piece p, each piece's MAC adding into h' (the MAC is a sum over the
   // bits).  Otherwise the request is prepared whole.
   constexpr int npieces = pepsi_ctx::kPieces;
-  const bool pieces = !is_device_ptr(cts) && res_end > layer0 && c->ell >= 4 * npieces;
-  if (!pieces) CKS(prepare_request(c, cts, b.C, st));
+  // (Below 128 bits a second launch's sums and reductions cost more than the
+  // upload they hide.)
+  const bool pieces = !is_device_ptr(cts) && resident && c->ell >= 128;
+  if (!pieces) CKS(prepare_request(c, cts, Cs, Cp, st));
   // a5 on the resident layers: a multiply-accumulate launch over all of
   // them (one per piece), so the request is read from HBM once
   u64* Hall = nullptr;
   if (res_end > layer0) {
     Hall = (u64*)scratch(c, S_HALL, (size_t)(res_end - layer0) * ct2 * 8, &e);
     if (!Hall) return cuda_status(e);
-    const PlainTab P0 = S.plain(kN, c->ell, layer0);
-    if (pieces) {
-      // Piece boundaries in multiples of 4 bits.  The first piece is short, so
+    const PlaneTab P0 = S.planes(c->npl);
+    const u32* planes = reinterpret_cast<const u32*>(Cp);
+    if (S.words) {
+      Prof p(c, PC_MAC, st);
+      CKS(mac_status(launch_mac(c->V, Cs, S.word_table(kN, c->ell, layer0), Hall, c->ell, (int)(res_end - layer0),
+                                c->mac_fold, c->d_err, st)));
+    } else if (pieces) {
+      // Piece boundaries in steps of 16 bits.  The first piece is short, so
       // that little of the upload is exposed, yet its NTT and MAC must cover
       // the upload of the rest.  The MAC reads nres*ell*k*N table words while
       // the rest of the request is 2*(ell - j1)*k*N words, copied from the host
       // at well over 1/32 of HBM bandwidth: j1 = 64/nres of the bits covers it,
-      // at least 4 bits and at most half.
+      // at least 16 bits and at most half.
       static_assert(pepsi_ctx::kPieces == 2, "two pieces");
       const double w = std::min(0.5, 64.0 / (double)(res_end - layer0));
-      const int j1 = std::max(4, std::min((int)(c->ell * w) & ~3, (c->ell / 2) & ~3));
+      const int j1 = std::max(16, std::min((int)(c->ell * w) & ~15, (c->ell / 2) & ~15));
       const int jb[3] = {0, j1, c->ell};
+      u64* W = Cs ? Cs : (u64*)scratch(c, S_CW, (size_t)c->ell * ct2 * 8, &e);
+      if (!W) return cuda_status(e);
       CKS(ensure_copy_stream(c));
       CKS(cudaEventRecord(c->copy_ready, st));  // earlier work on st no longer reads the request buffer
       CKS(cudaStreamWaitEvent(c->copy_stream, c->copy_ready, 0));
       for (int q = 0; q < npieces; ++q) {
-        CKS(cudaMemcpyAsync(b.C + (size_t)jb[q] * ct2, cts + (size_t)jb[q] * ct2,
+        CKS(cudaMemcpyAsync(W + (size_t)jb[q] * ct2, cts + (size_t)jb[q] * ct2,
                             (size_t)(jb[q + 1] - jb[q]) * ct2 * 8, cudaMemcpyHostToDevice, c->copy_stream));
         CKS(cudaEventRecord(c->copy_ev[q], c->copy_stream));
       }
       for (int q = 0; q < npieces; ++q) {
+        const int ks0 = jb[q] / 16, ks1 = plane_steps(jb[q + 1]);
         CKS(cudaStreamWaitEvent(st, c->copy_ev[q], 0));
         {
-          Prof p(c, PC_NTT, st);  // forward NTT of the piece, stored in the split format
-          launch_ntt(c->V, true, b.C + (size_t)jb[q] * ct2, b.C + (size_t)jb[q] * ct2,
-                     (size_t)(jb[q + 1] - jb[q]) * 2, c->k, 0, kN, kN, st, true,
-                     request_sums(b.C, c->ell, kN) + (size_t)jb[q] * ct2);
+          Prof p(c, PC_NTT, st, 2);  // forward NTT of the piece, then its byte planes
+          u64* piece = W + (size_t)jb[q] * ct2;
+          launch_ntt(c->V, true, piece, piece, (size_t)(jb[q + 1] - jb[q]) * 2, c->k, 0, kN, kN, st, streamed,
+                     streamed ? request_sums(Cs, c->ell, kN) + (size_t)jb[q] * ct2 : nullptr);
+          launch_pack_request(c->V, W, streamed, c->ell, reinterpret_cast<u32*>(Cp), st, ks0, ks1);
         }
         Prof p(c, PC_MAC, st);
-        CKS(mac_status(launch_mac(c->V, b.C, P0, Hall, c->ell, (int)(res_end - layer0), c->mac_fold, c->d_err, st,
-                                  jb[q], jb[q + 1] - jb[q], q > 0)));
+        launch_mac_planes(c->V, 1, &planes, P0, &Hall, c->ell, (int)layer0, (int)(res_end - layer0), c->d_err, st, ks0,
+                          ks1, q > 0);
       }
     } else {
       Prof p(c, PC_MAC, st);
-      CKS(mac_status(launch_mac(c->V, b.C, P0, Hall, c->ell, (int)(res_end - layer0), c->mac_fold, c->d_err, st)));
+      launch_mac_planes(c->V, 1, &planes, P0, &Hall, c->ell, (int)layer0, (int)(res_end - layer0), c->d_err, st);
     }
   }
   bool first = true;
@@ -527,7 +545,7 @@ int eval_core(pepsi_ctx* c, int set_id, const u64* cts, u32 layer0, u32 nl, int 
         launch_ptgen(c->V, S.dpos + (size_t)l0 * N * c->h, L, c->ell, c->h, b.Pc, st);
       }
       Prof p(c, PC_MAC, st);  // a5 on a regenerated chunk
-      CKS(mac_status(launch_mac(c->V, b.C, plain_words(b.Pc), b.H, c->ell, L, c->mac_fold, c->d_err, st)));
+      CKS(mac_status(launch_mac(c->V, Cs, b.Pc, b.H, c->ell, L, c->mac_fold, c->d_err, st)));
     }
     const u64* VP = valued ? S.dVP + (size_t)l0 * vstride : nullptr;
     if (G > 1) {  // a6 + a7 with lazy rescaling
@@ -618,10 +636,17 @@ int eval_batch_core(pepsi_ctx* c, int nq, const int* set_ids, const u64* const* 
     e = eval_bufs(c, Lc, mres < mu, &b);
     if (e != cudaSuccess) return cuda_status(e);
     const size_t hq = (size_t)std::max<u32>(mres, (u32)Lc) * ct2;
-    u64* CB = (u64*)scratch(c, slot ? S_CB2 : S_CB, (size_t)PEPSI_MAC_MAX_REQUESTS * cwords * 8, &e);
+    // the requests in the formats their multiply-accumulates read: byte planes
+    // for resident layers (read on the auxiliary stream only, so one buffer
+    // when the split words of regenerated chunks take the double-buffered ones)
+    const bool streamed = mres < mu || S.words;
+    const size_t pwords = request_plane_words(c->ell, kN);
+    u64* CB = (u64*)scratch(c, slot ? S_CB2 : S_CB,
+                            (streamed ? (size_t)PEPSI_MAC_MAX_REQUESTS * cwords : (size_t)G * pwords) * 8, &e);
+    u64* CP = streamed && mres && !S.words ? (u64*)scratch(c, S_CP, (size_t)G * pwords * 8, &e) : CB;
     u64* HB = (u64*)scratch(c, slot ? S_HB2 : S_HB, (size_t)PEPSI_MAC_MAX_REQUESTS * hq * 8, &e);
     u64* ACC = (u64*)scratch(c, S_ACCB, (size_t)PEPSI_MAC_MAX_REQUESTS * ct3 * 8, &e);
-    if (!CB || !HB || !ACC) return cuda_status(e);
+    if (!CB || !CP || !HB || !ACC) return cuda_status(e);
     // per request: its mode, value plaintexts and rounding run length
     const size_t xw = (size_t)3 * (c->k + c->kb) * N, vstride = (size_t)(c->k + c->kb) * N;
     int gmode[PEPSI_MAC_MAX_REQUESTS];
@@ -641,16 +666,29 @@ int eval_batch_core(pepsi_ctx* c, int nq, const int* set_ids, const u64* const* 
       // requests and multiply-accumulate over the resident layers on the auxiliary
       // stream, once the circuits that last used this slot's buffers are done
       CKS(cudaStreamWaitEvent(ax, circ_done[slot], 0));
-      for (int g = 0; g < G; ++g) CKS(prepare_request(c, cts[grp[g]], CB + (size_t)g * cwords, ax));
+      const u32* planes[PEPSI_MAC_MAX_REQUESTS];
+      const u64* cq[PEPSI_MAC_MAX_REQUESTS];
+      u64* hs[PEPSI_MAC_MAX_REQUESTS];
+      for (int g = 0; g < G; ++g) {
+        u64* sp = streamed ? CB + (size_t)g * cwords : nullptr;
+        u64* pl = S.words ? nullptr : CP + (size_t)g * pwords;
+        CKS(prepare_request(c, cts[grp[g]], sp, pl, ax));
+        planes[g] = reinterpret_cast<const u32*>(pl);
+        cq[g] = sp;
+        hs[g] = HB + (size_t)g * hq;
+      }
       {
         Prof p(c, PC_MAC, ax);
-        CKS(mac_status(launch_mac_multi(c->V, CB, G, S.plain(kN, c->ell), HB, hq, c->ell, (int)mres, c->mac_fold,
-                                        c->d_err, ax, c->batch_points, c->batch_groups)));
+        if (S.words)
+          CKS(mac_status(launch_mac_requests(c->V, G, cq, S.word_table(kN, c->ell, 0), hs, c->ell, (int)mres,
+                                             c->mac_fold, c->d_err, ax, c->batch_points, c->batch_groups)));
+        else
+          launch_mac_planes(c->V, G, planes, S.planes(c->npl), hs, c->ell, 0, (int)mres, c->d_err, ax);
       }
       CKS(cudaEventRecord(mac_done[slot], ax));
       CKS(cudaStreamWaitEvent(st, mac_done[slot], 0));
     } else {
-      for (int g = 0; g < G; ++g) CKS(prepare_request(c, cts[grp[g]], CB + (size_t)g * cwords, st));
+      for (int g = 0; g < G; ++g) CKS(prepare_request(c, cts[grp[g]], CB + (size_t)g * cwords, nullptr, st));
     }
     for (u32 l0 = 0; l0 < mu;) {
       int L = (int)std::min<u32>(Lc, mu - l0);
@@ -663,8 +701,14 @@ int eval_batch_core(pepsi_ctx* c, int nq, const int* set_ids, const u64* const* 
           launch_ptgen(c->V, S.dpos + (size_t)l0 * N * c->h, L, c->ell, c->h, b.Pc, st);
         }
         Prof p(c, PC_MAC, st);
-        CKS(mac_status(launch_mac_multi(c->V, CB, G, plain_words(b.Pc), HB, hq, c->ell, L, c->mac_fold, c->d_err, st,
-                                        c->batch_points, c->batch_groups)));
+        const u64* cq[PEPSI_MAC_MAX_REQUESTS];
+        u64* hs[PEPSI_MAC_MAX_REQUESTS];
+        for (int g = 0; g < G; ++g) {
+          cq[g] = CB + (size_t)g * cwords;
+          hs[g] = HB + (size_t)g * hq;
+        }
+        CKS(mac_status(launch_mac_requests(c->V, G, cq, b.Pc, hs, c->ell, L, c->mac_fold, c->d_err, st,
+                                           c->batch_points, c->batch_groups)));
       }
       for (int g = 0; g < G; ++g) {
         b.H = HB + (size_t)g * hq + (res ? (size_t)l0 * ct2 : 0);
@@ -775,8 +819,8 @@ pepsi_ctx* ctx_fork(const pepsi_ctx* p, cudaError_t* err) {
     F.dT = S.dT;
     F.dpos = S.dpos;
     F.dP = S.dP;
-    F.p7 = S.p7;
     F.mu_res = S.mu_res;
+    F.words = S.words;
     F.has_values = S.has_values;
     F.dVP = S.dVP;
     c->sets.push_back(std::move(F));
@@ -800,7 +844,8 @@ pepsi_ctx* ctx_fork(const pepsi_ctx* p, cudaError_t* err) {
   c->rescale_cap = p->rescale_cap;
   c->value_margin = p->value_margin;
   c->resp = p->resp;
-  c->p7 = p->p7;
+  c->plaintext_bytes = p->plaintext_bytes;
+  c->npl = p->npl;
   cudaError_t e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, sizeof(int));
@@ -986,16 +1031,18 @@ int pepsi_setup(const pepsi_params* params, uint64_t key_seed, pepsi_ctx** out) 
   }
   c->gamma = params->gamma ? params->gamma : 1;
   c->resp = params->response_primes ? (int)params->response_primes : c->k;
-  // resident plaintexts in 7 bytes per word on request (every q_i < 2^56)
+  // resident plaintexts: ceil(bits / 8) bytes per word; plaintext_bytes = 7 asks for
+  // a table of at most 7 (every q_i < 2^56)
   {
-    bool fits = true;
-    for (u64 q : c->Q) fits = fits && q < (1ull << 56);
+    int bits = 0;
+    for (u64 q : c->Q) bits = std::max(bits, 64 - __builtin_clzll(q));
     const u32 pb = params->plaintext_bytes;
-    if ((pb != 0 && pb != 7 && pb != 8) || (pb == 7 && !fits)) {
+    if ((pb != 0 && pb != 7 && pb != 8) || (pb == 7 && bits > 56)) {
       delete c;
       return PEPSI_E_PARAM;
     }
-    c->p7 = pb == 7;
+    c->plaintext_bytes = pb == 7 ? 7 : 8;
+    c->npl = std::max(4, (bits + 7) / 8);
   }
   // lazy rescaling: runs of up to rescale_cap layers share one rounding
   {
@@ -1161,7 +1208,7 @@ int pepsi_get_info(const pepsi_ctx* c, pepsi_info* info) {
   info->response_primes = (uint32_t)c->resp;
   info->bins = c->blocks * (uint32_t)c->N;
   info->blocks = c->blocks;
-  info->plaintext_bytes = c->p7 ? 7 : 8;
+  info->plaintext_bytes = c->plaintext_bytes;
   info->gamma = c->gamma;
   return PEPSI_OK;
 }
@@ -1269,15 +1316,35 @@ int load_block(pepsi_ctx* c, std::vector<u64>&& hT, std::vector<uint32_t>* hV, u
       return cuda_status(e);
     }
   }
-  const size_t per_layer = (size_t)c->ell * k * N;  // plaintext words of a layer
   S.mu_res = mu_res;
-  if (S.mu_res) {
-    u64* tmp = nullptr;  // split-format words of a few layers, before packing
-    int G = 64;          // layers per generation launch
-    e = cudaMalloc(&S.dP, (size_t)S.mu_res * per_layer * (c->p7 ? 7 : 8));
-    if (e == cudaSuccess && c->p7) {
-      G = (int)std::max<size_t>(1, std::min<size_t>(64, ((size_t)1 << 30) / (per_layer * 8)));
+  S.words = !table_in_planes(c->ell, c->npl);
+  if (S.mu_res && S.words) {
+    e = cudaMalloc((void**)&S.dP, (size_t)S.mu_res * c->ell * k * N * 8);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      S.dP = nullptr;
+      S.mu_res = 0;
+    }
+    for (u32 l0 = 0; l0 < S.mu_res; l0 += 64) {
+      const int L = (int)std::min<u32>(64, S.mu_res - l0);
+      Prof p(c, PC_PTGEN, c->stream);
+      launch_ptgen(c->V, S.dpos + (size_t)l0 * N * c->h, L, c->ell, c->h,
+                   reinterpret_cast<u64*>(S.dP) + (size_t)l0 * c->ell * k * N, c->stream);
+    }
+  } else if (S.mu_res) {
+    // the table, and words of up to one tile of layers to pack from (fewer when
+    // memory is short)
+    const size_t per_layer = (size_t)c->ell * k * N;  // plaintext words of a layer
+    u64* tmp = nullptr;
+    int G = (int)std::min<u32>(16, S.mu_res);
+    e = cudaMalloc((void**)&S.dP, (size_t)S.mu_res * plane_layer_bytes(c->ell, k * N, c->npl));
+    if (e == cudaSuccess) {
       e = cudaMalloc((void**)&tmp, (size_t)G * per_layer * 8);
+      while (e != cudaSuccess && G > 1) {
+        cudaGetLastError();
+        G /= 2;
+        e = cudaMalloc((void**)&tmp, (size_t)G * per_layer * 8);
+      }
     }
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -1285,20 +1352,12 @@ int load_block(pepsi_ctx* c, std::vector<u64>&& hT, std::vector<uint32_t>* hV, u
       S.dP = nullptr;
       S.mu_res = 0;
     } else {
-      S.p7 = c->p7;
-      const PlainTab T = S.plain(k * N, c->ell);
+      const PlaneTab T = S.planes(c->npl);
       for (u32 l0 = 0; l0 < S.mu_res; l0 += G) {
         const int L = (int)std::min<u32>(G, S.mu_res - l0);
-        const size_t off = (size_t)l0 * per_layer;
-        Prof p(c, PC_PTGEN, c->stream);
-        if (!S.p7) {
-          launch_ptgen(c->V, S.dpos + (size_t)l0 * N * c->h, L, c->ell, c->h, static_cast<u64*>(S.dP) + off,
-                       c->stream);
-        } else {
-          launch_ptgen(c->V, S.dpos + (size_t)l0 * N * c->h, L, c->ell, c->h, tmp, c->stream);
-          launch_pack7(c->V, tmp, (size_t)L * per_layer, const_cast<u32*>(T.a) + off,
-                       const_cast<uint16_t*>(T.b) + off, const_cast<uint8_t*>(T.c) + off, c->stream);
-        }
+        Prof p(c, PC_PTGEN, c->stream, 2);
+        launch_ptgen(c->V, S.dpos + (size_t)l0 * N * c->h, L, c->ell, c->h, tmp, c->stream);
+        launch_pack_planes(c->V, tmp, c->ell, (int)l0, L, T, c->stream);
       }
     }
     if (tmp) {
@@ -1337,7 +1396,8 @@ int server_load_impl(pepsi_ctx* c, const uint64_t* items, bool with_values, cons
   if (rc) return rc;
   // resident NTT-form plaintexts: the longest prefix of layers the budget
   // holds for every block
-  const size_t per_layer = (size_t)c->ell * c->k * N * (c->p7 ? 7 : 8) * c->blocks;
+  const size_t per_layer = (table_in_planes(c->ell, c->npl) ? plane_layer_bytes(c->ell, c->k * N, c->npl)
+                                                             : (size_t)c->ell * c->k * N * 8) * c->blocks;
   size_t freeb = 0, totalb = 0;
   cudaMemGetInfo(&freeb, &totalb);
   const u64 cap = c->prm.resident_bytes;
@@ -1408,18 +1468,18 @@ int pepsi_server_plaintexts(pepsi_ctx* c, int set_id, uint32_t layer0, uint32_t 
   if (!tmp) return cuda_status(e);
   for (size_t b = 0; b < G->blk.size(); ++b) {
     ServerSet& S = c->sets[G->blk[b]];
-    if ((u64)layer0 + nl <= S.mu_res && S.p7) {  // the stored planes, put back together
-      const PlainTab T = S.plain((size_t)c->k * c->N, c->ell, layer0);
-      launch_unpack7(T.a, T.b, T.c, (size_t)nl * per, tmp, st);
+    if ((u64)layer0 + nl <= S.mu_res && S.words) {  // from the table
+      CKS(cudaMemcpyAsync(tmp, S.word_table((size_t)c->k * c->N, c->ell, layer0), (size_t)nl * per * 8,
+                          cudaMemcpyDeviceToDevice, st));
+      launch_split(c->V, tmp, (size_t)nl * c->ell, false, st);  // stored split; returned reduced
+    } else if ((u64)layer0 + nl <= S.mu_res) {
+      launch_unpack_planes(c->V, S.planes(c->npl), c->ell, (int)layer0, (int)nl, tmp, st);
     } else {
-      if ((u64)layer0 + nl <= S.mu_res) {
-        CKS(cudaMemcpyAsync(tmp, static_cast<const u64*>(S.dP) + (size_t)layer0 * per, (size_t)nl * per * 8,
-                            cudaMemcpyDeviceToDevice, st));
-      } else {
+      {
         Prof p(c, PC_PTGEN, st);
         launch_ptgen(c->V, S.dpos + (size_t)layer0 * c->N * c->h, nl, c->ell, c->h, tmp, st);
       }
-      launch_split(c->V, tmp, (size_t)nl * c->ell, false, st);  // stored split; returned reduced
+      launch_split(c->V, tmp, (size_t)nl * c->ell, false, st);  // generated split; returned reduced
     }
     e = copy_any(out + b * nl * per, tmp, (size_t)nl * per * 8, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
