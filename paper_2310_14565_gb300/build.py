@@ -47,7 +47,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         obj = os.path.join(OBJDIR, src + ".o")
         if force or _stale(obj, [path] + headers):
             cmd = [nv, "-c", path, "-o", obj] + common
-            cmd += ARCH + ["-lineinfo", "--expt-relaxed-constexpr"]
+            cmd += ARCH + ["-lineinfo", "--expt-relaxed-constexpr", "--split-compile=0"]
             if not src.endswith(".cu"):
                 cmd += ["-x", "cu", "-diag-suppress", "20208"]
             jobs.append(cmd)

@@ -30,8 +30,12 @@ typedef int64_t i64;
 // s = ceil(n/2) of the split operand format (hi << 32 | lo with x = hi 2^s +
 // lo) used by the multiply-accumulate; and the reduction constants
 // mu = floor(2^(n+63)/q), m64 = floor(2^64/q), c64 = 2^64 mod q (Shoup).
+// pm: q = 2^n - d with d small enough for the folding products below (PmMul);
+// the companion of a fixed operand w in the transform tables (and ninvs) is
+// then w 2^s mod q instead of Shoup's quotient.
 struct DevPrime {
   u64 q, ninv, ninvs, split, nbits, mu, m64, c64, c64s;
+  u32 pm, d, s, pad;
 };
 __host__ __device__ __forceinline__ u64 to_split(u64 x, u64 s) { return ((x >> s) << 32) | (x & ((1ull << s) - 1)); }
 __host__ __device__ __forceinline__ u64 from_split(u64 w, u64 s) { return ((w >> 32) << s) | (w & 0xFFFFFFFFull); }
@@ -92,6 +96,42 @@ __device__ __forceinline__ u64 shoup(u64 x, u64 w, u64 ws, u64 q) {
   u64 r = shoup_lazy(x, w, ws, q);
   return r >= q ? r - q : r;
 }
+// Products by a fixed w modulo q = 2^n - d (the primes are the largest below a
+// power of two, so d is small).  With v = w 2^s mod q, s = ceil((n + 5) / 2), and
+// x = x1 2^s + x0 < 2^(n+5): x w = x0 w + x1 v (mod q), a sum S below 2^(n+s+1)
+// of four 32-bit wide products, and 2^n = d folds its top: S mod 2^n + floor(S /
+// 2^n) d < 2 q, one more product.  Five wide products (the quarter-rate
+// operation that bounds the transforms) against the eight or so of Shoup's method
+// (a 64-bit high product and two low ones): 32 against 41 cycles a warp for a
+// butterfly in registers.
+struct PmMul {
+  u64 q;
+  u32 d, s, n32, smask, nmask;
+  __device__ __forceinline__ explicit PmMul(const DevPrime& p)
+      : q(p.q), d(p.d), s(p.s), n32((u32)p.nbits - 32), smask((1u << p.s) - 1), nmask((1u << (p.nbits - 32)) - 1) {}
+  // x < 2^(n+5) -> [0, 2q)
+  __device__ __forceinline__ u64 mul(u64 x, u64 w, u64 v) const {
+    const u32 x0 = (u32)x & smask, x1 = __funnelshift_r((u32)x, (u32)(x >> 32), s);
+    u64 r;  // L = x0 wl + x1 vl < 2^(s+33) <= 2^64, M = x0 wh + x1 vh + (L >> 32)
+    asm("{\n\t"
+        ".reg .u64 L, M;\n\t.reg .u32 l, h, m, k, t;\n\t"
+        "mul.wide.u32 L, %1, %3;\n\tmul.wide.u32 M, %1, %4;\n\t"
+        "mad.wide.u32 L, %2, %5, L;\n\tmad.wide.u32 M, %2, %6, M;\n\t"
+        "mov.b64 {l, h}, L;\n\tmov.b64 {m, k}, M;\n\t"
+        "add.cc.u32 m, m, h;\n\taddc.u32 k, k, 0;\n\t"
+        "shf.r.wrap.b32 t, m, k, %7;\n\tand.b32 m, m, %8;\n\t"
+        "mov.b64 L, {l, m};\n\tmad.wide.u32 %0, t, %9, L;\n\t}"
+        : "=l"(r)
+        : "r"(x0), "r"(x1), "r"((u32)w), "r"((u32)(w >> 32)), "r"((u32)v), "r"((u32)(v >> 32)), "r"(n32), "r"(nmask),
+          "r"(d));
+    return r;
+  }
+  // x < 2^(n+5) -> [0, 2^n + 2^29) with x = x1 2^n + x0: x0 + x1 d
+  __device__ __forceinline__ u64 fold(u64 x) const {
+    const u32 h = (u32)(x >> 32);
+    return ((u64)(h & nmask) << 32 | (u32)x) + (h >> n32) * d;
+  }
+};
 // x mod q for any 64-bit x: one-word Barrett, floor(x m64 / 2^64) is short
 // of floor(x/q) by at most 1.
 __device__ __forceinline__ u64 barrett64(u64 x, const DevPrime& p) {

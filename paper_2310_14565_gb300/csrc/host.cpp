@@ -104,8 +104,22 @@ DevPrime make_prime(u64 q, u32 N) {
   p.m64 = (u64)(((u128)1 << 64) / q);
   p.c64 = (u64)(((u128)1 << 64) % q);
   p.c64s = shoup_of(p.c64, q);
+  // q = 2^bits - d: the product's fold leaves less than 2^bits + 2^(s+1) d, which
+  // has to stay below 2 q, and 31 d has to fit 32 bits (PmMul::fold)
+  p.pm = p.d = p.s = p.pad = 0;
+  if (bits >= 40 && bits <= 57) {
+    const u64 d = ((u64)1 << bits) - q;
+    const int sh = (bits + 6) / 2;
+    if (d < ((u64)1 << 27) && ((u128)d << (sh + 1)) + 2 * d < ((u128)1 << bits)) {
+      p.pm = 1;
+      p.d = (u32)d;
+      p.s = (u32)sh;
+      p.ninvs = companion(p.ninv, p);
+    }
+  }
   return p;
 }
+u64 companion(u64 w, const DevPrime& p) { return p.pm ? mulmod(w, (u64)1 << p.s, p.q) : shoup_of(w, p.q); }
 
 static u32 bitrev(u32 x, u32 bits) {
   u32 r = 0;
@@ -113,7 +127,8 @@ static u32 bitrev(u32 x, u32 bits) {
   return r;
 }
 
-void twiddles(u64 q, u64 psi, u32 N, u64* tw, u64* tws, u64* itw, u64* itws) {
+void twiddles(const DevPrime& p, u64 psi, u32 N, u64* tw, u64* tws, u64* itw, u64* itws) {
+  const u64 q = p.q;
   u32 lg = 0;
   while ((1u << lg) < N) ++lg;
   std::vector<u64> pw(N), ipw(N);
@@ -126,16 +141,16 @@ void twiddles(u64 q, u64 psi, u32 N, u64* tw, u64* tws, u64* itw, u64* itws) {
   for (u32 i = 0; i < N; ++i) {
     const u32 r = bitrev(i, lg);
     tw[i] = pw[r];
-    tws[i] = shoup_of(tw[i], q);
+    tws[i] = companion(tw[i], p);
     itw[i] = ipw[r];
-    itws[i] = shoup_of(itw[i], q);
+    itws[i] = companion(itw[i], p);
   }
   // entry 0 is not a stage twiddle (stage s uses [2^s, 2^(s+1))): the
   // inverse table keeps there its stage-0 twiddle times N^-1, which the last
   // inverse stage applies to its difference outputs
   if (N > 1) {
     itw[0] = mulmod(itw[1], invmod(N % q, q), q);
-    itws[0] = shoup_of(itw[0], q);
+    itws[0] = companion(itw[0], p);
   }
 }
 

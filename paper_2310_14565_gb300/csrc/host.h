@@ -19,8 +19,10 @@ u64 find_prime(int bits, u32 N, const std::vector<u64>& taken);
 u64 min_root(u64 q, u32 N);
 u64 shoup_of(u64 w, u64 q);
 DevPrime make_prime(u64 q, u32 N);
-// twiddles psi^brev(i) (fwd) and psi^-brev(i) (inv) with Shoup companions
-void twiddles(u64 q, u64 psi, u32 N, u64* tw, u64* tws, u64* itw, u64* itws);
+// companion of a fixed operand w of the transforms modulo p: w 2^s mod q where p.pm, else Shoup's
+u64 companion(u64 w, const DevPrime& p);
+// twiddles psi^brev(i) (fwd) and psi^-brev(i) (inv) with their companions
+void twiddles(const DevPrime& p, u64 psi, u32 N, u64* tw, u64* tws, u64* itw, u64* itws);
 // constants of the exact RNS conversions
 void rns_constants(const std::vector<u64>& Qp, const std::vector<u64>& Bp, u64 t, RnsConst* rc);
 // round(Q v / t) mod q_i for v in [0, t)

@@ -24,18 +24,24 @@ int sm_count() {
 namespace {
 
 // Threads of a block running the register-blocked NTT: one per group of 8
-// elements, at most 512 (two blocks of 64 KB per SM up to N = 8192), and
-// 1024 at N = 16384, whose 128 KB polynomial leaves room for one block per
-// SM.  The kernels below are compiled for 1024 threads at 64 registers, so
-// either shape keeps 32 warps on an SM.
+// elements, at most 256 (three blocks of 64 KB per SM at N = 8192: 1200 x 4 rows
+// took 289 us against 293 us with 512 threads and 336 us with 128; N = 4096: 137
+// us against 147 and 147 us), and 1024 at N = 16384, whose 128 KB polynomial leaves
+// room for one block per SM (301 us for 256 x 8 rows against 321 us with 512).
 constexpr int NTT_MAX_THREADS = 1024;
 inline int ntt_threads(int N) {
   if (N >= 16384) return NTT_MAX_THREADS;
   int t = N / 8;
-  if (t > 512) t = 512;
+  if (t > 256) t = 256;
   if (t < 32) t = 32;
   return t;
 }
+// Threads of the kernels that give a block a chain of transforms (plaintexts,
+// encryption, keys, decryption): their larger shared memory leaves room for two
+// blocks per SM at most, so they take twice the threads.
+inline int chain_threads(int N) { return N >= 16384 ? NTT_MAX_THREADS : std::max(32, std::min(512, N / 8)); }
+// Threads of launches of a few blocks, whose time is one block's latency.
+inline int latency_threads(int N) { return std::min(NTT_MAX_THREADS, std::max(32, N / 8)); }
 // Threads of the hot-path transform kernels: the schedule's choice
 // (DevView::nt, picked by the autotuner), else the default above.
 inline int xform_threads(const DevView& V) { return V.nt > 0 ? V.nt : ntt_threads(V.N); }
@@ -45,7 +51,7 @@ inline int xform_threads(const DevView& V) { return V.nt > 0 ? V.nt : ntt_thread
 // transform's chain of phases.
 inline int xform_threads(const DevView& V, size_t rows) {
   const int base = xform_threads(V);
-  const int wide = std::min(NTT_MAX_THREADS, std::max(32, V.N / 8));
+  const int wide = latency_threads(V.N);
   return rows <= (size_t)sm_count() && wide > base ? wide : base;
 }
 // The relinearisation transforms come in two register budgets: MT = 256 for
@@ -154,6 +160,37 @@ __global__ void k_cw_unrank(const u64* __restrict__ T, size_t count, const u64* 
   }
 }
 
+// floor(x / t) with the one-word Barrett constant of t
+__device__ __forceinline__ u64 div_by(u64 x, const DevPrime& t) {
+  const u64 d = __umul64hi(x, t.m64);  // short by at most 1
+  return x - d * t.q >= t.q ? d + 1 : d;
+}
+// round(Q m / t) mod q_p for m in [0, t): floor(Q/t) m + round((Q mod t) m / t)
+__device__ __forceinline__ u64 delta_of(const RnsConst& rc, u64 m, int p, const DevPrime& pq, const DevPrime& t) {
+  const u64 a = shoup(m, rc.qdt_q[p], rc.qdt_qs[p], pq.q);
+  return addmod(a, barrett64(div_by(rc.qmt * m + (t.q - 1) / 2, t), pq), pq.q);
+}
+// sample_uniform modulo p.q, with p's reduction constants (2^64 mod q = c64) in
+// place of two 64-bit remainders
+__device__ __forceinline__ u64 sample_mod(u64 key, u64 pos, const DevPrime& p) {
+  u64 r = 0;
+  for (u64 a = 0; a < 256; a++) {
+    r = draw_keyed(key, (pos << 8) | a);
+    if (p.c64 == 0 || r < (u64)(0 - p.c64)) break;
+  }
+  return barrett64(r, p);
+}
+// Encode: inverse transform modulo t of ld (a slot value below t per position)
+// into m[], in 32-bit words for t below 2^30.  a: N words of scratch.
+template <class Load>
+__device__ __forceinline__ void encode_block(u64* a, const Load& ld, u32* m, const DevView& V) {
+  if (V.pr[V.tidx].q < (1ull << 30))
+    ntt_inv_gg_small(reinterpret_cast<u32*>(a), ld, [&](int i, u32 v) { m[i] = v; }, V, V.tidx);
+  else
+    ntt_inv_gg(a, [&](int i) -> u64 { return ld(i); }, [&](int i, u64 v) { m[i] = (u32)v; }, V, V.tidx);
+  __syncthreads();
+}
+
 // ------------------------------------------------- server plaintexts (K3)
 // Block (layer l, j-chunk): bit planes of the layer's codewords, encoded
 // (inverse NTT mod t of the slot vector in bit-reversed order), centred
@@ -184,27 +221,15 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ptgen(DevView V, const u
   for (int jj = 0; jj < JC; ++jj) {
     const int j = j0 + jj;
     if (j >= ell) break;
-    // Encode: slot s at position brev(s), inverse NTT mod t into mbuf (in
-    // 32-bit words for t below 2^30)
+    // Encode: slot s at position brev(s), inverse NTT mod t into mbuf
     const u32* bj = bits + jj * words;
-    if (t < (1ull << 30)) {
-      ntt_inv_gg_small(
-          reinterpret_cast<u32*>(poly),
-          [&](int i) -> u32 {
-            const u32 s = brev_bits(i, V.logN);
-            return (bj[s >> 5] >> (s & 31)) & 1u;
-          },
-          [&](int i, u32 v) { mbuf[i] = v; }, V, V.tidx);
-    } else {
-      ntt_inv_gg(
-          poly,
-          [&](int i) -> u64 {
-            const u32 s = brev_bits(i, V.logN);
-            return (bj[s >> 5] >> (s & 31)) & 1u;
-          },
-          [&](int i, u64 v) { mbuf[i] = (u32)v; }, V, V.tidx);
-    }
-    __syncthreads();
+    encode_block(
+        poly,
+        [&](int i) -> u32 {
+          const u32 s = brev_bits(i, V.logN);
+          return (bj[s >> 5] >> (s & 31)) & 1u;
+        },
+        mbuf, V);
     for (int p = 0; p < k; ++p) {
       // centred lift to q_p on the load, split operand format on the store
       const u64 q = V.pr[p].q, sp = V.pr[p].split;
@@ -1120,13 +1145,6 @@ __global__ void k_accum(DevView V, const u64* __restrict__ D, int L, u64* acc, i
 }
 
 // ---------------------------------------------------------------- client
-// round(Q m / t) mod q_p for m in [0, t): floor(Q/t) m + round((Q mod t) m / t)
-__device__ __forceinline__ u64 delta_of(const DevView& V, u64 m, int p, u64 t) {
-  const DevPrime pq = V.pr[p];
-  const u64 a = shoup(m, V.rc->qdt_q[p], V.rc->qdt_qs[p], pq.q);
-  const u64 b = (V.rc->qmt * m + (t - 1) / 2) / t;
-  return addmod(a, b % pq.q, pq.q);
-}
 __device__ __forceinline__ u64 smod_dev(i64 v, u64 q) { return v >= 0 ? (u64)v : q - (u64)(-v); }
 
 // Block per ciphertext j: encode bit plane j, then for each prime sample
@@ -1137,41 +1155,42 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_encrypt(DevView V, const
   const int N = V.N, k = V.k, j = blockIdx.x;
   u64* poly = sm;
   u32* mbuf = reinterpret_cast<u32*>(sm + N);
-  const u64 t = V.pr[V.tidx].q;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    const int s = (int)brev_bits(i, V.logN);
-    const uint16_t* ps = pos + (size_t)s * h;
-    u64 bit = 0;
-    if (ps[0] != PEPSI_CW_NONE)
-      for (int r = 0; r < h; ++r) bit |= (ps[r] == j);
-    poly[nsw(i)] = bit;
-  }
-  __syncthreads();
-  ntt_inv_view(poly, V, V.tidx);
-  for (int i = threadIdx.x; i < N; i += blockDim.x) mbuf[i] = (u32)poly[nsw(i)];
-  __syncthreads();
+  const DevPrime t = V.pr[V.tidx];
+  encode_block(
+      poly,
+      [&](int i) -> u32 {
+        const uint16_t* ps = pos + (size_t)brev_bits(i, V.logN) * h;
+        u32 bit = 0;
+        if (ps[0] != PEPSI_CW_NONE)
+          for (int r = 0; r < h; ++r) bit |= (ps[r] == j);
+        return bit;
+      },
+      mbuf, V);
   const u64 key_e = stream_key(seed, make_stream(STREAM_ENC_E, idx0 + j, 0));
   for (int p = 0; p < k; ++p) {
     const DevPrime pq = V.pr[p];
     const u64 key_a = stream_key(seed, make_stream(STREAM_ENC_A, idx0 + j, p));
     u64* c0 = cts + (((size_t)j * 2 + 0) * k + p) * N;
     u64* c1 = cts + (((size_t)j * 2 + 1) * k + p) * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const u64 a = sample_uniform(key_a, i, pq.q);
-      c1[i] = a;
-      poly[nsw(i)] = a;
-    }
-    __syncthreads();
-    ntt_fwd_view(poly, V, p);
     const u64* sr = s_ntt + (size_t)p * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) poly[nsw(i)] = mulmod(poly[nsw(i)], sr[i], pq);
-    __syncthreads();
-    ntt_inv_view(poly, V, p);
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const u64 e = smod_dev(sample_cbd21(key_e, i), pq.q);
-      c0[i] = addmod(submod(e, poly[nsw(i)], pq.q), delta_of(V, mbuf[i], p, t), pq.q);
-    }
-    __syncthreads();
+    // a, its transform times s left in place, and back: every thread's last
+    // elements of the first transform are its first of the second
+    ntt_fwd_gg(
+        poly,
+        [&](int i) {
+          const u64 a = sample_mod(key_a, i, pq);
+          c1[i] = a;
+          return a;
+        },
+        [&](int i, u64 v) { poly[nsw(i)] = mulmod(v, sr[i], pq); }, V, p);
+    ntt_inv_gg(
+        poly, [&](int i) { return poly[nsw(i)]; },
+        [&](int i, u64 v) {
+          const u64 e = smod_dev(sample_cbd21(key_e, i), pq.q);
+          c0[i] = addmod(submod(e, v, pq.q), delta_of(*V.rc, mbuf[i], p, pq, t), pq.q);
+        },
+        V, p);
+    __syncthreads();  // the next transform overwrites poly
   }
 }
 
@@ -1225,13 +1244,12 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_dec_z(DevView V, const u
   const int p = blockIdx.x, N = V.N, k = V.k;
   const DevPrime pq = V.pr[p];
   const u64* c1 = ct + ((size_t)k + p) * N;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) sm[nsw(i)] = c1[i];
-  __syncthreads();
-  ntt_fwd_view(sm, V, p);
-  for (int i = threadIdx.x; i < N; i += blockDim.x) sm[nsw(i)] = mulmod(sm[nsw(i)], s_ntt[(size_t)p * N + i], pq);
-  __syncthreads();
-  ntt_inv_view(sm, V, p);
-  for (int i = threadIdx.x; i < N; i += blockDim.x) z[(size_t)p * N + i] = addmod(sm[nsw(i)], ct[(size_t)p * N + i], pq.q);
+  const u64 *c0 = ct + (size_t)p * N, *sr = s_ntt + (size_t)p * N;
+  u64* zr = z + (size_t)p * N;
+  ntt_fwd_gg(
+      sm, [&](int i) { return c1[i]; }, [&](int i, u64 v) { sm[nsw(i)] = mulmod(v, sr[i], pq); }, V, p);
+  ntt_inv_gg(
+      sm, [&](int i) { return sm[nsw(i)]; }, [&](int i, u64 v) { zr[i] = addmod(v, c0[i], pq.q); }, V, p);
 }
 // Step 2, per coefficient: m = round(t z / Q) mod t exactly (Garner of
 // w = t z + (Q-1)/2 over Q, then (w - [w]_Q)/Q mod t), and the noise
@@ -1241,7 +1259,8 @@ __global__ void k_dec_coef(const __grid_constant__ RnsArgs A, DevView V, const u
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   const int N = V.N, k = V.k;
   const RnsConst* rc = &A.rc;
-  const u64 t = V.pr[V.tidx].q;
+  const DevPrime Pt = V.pr[V.tidx];
+  const u64 t = Pt.q;
   double rabs = 0.0;
   if (n < N) {
     u64 w[PEPSI_MAXQ], v[PEPSI_MAXQ];
@@ -1255,8 +1274,8 @@ __global__ void k_dec_coef(const __grid_constant__ RnsArgs A, DevView V, const u
     u64 wq = 0;
 #pragma unroll
     for (int l = 0; l < PEPSI_MAXQ; ++l)
-      if (l < k) wq = (wq + (v[l] % t) * rc->pq_t[l]) % t;
-    m[n] = (u32)(((rc->qhalf_t + t - wq) % t) * rc->qinv_t % t);
+      if (l < k) wq = barrett64(wq + barrett64(v[l], Pt) * rc->pq_t[l], Pt);  // below t + (t - 1)^2 < 2^64
+    m[n] = (u32)barrett64(submod(rc->qhalf_t, wq, t) * rc->qinv_t, Pt);
 #pragma unroll
     for (int i = 0; i < PEPSI_MAXQ; ++i)
       if (i < k) w[i] = shoup(z[(size_t)i * N + n], rc->t_q[i], rc->t_qs[i], V.pr[i].q);
@@ -1285,11 +1304,8 @@ __global__ void k_dec_coef(const __grid_constant__ RnsArgs A, DevView V, const u
 // Step 3: slots = values of m at psi_t^(2s+1): forward NTT mod t, slot s in position brev(s).
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_dec_slots(DevView V, const u32* __restrict__ m, u32* slots) {
   extern __shared__ u64 sm[];
-  const int N = V.N;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) sm[nsw(i)] = m[i];
-  __syncthreads();
-  ntt_fwd_view(sm, V, V.tidx);
-  for (int s = threadIdx.x; s < N; s += blockDim.x) slots[s] = (u32)sm[nsw(brev_bits(s, V.logN))];
+  ntt_fwd_gg(
+      sm, [&](int i) -> u64 { return m[i]; }, [&](int i, u64 v) { slots[brev_bits(i, V.logN)] = (u32)v; }, V, V.tidx);
 }
 
 // Modulus switching of the response to the first r primes: per
@@ -1328,37 +1344,39 @@ __global__ void k_modswitch(const __grid_constant__ ModSwitchArgs M, DevView V, 
 }
 
 // Cardinality mask (Algorithm 5): r_s uniform in Z_t for s < N-1,
-// r_{N-1} = -sum; c0 += round(Q Encode(r) / t).  One block.
+// r_{N-1} = -sum; c0 += round(Q Encode(r) / t).  A block per prime: each draws
+// and encodes the same mask and adds it to its row (one block for all rows, with
+// 64-bit remainders, took 73 us at N = 8192, k = 4).
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_mask(DevView V, u64 seed, u64* ct) {
   extern __shared__ u64 sm[];
   __shared__ u64 red[32];
-  const int N = V.N, k = V.k;
-  const u64 t = V.pr[V.tidx].q;
+  const int N = V.N, p = blockIdx.x;
+  u32* r = reinterpret_cast<u32*>(sm + N);
+  const DevPrime t = V.pr[V.tidx], pq = V.pr[p];
   const u64 key = stream_key(seed, make_stream(STREAM_MASK, 0, 0));
-  u64 part = 0;
+  u64 part = 0;  // below N t < 2^46
   for (int s = threadIdx.x; s < N - 1; s += blockDim.x) {
-    const u64 r = sample_uniform(key, s, t);
-    sm[nsw(brev_bits(s, V.logN))] = r;
-    part += r;
+    const u64 v = sample_mod(key, s, t);
+    r[s] = (u32)v;
+    part += v;
   }
-  part %= t;
   for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part % t;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
   __syncthreads();
   if (threadIdx.x == 0) {
     u64 sum = 0;
-    for (int i = 0; i < (int)(blockDim.x + 31) / 32; ++i) sum = (sum + red[i]) % t;
-    sm[nsw(brev_bits(N - 1, V.logN))] = (t - sum) % t;
+    for (int i = 0; i < (int)(blockDim.x + 31) / 32; ++i) sum += red[i];
+    sum = barrett64(sum, t);
+    r[N - 1] = sum ? (u32)(t.q - sum) : 0;
   }
   __syncthreads();
-  ntt_inv_view(sm, V, V.tidx);
-  for (int p = 0; p < k; ++p) {
-    const u64 q = V.pr[p].q;
-    for (int n = threadIdx.x; n < N; n += blockDim.x) {
-      u64* c = ct + (size_t)p * N + n;
-      *c = addmod(*c, delta_of(V, sm[nsw(n)], p, t), q);
-    }
-  }
+  u64* row = ct + (size_t)p * N;
+  auto ld = [&](int i) -> u32 { return r[brev_bits(i, V.logN)]; };
+  auto st = [&](int i, u64 v) { row[i] = addmod(row[i], delta_of(*V.rc, v, p, pq, t), pq.q); };
+  if (t.q < (1ull << 30))
+    ntt_inv_gg_small(reinterpret_cast<u32*>(sm), ld, st, V, V.tidx);
+  else
+    ntt_inv_gg(sm, [&](int i) -> u64 { return ld(i); }, st, V, V.tidx);
 }
 
 inline unsigned grid_for(size_t total, int threads) { return (unsigned)((total + threads - 1) / threads); }
@@ -1402,7 +1420,7 @@ void launch_ptgen(const DevView& V, const uint16_t* pos, int L, int ell, int h, 
   if (L <= 0) return;
   const int JC = ptgen_jc(V.N);
   dim3 grid((ell + JC - 1) / JC, L);
-  k_ptgen<<<grid, ntt_threads(V.N), ptgen_smem(V.N), st>>>(V, pos, ell, h, JC, P);
+  k_ptgen<<<grid, chain_threads(V.N), ptgen_smem(V.N), st>>>(V, pos, ell, h, JC, P);
 }
 
 namespace {
@@ -1546,7 +1564,7 @@ void launch_tensor_sum(const DevView& V, const u64* AQ, const u64* AB, const u64
 
 void launch_valgen(const DevView& V, const u32* vals, int L, u64* VP, cudaStream_t st) {
   if (L <= 0) return;
-  k_valgen<<<L, ntt_threads(V.N), (size_t)V.N * 12, st>>>(V, vals, VP);
+  k_valgen<<<L, chain_threads(V.N), (size_t)V.N * 12, st>>>(V, vals, VP);
 }
 
 // Value-weighted layer sum with per-layer rounding: acc[c][p][n] (+)=
@@ -1635,13 +1653,13 @@ void launch_accum(const DevView& V, const u64* D, int L, u64* acc, bool init, cu
 void launch_encrypt(const DevView& V, const uint16_t* pos, int ell, int h, const u64* s_ntt, u64 seed, u64 idx0,
                     u64* cts, cudaStream_t st) {
   if (ell <= 0) return;
-  k_encrypt<<<ell, ntt_threads(V.N), (size_t)V.N * 12, st>>>(V, pos, h, s_ntt, seed, idx0, cts);
+  k_encrypt<<<ell, chain_threads(V.N), (size_t)V.N * 12, st>>>(V, pos, h, s_ntt, seed, idx0, cts);
 }
 
 void launch_keygen(const DevView& V, u64 seed, int8_t* s, u64* s_ntt, u64* rlk, cudaStream_t st) {
   k_keygen_s<<<grid_for(V.N, 256), 256, 0, st>>>(V, seed, s);
-  k_keygen_sntt<<<V.k, ntt_threads(V.N), (size_t)V.N * 8, st>>>(V, s, s_ntt);
-  k_keygen_rlk<<<V.k * V.k, ntt_threads(V.N), (size_t)V.N * 8, st>>>(V, seed, s_ntt, rlk);
+  k_keygen_sntt<<<V.k, chain_threads(V.N), (size_t)V.N * 8, st>>>(V, s, s_ntt);
+  k_keygen_rlk<<<V.k * V.k, chain_threads(V.N), (size_t)V.N * 8, st>>>(V, seed, s_ntt, rlk);
 }
 
 void launch_modswitch(const DevView& V, const ModSwitchArgs& M, const u64* in, u64* out, size_t n, cudaStream_t st) {
@@ -1671,13 +1689,13 @@ void launch_wait_probe(int arrive, int* err, cudaStream_t st) { k_wait_probe<<<1
 void launch_decrypt(const DevView& V, const u64* ct, const u64* s_ntt, u64* zbuf, u32* mbuf, u32* slots,
                     unsigned long long* maxr, cudaStream_t st) {
   cudaMemsetAsync(maxr, 0, sizeof(unsigned long long), st);
-  k_dec_z<<<V.k, ntt_threads(V.N), (size_t)V.N * 8, st>>>(V, ct, s_ntt, zbuf);
+  k_dec_z<<<V.k, latency_threads(V.N), (size_t)V.N * 8, st>>>(V, ct, s_ntt, zbuf);
   k_dec_coef<<<grid_for(V.N, 128), 128, 0, st>>>(*V.host_args, V, zbuf, mbuf, maxr);
-  k_dec_slots<<<1, ntt_threads(V.N), (size_t)V.N * 8, st>>>(V, mbuf, slots);
+  k_dec_slots<<<1, latency_threads(V.N), (size_t)V.N * 8, st>>>(V, mbuf, slots);
 }
 
 void launch_mask(const DevView& V, u64 seed, u64* ct, cudaStream_t st) {
-  k_mask<<<1, 512, (size_t)V.N * 8, st>>>(V, seed, ct);
+  k_mask<<<V.k, latency_threads(V.N), (size_t)V.N * 12, st>>>(V, seed, ct);
 }
 
 cudaError_t kernels_init(int N) {

@@ -22,38 +22,68 @@
 #include <type_traits>
 #include "common.cuh"
 
-__device__ __forceinline__ int nsw(int x) { return x ^ ((x >> 4) & 15); }
+__host__ __device__ __forceinline__ constexpr int nsw(int x) { return x ^ ((x >> 4) & 15); }
+
+// Element base + c of the array for base and c with no common bit, from nb =
+// nsw(base) * sizeof(T).  nsw is linear over XOR, so only c's part of the low four
+// bits is XORed in and the rest is an offset: with c a constant (the phases of
+// the fixed ring sizes) that is one operation or none per access, instead of the
+// five of nsw(base + c) on the ALU pipe, which the transforms keep as busy as the
+// multiply-add pipe.
+template <class T>
+__device__ __forceinline__ T& at(T* a, u32 nb, int c) {
+  const int low = (c & 15) ^ ((c >> 4) & 15), high = c & ~15;
+  return *reinterpret_cast<T*>(reinterpret_cast<char*>(a) + (nb ^ (u32)(low * (int)sizeof(T))) + high * (int)sizeof(T));
+}
 
 namespace nttd {
 
-// Word types of the transforms: 64-bit words for the ciphertext primes, and
-// 32-bit words for a modulus below 2^30 (the plaintext modulus t), where
-// Shoup's product takes one 32x32 high product and two low ones.  A twiddle
-// pair (w, floor(w 2^64 / q)) gives the 32-bit companion floor(w 2^32 / q)
-// as its upper half.
-__device__ __forceinline__ u64 lazy_mul(u64 x, u64 w, u64 ws, u64 q) { return shoup_lazy(x, w, ws, q); }
-__device__ __forceinline__ u32 lazy_mul(u32 x, u32 w, u32 ws, u32 q) { return x * w - __umulhi(x, ws) * q; }
-__device__ __forceinline__ void tw_split(const ulonglong2& t, u64& w, u64& ws) {
-  w = t.x;
-  ws = t.y;
-}
-__device__ __forceinline__ void tw_split(const ulonglong2& t, u32& w, u32& ws) {
-  w = (u32)t.x;
-  ws = (u32)(t.y >> 32);
-}
+// Arithmetic of a transform's modulus.  mul(x, t) multiplies by a table entry
+// t = (w, companion) into [0, 2q).
+//  - Shoup<G>: any q below 2^61.  G (q < 2^59): the forward butterfly's sum input
+//    is not reduced below 2q first, so values grow by 2q a stage (the product
+//    takes any 64-bit input): from [0, 4q) they stay below (4 + 2 log2 N) q <=
+//    32 q, which fits 64 bits, and one Barrett reduction at the end reduces them.
+//  - Pm: q = 2^n - d, n <= 57 (PmMul, inputs below 2^(n+5)): forward as above; the
+//    inverse's sums double from 4q to at most 32q over the three stages of a
+//    phase, and a fold of the sums at its end brings them below 2q.
+//  - Small: 32-bit words for a modulus below 2^30 (the plaintext modulus t), where
+//    Shoup's product takes one 32x32 high product and two low ones; the upper half
+//    of a Shoup companion floor(w 2^64 / q) is floor(w 2^32 / q).
+template <bool G>
+struct Shoup {
+  typedef u64 T;
+  static constexpr bool kGrow = G, kPm = false;
+  u64 q, m64;
+  __device__ __forceinline__ explicit Shoup(const DevPrime& p) : q(p.q), m64(p.m64) {}
+  __device__ __forceinline__ u64 mul(u64 x, const ulonglong2& t) const { return shoup_lazy(x, t.x, t.y, q); }
+};
+struct Pm {
+  typedef u64 T;
+  static constexpr bool kGrow = true, kPm = true;
+  PmMul m;
+  u64 q;
+  __device__ __forceinline__ explicit Pm(const DevPrime& p) : m(p), q(p.q) {}
+  __device__ __forceinline__ u64 mul(u64 x, const ulonglong2& t) const { return m.mul(x, t.x, t.y); }
+};
+struct Small {
+  typedef u32 T;
+  static constexpr bool kGrow = false, kPm = false;
+  u32 q;
+  __device__ __forceinline__ explicit Small(const DevPrime& p) : q((u32)p.q) {}
+  __device__ __forceinline__ u32 mul(u32 x, const ulonglong2& t) const {
+    return x * (u32)t.x - __umulhi(x, (u32)(t.y >> 32)) * q;
+  }
+};
 
 // Forward stages [s0, s0 + RR) on one group of 2^RR elements held in
 // registers, element i of the group at base + i * 2^(logN - s0 - RR).
-// Twiddles come as (w, Shoup companion) pairs, one 16-byte load each.
-// GROW: the butterfly's sum input is not reduced below 2q first, so values
-// grow by 2q a stage (Shoup's product takes any 64-bit input and returns
-// [0, 2q)): from [0, 4q) they stay below (4 + 2 log2 N) q <= 32 q, which fits
-// 64 bits for q < 2^59; the transform's end reduces them (fwd_final_grow).
-template <int RR, bool GROW = false>
-__device__ __forceinline__ void fwd_group(u64 (&x)[1 << RR], int base, int logN, int s0, u64 q,
+// Twiddles come as (w, companion) pairs, one 16-byte load each.
+template <int RR, class A>
+__device__ __forceinline__ void fwd_group(u64 (&x)[1 << RR], int base, int logN, int s0, const A& ar,
                                           const ulonglong2* __restrict__ tw) {
   constexpr int E = 1 << RR;
-  const u64 q2 = 2 * q;
+  const u64 q2 = 2 * ar.q;
 #pragma unroll
   for (int ss = 0; ss < RR; ++ss) {
     const int s = s0 + ss;
@@ -68,72 +98,79 @@ __device__ __forceinline__ void fwd_group(u64 (&x)[1 << RR], int base, int logN,
 #pragma unroll
     for (int i = 0; i < E; ++i) {
       if ((i & half) == 0) {
-        const u64 W = Wt[i >> (RR - ss)].x, Ws = Wt[i >> (RR - ss)].y;
         u64 U = x[i];
-        if constexpr (!GROW) U = U >= q2 ? U - q2 : U;
-        const u64 T = shoup_lazy(x[i + half], W, Ws, q);
+        if constexpr (!A::kGrow) U = U >= q2 ? U - q2 : U;
+        const u64 T = ar.mul(x[i + half], Wt[i >> (RR - ss)]);
         x[i] = U + T;
         x[i + half] = U + q2 - T;
       }
     }
   }
 }
-// [0, 4q) -> [0, q)
-template <int E>
-__device__ __forceinline__ void fwd_final(u64 (&x)[E], u64 q) {
-  const u64 q2 = 2 * q;
+// The transform's end: [0, 4q), or the grown range, -> [0, q)
+template <int E, class A>
+__device__ __forceinline__ void fwd_final(u64 (&x)[E], const A& ar) {
+  const u64 q = ar.q, q2 = 2 * q;
 #pragma unroll
   for (int i = 0; i < E; ++i) {
     u64 v = x[i];
-    v = v >= q2 ? v - q2 : v;
+    if constexpr (A::kPm) {
+      v = ar.m.fold(v);
+    } else if constexpr (A::kGrow) {
+      v -= __umul64hi(v, ar.m64) * q;  // floor(v m64 / 2^64) is short of floor(v / q) by at most 1
+    } else {
+      v = v >= q2 ? v - q2 : v;
+    }
     x[i] = v >= q ? v - q : v;
   }
 }
-// [0, 2^64) -> [0, q): one-word Barrett (floor(x m64 / 2^64) is short of
-// floor(x / q) by at most 1), then one conditional subtraction.
-template <int E>
-__device__ __forceinline__ void fwd_final_grow(u64 (&x)[E], u64 q, u64 m64) {
-#pragma unroll
-  for (int i = 0; i < E; ++i) {
-    const u64 v = x[i] - __umul64hi(x[i], m64) * q;
-    x[i] = v >= q ? v - q : v;
-  }
-}
-// Inverse (Gentleman-Sande) stages s0 + RR - 1 down to s0 on one group.
-template <int RR, class T>
-__device__ __forceinline__ void inv_group(T (&x)[1 << RR], int base, int logN, int s0, T q,
-                                          const ulonglong2* __restrict__ itw) {
+// Inverse (Gentleman-Sande) stages s0 + RR - 1 down to LO (the first LO of
+// the phase are left out) on one group.  Shoup: values stay in [0, 2q).  Pm:
+// sums double from [0, 4q) a stage.
+template <int RR, int LO, class A>
+__device__ __forceinline__ void inv_stages(typename A::T (&x)[1 << RR], int base, int logN, int s0, const A& ar,
+                                           const ulonglong2* __restrict__ itw) {
+  typedef typename A::T T;
   constexpr int E = 1 << RR;
-  const T q2 = 2 * q;
+  const T q2 = 2 * ar.q;
 #pragma unroll
-  for (int ss = RR - 1; ss >= 0; --ss) {
+  for (int ss = RR - 1; ss >= LO; --ss) {
     const int s = s0 + ss;
     const int half = 1 << (RR - 1 - ss);
     const int tbase = (1 << s) + (base >> (logN - s));
+    const T c = A::kPm ? (2 * q2) << (RR - 1 - ss) : q2;  // bound of V
     ulonglong2 Wt[1 << (RR - 1)];
 #pragma unroll
     for (int d = 0; d < (1 << ss); ++d) Wt[d] = __ldg(itw + tbase + d);
 #pragma unroll
     for (int i = 0; i < E; ++i) {
       if ((i & half) == 0) {
-        T W, Ws;
-        tw_split(Wt[i >> (RR - ss)], W, Ws);
         const T U = x[i], V = x[i + half];
         T S = U + V;
-        S = S >= q2 ? S - q2 : S;
+        if constexpr (!A::kPm) S = S >= q2 ? S - q2 : S;
         x[i] = S;
-        x[i + half] = lazy_mul((T)(U + q2 - V), W, Ws, q);
+        x[i + half] = ar.mul((T)(U + c - V), Wt[i >> (RR - ss)]);
       }
     }
   }
 }
+// A whole phase; Pm: the last stage's sums are folded below 2q.
+template <int RR, class A>
+__device__ __forceinline__ void inv_group(typename A::T (&x)[1 << RR], int base, int logN, int s0, const A& ar,
+                                          const ulonglong2* __restrict__ itw) {
+  inv_stages<RR, 0>(x, base, logN, s0, ar, itw);
+  if constexpr (A::kPm) {
+#pragma unroll
+    for (int i = 0; i < (1 << RR) / 2; ++i) x[i] = ar.m.fold(x[i]);
+  }
+}
 // times N^-1, [0, 2q) -> [0, q)
-template <int E, class T>
-__device__ __forceinline__ void inv_final(T (&x)[E], T q, T ninv, T ninvs) {
+template <int E, class A>
+__device__ __forceinline__ void inv_final(typename A::T (&x)[E], const A& ar, const ulonglong2& ninv) {
 #pragma unroll
   for (int i = 0; i < E; ++i) {
-    const T v = lazy_mul(x[i], ninv, ninvs, q);
-    x[i] = v >= q ? v - q : v;
+    const typename A::T v = ar.mul(x[i], ninv);
+    x[i] = v >= ar.q ? v - ar.q : v;
   }
 }
 
@@ -143,76 +180,60 @@ __device__ __forceinline__ void inv_final(T (&x)[E], T q, T ninv, T ninvs) {
 // twiddle, then every element is reduced to [0, q).  The same residues as
 // inv_group<3> at s0 = 0 followed by inv_final, with half the products of
 // the final scaling.
-template <class T>
-__device__ __forceinline__ void inv_group_last(T (&x)[8], int base, int logN, T q, const ulonglong2* __restrict__ itw,
-                                               T ninv, T ninvs) {
-  const T q2 = 2 * q;
-#pragma unroll
-  for (int ss = 2; ss >= 1; --ss) {
-    const int half = 1 << (2 - ss);
-    const int tbase = (1 << ss) + (base >> (logN - ss));
-    ulonglong2 Wt[4];
-#pragma unroll
-    for (int d = 0; d < (1 << ss); ++d) Wt[d] = __ldg(itw + tbase + d);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if ((i & half) == 0) {
-        T W, Ws;
-        tw_split(Wt[i >> (3 - ss)], W, Ws);
-        const T U = x[i], V = x[i + half];
-        T S = U + V;
-        S = S >= q2 ? S - q2 : S;
-        x[i] = S;
-        x[i + half] = lazy_mul((T)(U + q2 - V), W, Ws, q);
-      }
-    }
-  }
-  T Wn, Wns;
-  tw_split(__ldg(itw), Wn, Wns);
+template <class A>
+__device__ __forceinline__ void inv_group_last(typename A::T (&x)[8], int base, int logN, const A& ar,
+                                               const ulonglong2* __restrict__ itw, const ulonglong2& ninv) {
+  typedef typename A::T T;
+  inv_stages<3, 1>(x, base, logN, 0, ar, itw);
+  const T q = ar.q, q2 = 2 * q, c = A::kPm ? 8 * q2 : q2;
+  const ulonglong2 wn = __ldg(itw);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const T U = x[i], V = x[i + 4];
     T S = U + V;
-    S = S >= q2 ? S - q2 : S;
-    const T a = lazy_mul(S, ninv, ninvs, q), b = lazy_mul((T)(U + q2 - V), Wn, Wns, q);
+    if constexpr (!A::kPm) S = S >= q2 ? S - q2 : S;
+    const T a = ar.mul(S, ninv), b = ar.mul((T)(U + c - V), wn);
     x[i] = a >= q ? a - q : a;
     x[i + 4] = b >= q ? b - q : b;
   }
 }
 
-template <int RR, bool GROW = false>
-__device__ __forceinline__ void fwd_phase(u64* a, int N, int logN, int s0, u64 q, const ulonglong2* __restrict__ tw,
-                                          bool last) {
+template <int RR, class A>
+__device__ __forceinline__ void fwd_phase(u64* a, int N, int logN, int s0, const A& ar,
+                                          const ulonglong2* __restrict__ tw, bool last) {
   constexpr int E = 1 << RR;
   const int slog = logN - s0 - RR;  // log2 of the element stride inside a group
   const int groups = N >> RR;
   for (int g = threadIdx.x; g < groups; g += blockDim.x) {
     const int base = ((g >> slog) << (slog + RR)) + (g & ((1 << slog) - 1));
+    const u32 nb = (u32)nsw(base) * 8;
     u64 x[E];
 #pragma unroll
-    for (int i = 0; i < E; ++i) x[i] = a[nsw(base + (i << slog))];
-    fwd_group<RR, GROW>(x, base, logN, s0, q, tw);
-    if (last) fwd_final<E>(x, q);
+    for (int i = 0; i < E; ++i) x[i] = at(a, nb, i << slog);
+    fwd_group<RR>(x, base, logN, s0, ar, tw);
+    if (last) fwd_final<E>(x, ar);
 #pragma unroll
-    for (int i = 0; i < E; ++i) a[nsw(base + (i << slog))] = x[i];
+    for (int i = 0; i < E; ++i) at(a, nb, i << slog) = x[i];
   }
 }
 
-template <int RR, class T>
-__device__ __forceinline__ void inv_phase(T* a, int N, int logN, int s0, T q, const ulonglong2* __restrict__ itw,
-                                          bool last, T ninv, T ninvs) {
+template <int RR, class A>
+__device__ __forceinline__ void inv_phase(typename A::T* a, int N, int logN, int s0, const A& ar,
+                                          const ulonglong2* __restrict__ itw, bool last, const ulonglong2& ninv) {
+  typedef typename A::T T;
   constexpr int E = 1 << RR;
   const int slog = logN - s0 - RR;
   const int groups = N >> RR;
   for (int g = threadIdx.x; g < groups; g += blockDim.x) {
     const int base = ((g >> slog) << (slog + RR)) + (g & ((1 << slog) - 1));
+    const u32 nb = (u32)nsw(base) * (u32)sizeof(T);
     T x[E];
 #pragma unroll
-    for (int i = 0; i < E; ++i) x[i] = a[nsw(base + (i << slog))];
-    inv_group<RR>(x, base, logN, s0, q, itw);
-    if (last) inv_final<E>(x, q, ninv, ninvs);
+    for (int i = 0; i < E; ++i) x[i] = at(a, nb, i << slog);
+    inv_group<RR>(x, base, logN, s0, ar, itw);
+    if (last) inv_final<E>(x, ar, ninv);
 #pragma unroll
-    for (int i = 0; i < E; ++i) a[nsw(base + (i << slog))] = x[i];
+    for (int i = 0; i < E; ++i) at(a, nb, i << slog) = x[i];
   }
 }
 
@@ -220,101 +241,51 @@ __device__ __forceinline__ void inv_phase(T* a, int N, int logN, int s0, T q, co
 
 // a[0..N) in [0, 4q) on entry, [0, q) on exit.  Phases of three stages
 // from stage 0, then the remaining one or two.
-__device__ __forceinline__ void ntt_fwd_block(u64* a, int N, int logN, u64 q, const ulonglong2* __restrict__ tw) {
+template <class A>
+__device__ __forceinline__ void ntt_fwd_block(u64* a, int N, int logN, const A& ar, const ulonglong2* __restrict__ tw) {
   int s0 = 0;
   for (; s0 + 3 <= logN; s0 += 3) {
-    nttd::fwd_phase<3>(a, N, logN, s0, q, tw, s0 + 3 == logN);
+    nttd::fwd_phase<3>(a, N, logN, s0, ar, tw, s0 + 3 == logN);
     __syncthreads();
   }
   const int rem = logN - s0;
-  if (rem == 2) nttd::fwd_phase<2>(a, N, logN, s0, q, tw, true);
-  if (rem == 1) nttd::fwd_phase<1>(a, N, logN, s0, q, tw, true);
+  if (rem == 2) nttd::fwd_phase<2>(a, N, logN, s0, ar, tw, true);
+  if (rem == 1) nttd::fwd_phase<1>(a, N, logN, s0, ar, tw, true);
   if (rem) __syncthreads();
 }
 
 // a[0..N) in [0, 2q) on entry, [0, q) on exit.  The forward phases in
 // reverse order: the remainder first, then three stages at a time.
-template <class T>
-__device__ __forceinline__ void ntt_inv_block(T* a, int N, int logN, T q, const ulonglong2* __restrict__ itw, T ninv,
-                                              T ninvs) {
+template <class A>
+__device__ __forceinline__ void ntt_inv_block(typename A::T* a, int N, int logN, const A& ar,
+                                              const ulonglong2* __restrict__ itw, const ulonglong2& ninv) {
   const int rem = logN % 3;
   int s0 = logN - rem;
-  if (rem == 2) nttd::inv_phase<2>(a, N, logN, s0, q, itw, s0 == 0, ninv, ninvs);
-  if (rem == 1) nttd::inv_phase<1>(a, N, logN, s0, q, itw, s0 == 0, ninv, ninvs);
+  if (rem == 2) nttd::inv_phase<2>(a, N, logN, s0, ar, itw, s0 == 0, ninv);
+  if (rem == 1) nttd::inv_phase<1>(a, N, logN, s0, ar, itw, s0 == 0, ninv);
   if (rem) __syncthreads();
   for (s0 -= 3; s0 >= 0; s0 -= 3) {
-    nttd::inv_phase<3>(a, N, logN, s0, q, itw, s0 == 0, ninv, ninvs);
+    nttd::inv_phase<3>(a, N, logN, s0, ar, itw, s0 == 0, ninv);
     __syncthreads();
   }
 }
 
 __device__ __forceinline__ void ntt_fwd_view(u64* a, const DevView& V, int pi) {
-  ntt_fwd_block(a, V.N, V.logN, V.pr[pi].q, V.twp + (size_t)pi * V.N);
+  const DevPrime P = V.pr[pi];
+  const ulonglong2* tw = V.twp + (size_t)pi * V.N;
+  if (P.pm)
+    ntt_fwd_block(a, V.N, V.logN, nttd::Pm(P), tw);
+  else
+    ntt_fwd_block(a, V.N, V.logN, nttd::Shoup<false>(P), tw);
 }
 __device__ __forceinline__ void ntt_inv_view(u64* a, const DevView& V, int pi) {
   const DevPrime P = V.pr[pi];
-  ntt_inv_block(a, V.N, V.logN, P.q, V.itwp + (size_t)pi * V.N, P.ninv, P.ninvs);
-}
-
-// The same transforms with log2 N fixed at compile time: the phase bounds,
-// strides and shift amounts become constants.
-template <int LOGN>
-__device__ __forceinline__ void ntt_fwd_fixed(u64* a, u64 q, const ulonglong2* __restrict__ tw) {
-  constexpr int N = 1 << LOGN, REM = LOGN % 3;
-#pragma unroll
-  for (int s0 = 0; s0 + 3 <= LOGN; s0 += 3) {
-    nttd::fwd_phase<3>(a, N, LOGN, s0, q, tw, s0 + 3 == LOGN);
-    __syncthreads();
-  }
-  if constexpr (REM == 2) {
-    nttd::fwd_phase<2>(a, N, LOGN, LOGN - 2, q, tw, true);
-    __syncthreads();
-  }
-  if constexpr (REM == 1) {
-    nttd::fwd_phase<1>(a, N, LOGN, LOGN - 1, q, tw, true);
-    __syncthreads();
-  }
-}
-template <int LOGN>
-__device__ __forceinline__ void ntt_inv_fixed(u64* a, u64 q, const ulonglong2* __restrict__ itw, u64 ninv,
-                                              u64 ninvs) {
-  constexpr int N = 1 << LOGN, REM = LOGN % 3, TOP = LOGN - REM;
-  if constexpr (REM == 2) {
-    nttd::inv_phase<2>(a, N, LOGN, TOP, q, itw, TOP == 0, ninv, ninvs);
-    __syncthreads();
-  }
-  if constexpr (REM == 1) {
-    nttd::inv_phase<1>(a, N, LOGN, TOP, q, itw, TOP == 0, ninv, ninvs);
-    __syncthreads();
-  }
-#pragma unroll
-  for (int s0 = TOP - 3; s0 >= 0; s0 -= 3) {
-    nttd::inv_phase<3>(a, N, LOGN, s0, q, itw, s0 == 0, ninv, ninvs);
-    __syncthreads();
-  }
-}
-
-// ntt_fwd_view / ntt_inv_view with the ring sizes of the workloads
-// (N = 4096, 8192, 16384) compiled for their fixed size.
-__device__ __forceinline__ void ntt_fwd_fast(u64* a, const DevView& V, int pi) {
-  const ulonglong2* tw = V.twp + (size_t)pi * V.N;
-  const u64 q = V.pr[pi].q;
-  switch (V.logN) {
-    case 12: ntt_fwd_fixed<12>(a, q, tw); break;
-    case 13: ntt_fwd_fixed<13>(a, q, tw); break;
-    case 14: ntt_fwd_fixed<14>(a, q, tw); break;
-    default: ntt_fwd_block(a, V.N, V.logN, q, tw); break;
-  }
-}
-__device__ __forceinline__ void ntt_inv_fast(u64* a, const DevView& V, int pi) {
   const ulonglong2* itw = V.itwp + (size_t)pi * V.N;
-  const DevPrime P = V.pr[pi];
-  switch (V.logN) {
-    case 12: ntt_inv_fixed<12>(a, P.q, itw, P.ninv, P.ninvs); break;
-    case 13: ntt_inv_fixed<13>(a, P.q, itw, P.ninv, P.ninvs); break;
-    case 14: ntt_inv_fixed<14>(a, P.q, itw, P.ninv, P.ninvs); break;
-    default: ntt_inv_block(a, V.N, V.logN, P.q, itw, P.ninv, P.ninvs); break;
-  }
+  const ulonglong2 ninv = make_ulonglong2(P.ninv, P.ninvs);
+  if (P.pm)
+    ntt_inv_block(a, V.N, V.logN, nttd::Pm(P), itw, ninv);
+  else
+    ntt_inv_block(a, V.N, V.logN, nttd::Shoup<false>(P), itw, ninv);
 }
 
 // Row accessors for the global-to-global transforms.  A functor with a
@@ -412,69 +383,97 @@ __device__ __forceinline__ void store_run(const u64 (&x)[E], const Store& st, in
 // of the global load and the last R stages (R = 1, 2 or 3, the rest after
 // radix-8 phases) on those of the global store, so of the log2(N) stages
 // only the middle ones take shared-memory phases (N = 8192: three instead
-// of five).  The butterflies and their order are those of ntt_fwd_fixed /
-// ntt_inv_fixed, so are the results.  ld(x) returns input element x (forward:
+// of five).  The butterflies are those of ntt_fwd_block / ntt_inv_block, so
+// are the results.  ld(x) returns input element x (forward:
 // in [0, 4q); inverse: in [0, 2q)); st(x, v) receives output element x,
-// reduced.  Every read through ld happens before the first barrier and
-// every st after the last, so input and output rows may alias.  Every
+// reduced.  Every read through ld comes before a barrier of the whole block
+// that every st comes after, so input and output rows may alias.  Every
 // thread of the block must call these.
-// GROW (q < 2^59): butterflies without the reduction of their sum input,
-// one Barrett reduction (m64 = floor(2^64 / q)) at the store; the same
-// residues.
-template <int LOGN, bool GROW, class Load, class Store>
-__device__ __forceinline__ void ntt_fwd_fused(u64* a, const Load& ld, const Store& st, u64 q, u64 m64,
+// Only the exchange around stages 0-2 crosses the whole block.  After stage 2
+// the transform falls into 8 parts of N/8 elements, each the work of N/64
+// consecutive threads, which one named barrier joins; after stage 5 the parts
+// of N/64 elements lie within a warp's 256 elements, and the short last (first)
+// phase keeps to the warp's own elements too, so warp barriers do and the warps
+// of a block drift apart and fill both the multiply-add and the ALU pipe.
+template <int LOGN>
+__device__ __forceinline__ void part_sync() {
+  constexpr int T = 1 << (LOGN - 6);
+  const int sets = (int)blockDim.x / T;
+  if (sets > 1 && sets <= 15)
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / T), "n"(T) : "memory");
+  else
+    __syncthreads();
+}
+template <int LOGN, class A, class Load, class Store>
+__device__ __forceinline__ void ntt_fwd_fused(u64* a, const Load& ld, const Store& st, const A& ar,
                                               const ulonglong2* __restrict__ tw) {
   constexpr int N = 1 << LOGN, R = (LOGN - 4) % 3 + 1, M = (LOGN - 3 - R) / 3, S8 = LOGN - 3;
   for (int g = threadIdx.x; g < (N >> 3); g += blockDim.x) {  // stages 0-2
     u64 x[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) x[i] = ld(g + (i << S8));
-    nttd::fwd_group<3, GROW>(x, g, LOGN, 0, q, tw);
+    nttd::fwd_group<3>(x, g, LOGN, 0, ar, tw);
+    const u32 nb = (u32)nsw(g) * 8;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) a[nsw(g + (i << S8))] = x[i];
+    for (int i = 0; i < 8; ++i) at(a, nb, i << S8) = x[i];
   }
   __syncthreads();
 #pragma unroll
   for (int m = 0; m < M; ++m) {
-    nttd::fwd_phase<3, GROW>(a, N, LOGN, 3 + 3 * m, q, tw, false);
-    __syncthreads();
-  }
-  for (int g = threadIdx.x; g < (N >> R); g += blockDim.x) {  // stages LOGN-R .. LOGN-1
-    const int base = g << R;
-    u64 x[1 << R];
-#pragma unroll
-    for (int i = 0; i < (1 << R); ++i) x[i] = a[nsw(base + i)];
-    nttd::fwd_group<R, GROW>(x, base, LOGN, LOGN - R, q, tw);
-    if constexpr (GROW)
-      nttd::fwd_final_grow<1 << R>(x, q, m64);
+    nttd::fwd_phase<3>(a, N, LOGN, 3 + 3 * m, ar, tw, false);
+    if (m == 0)
+      part_sync<LOGN>();
     else
-      nttd::fwd_final<1 << R>(x, q);
-    store_run<1 << R>(x, st, base);
+      __syncwarp();
+  }
+  for (int g = threadIdx.x; g < (N >> 3); g += blockDim.x) {  // stages LOGN-R .. LOGN-1 of the warp's 256 elements
+#pragma unroll
+    for (int it = 0; it < (8 >> R); ++it) {
+      const int base = (((g & ~31) << 3) + ((it * 32 + (g & 31)) << R));
+      const u32 nb = (u32)nsw(base) * 8;
+      u64 x[1 << R];
+#pragma unroll
+      for (int i = 0; i < (1 << R); ++i) x[i] = at(a, nb, i);
+      nttd::fwd_group<R>(x, base, LOGN, LOGN - R, ar, tw);
+      nttd::fwd_final<1 << R>(x, ar);
+      store_run<1 << R>(x, st, base);
+    }
   }
 }
-template <int LOGN, class T, class Load, class Store>
-__device__ __forceinline__ void ntt_inv_fused(T* a, const Load& ld, const Store& st, T q,
-                                              const ulonglong2* __restrict__ itw, T ninv, T ninvs) {
+template <int LOGN, class A, class Load, class Store>
+__device__ __forceinline__ void ntt_inv_fused(typename A::T* a, const Load& ld, const Store& st, const A& ar,
+                                              const ulonglong2* __restrict__ itw, const ulonglong2& ninv) {
+  typedef typename A::T T;
   constexpr int N = 1 << LOGN, R = (LOGN - 4) % 3 + 1, M = (LOGN - 3 - R) / 3, S8 = LOGN - 3;
-  for (int g = threadIdx.x; g < (N >> R); g += blockDim.x) {  // stages LOGN-1 .. LOGN-R
-    const int base = g << R;
-    T x[1 << R];
-    load_run<1 << R>(x, ld, base);
-    nttd::inv_group<R>(x, base, LOGN, LOGN - R, q, itw);
+  for (int g = threadIdx.x; g < (N >> 3); g += blockDim.x) {  // stages LOGN-1 .. LOGN-R of the warp's 256 elements
 #pragma unroll
-    for (int i = 0; i < (1 << R); ++i) a[nsw(base + i)] = x[i];
+    for (int it = 0; it < (8 >> R); ++it) {
+      const int base = (((g & ~31) << 3) + ((it * 32 + (g & 31)) << R));
+      T x[1 << R];
+      load_run<1 << R>(x, ld, base);
+      nttd::inv_group<R>(x, base, LOGN, LOGN - R, ar, itw);
+      const u32 nb = (u32)nsw(base) * (u32)sizeof(T);
+#pragma unroll
+      for (int i = 0; i < (1 << R); ++i) at(a, nb, i) = x[i];
+    }
   }
-  __syncthreads();
+  __syncwarp();
 #pragma unroll
   for (int m = M - 1; m >= 0; --m) {
-    nttd::inv_phase<3>(a, N, LOGN, 3 + 3 * m, q, itw, false, ninv, ninvs);
-    __syncthreads();
+    nttd::inv_phase<3>(a, N, LOGN, 3 + 3 * m, ar, itw, false, ninv);
+    if (m > 1)
+      __syncwarp();
+    else if (m == 1)
+      part_sync<LOGN>();
+    else
+      __syncthreads();
   }
   for (int g = threadIdx.x; g < (N >> 3); g += blockDim.x) {  // stages 2-0 and N^-1
+    const u32 nb = (u32)nsw(g) * (u32)sizeof(T);
     T x[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = a[nsw(g + (i << S8))];
-    nttd::inv_group_last(x, g, LOGN, q, itw, ninv, ninvs);
+    for (int i = 0; i < 8; ++i) x[i] = at(a, nb, i << S8);
+    nttd::inv_group_last(x, g, LOGN, ar, itw, ninv);
 #pragma unroll
     for (int i = 0; i < 8; ++i) st(g + (i << S8), x[i]);
   }
@@ -482,42 +481,55 @@ __device__ __forceinline__ void ntt_inv_fused(T* a, const Load& ld, const Store&
 
 // Global-to-global transforms of row pi with the fused forms for the ring
 // sizes of the workloads (N = 4096, 8192, 16384), else load, block
-// transform and store.
+// transform and store; each in the arithmetic of the row's prime.
+template <class A, class Load, class Store>
+__device__ __forceinline__ void ntt_fwd_with(u64* a, const Load& ld, const Store& st, const A& ar, int N, int logN,
+                                             const ulonglong2* __restrict__ tw) {
+  switch (logN) {
+    case 12: ntt_fwd_fused<12>(a, ld, st, ar, tw); return;
+    case 13: ntt_fwd_fused<13>(a, ld, st, ar, tw); return;
+    case 14: ntt_fwd_fused<14>(a, ld, st, ar, tw); return;
+    default: break;
+  }
+  for (int x = threadIdx.x; x < N; x += blockDim.x) a[nsw(x)] = ld(x);
+  __syncthreads();
+  ntt_fwd_block(a, N, logN, ar, tw);
+  for (int x = threadIdx.x; x < N; x += blockDim.x) st(x, a[nsw(x)]);
+}
+template <class A, class Load, class Store>
+__device__ __forceinline__ void ntt_inv_with(typename A::T* a, const Load& ld, const Store& st, const A& ar, int N,
+                                             int logN, const ulonglong2* __restrict__ itw, const ulonglong2& ninv) {
+  switch (logN) {
+    case 12: ntt_inv_fused<12>(a, ld, st, ar, itw, ninv); return;
+    case 13: ntt_inv_fused<13>(a, ld, st, ar, itw, ninv); return;
+    case 14: ntt_inv_fused<14>(a, ld, st, ar, itw, ninv); return;
+    default: break;
+  }
+  for (int x = threadIdx.x; x < N; x += blockDim.x) a[nsw(x)] = ld(x);
+  __syncthreads();
+  ntt_inv_block(a, N, logN, ar, itw, ninv);
+  for (int x = threadIdx.x; x < N; x += blockDim.x) st(x, a[nsw(x)]);
+}
 template <class Load, class Store>
 __device__ __forceinline__ void ntt_fwd_gg(u64* a, const Load& ld, const Store& st, const DevView& V, int pi) {
   const ulonglong2* tw = V.twp + (size_t)pi * V.N;
   const DevPrime P = V.pr[pi];
-  const u64 q = P.q;
-  // values reach (4 + 2 log2 N) q <= 32 q without per-stage reduction
-  const bool grow = q < (1ull << 59);
-  switch (V.logN * 2 + (grow ? 1 : 0)) {
-    case 12 * 2: ntt_fwd_fused<12, false>(a, ld, st, q, P.m64, tw); return;
-    case 12 * 2 + 1: ntt_fwd_fused<12, true>(a, ld, st, q, P.m64, tw); return;
-    case 13 * 2: ntt_fwd_fused<13, false>(a, ld, st, q, P.m64, tw); return;
-    case 13 * 2 + 1: ntt_fwd_fused<13, true>(a, ld, st, q, P.m64, tw); return;
-    case 14 * 2: ntt_fwd_fused<14, false>(a, ld, st, q, P.m64, tw); return;
-    case 14 * 2 + 1: ntt_fwd_fused<14, true>(a, ld, st, q, P.m64, tw); return;
-    default: break;
-  }
-  for (int x = threadIdx.x; x < V.N; x += blockDim.x) a[nsw(x)] = ld(x);
-  __syncthreads();
-  ntt_fwd_block(a, V.N, V.logN, q, tw);
-  for (int x = threadIdx.x; x < V.N; x += blockDim.x) st(x, a[nsw(x)]);
+  if (P.pm)
+    ntt_fwd_with(a, ld, st, nttd::Pm(P), V.N, V.logN, tw);
+  else if (P.q < (1ull << 59))
+    ntt_fwd_with(a, ld, st, nttd::Shoup<true>(P), V.N, V.logN, tw);
+  else
+    ntt_fwd_with(a, ld, st, nttd::Shoup<false>(P), V.N, V.logN, tw);
 }
 template <class Load, class Store>
 __device__ __forceinline__ void ntt_inv_gg(u64* a, const Load& ld, const Store& st, const DevView& V, int pi) {
   const ulonglong2* itw = V.itwp + (size_t)pi * V.N;
   const DevPrime P = V.pr[pi];
-  switch (V.logN) {
-    case 12: ntt_inv_fused<12>(a, ld, st, P.q, itw, P.ninv, P.ninvs); return;
-    case 13: ntt_inv_fused<13>(a, ld, st, P.q, itw, P.ninv, P.ninvs); return;
-    case 14: ntt_inv_fused<14>(a, ld, st, P.q, itw, P.ninv, P.ninvs); return;
-    default: break;
-  }
-  for (int x = threadIdx.x; x < V.N; x += blockDim.x) a[nsw(x)] = ld(x);
-  __syncthreads();
-  ntt_inv_block(a, V.N, V.logN, P.q, itw, P.ninv, P.ninvs);
-  for (int x = threadIdx.x; x < V.N; x += blockDim.x) st(x, a[nsw(x)]);
+  const ulonglong2 ninv = make_ulonglong2(P.ninv, P.ninvs);
+  if (P.pm)
+    ntt_inv_with(a, ld, st, nttd::Pm(P), V.N, V.logN, itw, ninv);
+  else
+    ntt_inv_with(a, ld, st, nttd::Shoup<false>(P), V.N, V.logN, itw, ninv);
 }
 
 // ntt_inv_gg for a modulus q_pi below 2^30 (the plaintext modulus) in 32-bit
@@ -525,17 +537,6 @@ __device__ __forceinline__ void ntt_inv_gg(u64* a, const Load& ld, const Store& 
 // u32, st(x, v) receives it reduced.  The same residues as ntt_inv_gg.
 template <class Load, class Store>
 __device__ __forceinline__ void ntt_inv_gg_small(u32* a, const Load& ld, const Store& st, const DevView& V, int pi) {
-  const ulonglong2* itw = V.itwp + (size_t)pi * V.N;
   const DevPrime P = V.pr[pi];
-  const u32 q = (u32)P.q, ninv = (u32)P.ninv, ninvs = (u32)(P.ninvs >> 32);
-  switch (V.logN) {
-    case 12: ntt_inv_fused<12>(a, ld, st, q, itw, ninv, ninvs); return;
-    case 13: ntt_inv_fused<13>(a, ld, st, q, itw, ninv, ninvs); return;
-    case 14: ntt_inv_fused<14>(a, ld, st, q, itw, ninv, ninvs); return;
-    default: break;
-  }
-  for (int x = threadIdx.x; x < V.N; x += blockDim.x) a[nsw(x)] = ld(x);
-  __syncthreads();
-  ntt_inv_block(a, V.N, V.logN, q, itw, ninv, ninvs);
-  for (int x = threadIdx.x; x < V.N; x += blockDim.x) st(x, a[nsw(x)]);
+  ntt_inv_with(a, ld, st, nttd::Small(P), V.N, V.logN, V.itwp + (size_t)pi * V.N, make_ulonglong2(P.ninv, P.ninvs));
 }

@@ -1052,13 +1052,15 @@ int pepsi_setup(const pepsi_params* params, uint64_t key_seed, pepsi_ctx** out) 
   // auxiliary base B: primes with log2 B >= log2(t N Q G) + 3, G the
   // longest run of layers whose exact products are summed before rounding
   // (and, for the value modes, N t / 2 times more: the product with a value
-  // plaintext of centred coefficients).  59-bit primes where as few of them
-  // cover the bound as of 61-bit ones (their forward transforms then skip the
-  // per-stage reduction: 32 q < 2^64), else 61-bit primes.
+  // plaintext of centred coefficients).  57-bit primes (folding products), or
+  // 59-bit ones (forward transforms without the per-stage reduction), where as
+  // few of them cover the bound as of 61-bit ones, else 61-bit primes.
   c->value_margin = params->server_values != 0 && c->rescale_cap > 1;
   const double needB = std::log2((double)c->t) + c->logN + lq + std::ceil(std::log2((double)c->rescale_cap)) + 3.0 +
                        (c->value_margin ? std::ceil(c->logN + std::log2((double)c->t) - 1.0) : 0.0);
-  const int bbits = std::ceil(needB / 58.9) <= std::ceil(needB / 60.9) ? 59 : 61;
+  int bbits = 61;
+  for (int b : {59, 57})
+    if (std::ceil(needB / (b - 0.1)) <= std::ceil(needB / 60.9)) bbits = b;
   double haveB = 0;
   std::vector<u64> taken = c->Q;
   while (haveB < needB) {
@@ -1096,7 +1098,7 @@ int pepsi_setup(const pepsi_params* params, uint64_t key_seed, pepsi_ctx** out) 
     if (i < c->k) c->psi.push_back(root);
     if (i == np - 1) c->psi_t = root;
     pr[i] = hostmath::make_prime(all[i], c->N);
-    hostmath::twiddles(all[i], root, c->N, &tw[(size_t)i * c->N], &tws[(size_t)i * c->N], &itw[(size_t)i * c->N],
+    hostmath::twiddles(pr[i], root, c->N, &tw[(size_t)i * c->N], &tws[(size_t)i * c->N], &itw[(size_t)i * c->N],
                        &itws[(size_t)i * c->N]);
   }
   RnsConst rcst;
@@ -1673,7 +1675,7 @@ int pepsi_autotune(pepsi_ctx* c, int set_id, const uint64_t* cts, void* stream, 
   c->chunk = best_chunk;
   // 2: threads per transform block (the default, half and twice it)
   if (!rc) {
-    const int def = c->N >= 16384 ? 1024 : std::max(32, std::min(512, c->N / 8));
+    const int def = c->N >= 16384 ? 1024 : std::max(32, std::min(256, c->N / 8));
     int best_nt = 0;
     for (int nt : {def / 2, def * 2}) {
       if (nt < 64 || nt > 1024) continue;
