@@ -192,8 +192,8 @@ typedef struct {
                            fill the GPU with more blocks per launch and need more
                            scratch (about 4.7 MB per layer at N = 8192, k = 4) */
   uint32_t ntt_threads; /* threads per block of the ciphertext transforms (the NTTs and
-                           the kernels fused with them): 0 = the default for N (N / 8,
-                           at most 256; 1024 at N = 16384), else a power of two in
+                           the kernels fused with them): 0 = the default for N (N / 16
+                           from N = 4096 on, else N / 8), else a power of two in
                            64..1024 */
   uint32_t relin_fused; /* 1 (default): where a relinearised product only feeds the
                            affine step after it (u = R(h'^2) - 3h' and the like), the

@@ -17,7 +17,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJDIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libpepsi_gb300.so")
-SOURCES = ["kernels.cu", "mac_planes.cu", "pepsi.cu", "engine.cu", "host.cpp"]
+SOURCES = ["tensor.cu", "relin.cu", "transforms.cu", "client.cu", "mac_planes.cu", "rns.cu", "kernels.cu", "pepsi.cu",
+           "engine.cu", "host.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -47,7 +48,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         obj = os.path.join(OBJDIR, src + ".o")
         if force or _stale(obj, [path] + headers):
             cmd = [nv, "-c", path, "-o", obj] + common
-            cmd += ARCH + ["-lineinfo", "--expt-relaxed-constexpr", "--split-compile=0"]
+            cmd += ARCH + ["-lineinfo", "--expt-relaxed-constexpr"]
             if not src.endswith(".cu"):
                 cmd += ["-x", "cu", "-diag-suppress", "20208"]
             jobs.append(cmd)

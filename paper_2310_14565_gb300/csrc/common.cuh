@@ -40,9 +40,11 @@ struct DevPrime {
 __host__ __device__ __forceinline__ u64 to_split(u64 x, u64 s) { return ((x >> s) << 32) | (x & ((1ull << s) - 1)); }
 __host__ __device__ __forceinline__ u64 from_split(u64 w, u64 s) { return ((w >> 32) << s) | (w & 0xFFFFFFFFull); }
 
-// Constants of the exact RNS conversions (all residues reduced, Shoup
-// companions where the value multiplies a varying operand).
+// Constants of the exact RNS conversions (all residues reduced, companions
+// where the value multiplies a varying operand: Shoup's, or with pm the folding
+// products' for cq, qb, qinv_b, cb and bq).
 struct RnsConst {
+  u64 pm;  // every prime has folding products and their inputs fit (host.cpp)
   // Garner over Q: cq[i][j] = q_j^-1 mod q_i (j < i)
   u64 cq[PEPSI_MAXQ][PEPSI_MAXQ], cqs[PEPSI_MAXQ][PEPSI_MAXQ];
   // radices of Q in B for Horner's rule: qb[j][l] = q_l mod p_j (Shoup)
@@ -126,6 +128,11 @@ struct PmMul {
           "r"(d));
     return r;
   }
+  // x c for c < 2^32 and x c < 2^(n+32) -> below 2^n + 2^32 d
+  __device__ __forceinline__ u64 mul_small(u64 x, u32 c) const {
+    const u64 L = (u64)(u32)x * c, M = (u64)(u32)(x >> 32) * c + (L >> 32);
+    return (u64)(u32)(M >> n32) * d + ((u64)((u32)M & nmask) << 32 | (u32)L);
+  }
   // x < 2^(n+5) -> [0, 2^n + 2^29) with x = x1 2^n + x0: x0 + x1 d
   __device__ __forceinline__ u64 fold(u64 x) const {
     const u32 h = (u32)(x >> 32);
@@ -165,6 +172,18 @@ __device__ __forceinline__ u64 addmod(u64 a, u64 b, u64 q) {
   return s >= q ? s - q : s;
 }
 __device__ __forceinline__ u64 submod(u64 a, u64 b, u64 q) { return a >= b ? a - b : a + q - b; }
+// (hi:lo) < 2^(2n+5) mod q = 2^n - d (a sum of up to 32 products of residues): two
+// folds, three wide products against the six or so of Barrett's.  d < 2^(n/2 - 4)
+// (the condition of pm), so the second fold's product stays below 2^(n-3).
+__device__ __forceinline__ u64 pm_reduce(u64 hi, u64 lo, const PmMul& m, int n) {
+  const u64 h = hi << (64 - n) | lo >> n;
+  const u64 low = (u64)((u32)(lo >> 32) & m.nmask) << 32 | (u32)lo;
+  const u64 L = (u64)(u32)h * m.d, M = (u64)(u32)(h >> 32) * m.d + (L >> 32);  // h d = M 2^32 + L mod 2^32
+  const u64 f = (u64)((u32)M & m.nmask) << 32 | (u32)L;
+  u64 r = low + f + (u64)(u32)(M >> m.n32) * m.d;  // M / 2^(n-32) = h d / 2^n < 32 d < 2^32
+  r = m.fold(r);
+  return r >= m.q ? r - m.q : r;
+}
 // 128-bit accumulate acc += a*b
 __device__ __forceinline__ void mac128(u64& lo, u64& hi, u64 a, u64 b) {
   asm("mad.lo.cc.u64 %0, %2, %3, %0;\n\tmadc.hi.u64 %1, %2, %3, %1;" : "+l"(lo), "+l"(hi) : "l"(a), "l"(b));

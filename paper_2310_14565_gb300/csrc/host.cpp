@@ -168,18 +168,43 @@ static std::vector<u64> garner(const std::vector<u64>& x, const std::vector<u64>
   return v;
 }
 
+// Whether the folding products modulo p take inputs below x: the conditions
+// of PmMul::mul (32-bit parts, 64-bit sums, a result below 2 p) and of
+// PmMul::fold.
+static bool folds_below(const DevPrime& p, u128 x) {
+  if (!p.pm) return false;
+  const u128 x1 = x >> p.s, top = ((u128)1 << p.s) + x1 + 1;  // x1, floor(S / 2^n)
+  return x1 < ((u128)1 << 32) - ((u128)1 << p.s) && top < ((u128)1 << 32) &&
+         ((u128)1 << p.nbits) + top * p.d < 2 * (u128)p.q && (x >> p.nbits) * p.d < ((u128)1 << 31);
+}
+
 void rns_constants(const std::vector<u64>& Q, const std::vector<u64>& B, u64 t, RnsConst* rc) {
   const size_t k = Q.size(), kb = B.size();
   *rc = RnsConst{};
+  // folding products throughout when every intermediate value of the conversions
+  // fits: Garner steps below 3 q_i + 4 q_i (digits of other primes below 4 q_i),
+  // Horner sums below 2 p + a digit, t x below 2^(n+32)
+  std::vector<u64> all = Q;
+  all.insert(all.end(), B.begin(), B.end());
+  const u64 qmax = *std::max_element(Q.begin(), Q.end()), bmax = *std::max_element(B.begin(), B.end());
+  bool pm = t < (1ull << 27);
+  for (size_t i = 0; i < all.size() && pm; ++i) {
+    const DevPrime p = make_prime(all[i], 1);
+    const u64 own = i < k ? qmax : bmax, other = i < k ? bmax : qmax;
+    pm = folds_below(p, 8 * (u128)p.q) && folds_below(p, 2 * (u128)p.q + other) && own < 4 * p.q &&
+         (i < k || other < 2 * p.q) && ((u128)1 << p.nbits) + (u128)(t + 1) * p.d < 2 * (u128)p.q;
+  }
+  rc->pm = pm ? 1 : 0;
+  auto comp = [&](u64 w, u64 q) { return pm ? companion(w, make_prime(q, 1)) : shoup_of(w, q); };
   for (size_t i = 0; i < k; ++i)
     for (size_t j = 0; j < i; ++j) {
       rc->cq[i][j] = invmod(Q[j] % Q[i], Q[i]);
-      rc->cqs[i][j] = shoup_of(rc->cq[i][j], Q[i]);
+      rc->cqs[i][j] = comp(rc->cq[i][j], Q[i]);
     }
   for (size_t i = 0; i < kb; ++i)
     for (size_t j = 0; j < i; ++j) {
       rc->cb[i][j] = invmod(B[j] % B[i], B[i]);
-      rc->cbs[i][j] = shoup_of(rc->cb[i][j], B[i]);
+      rc->cbs[i][j] = comp(rc->cb[i][j], B[i]);
     }
   auto prod_mod = [](const std::vector<u64>& ps, size_t upto, u64 m) {
     u64 r = 1 % m;
@@ -189,13 +214,13 @@ void rns_constants(const std::vector<u64>& Q, const std::vector<u64>& B, u64 t, 
   for (size_t j = 0; j < kb; ++j) {
     for (size_t l = 0; l < k; ++l) {
       rc->qb[j][l] = Q[l] % B[j];
-      rc->qbs[j][l] = shoup_of(rc->qb[j][l], B[j]);
+      rc->qbs[j][l] = comp(rc->qb[j][l], B[j]);
     }
     rc->qmodb[j] = prod_mod(Q, k, B[j]);
     const u64 inv2 = invmod(2, B[j]);
     rc->qhalf_b[j] = mulmod((rc->qmodb[j] + B[j] - 1) % B[j], inv2, B[j]);
     rc->qinv_b[j] = invmod(rc->qmodb[j], B[j]);
-    rc->qinv_bs[j] = shoup_of(rc->qinv_b[j], B[j]);
+    rc->qinv_bs[j] = comp(rc->qinv_b[j], B[j]);
     rc->t_b[j] = t % B[j];
     rc->t_bs[j] = shoup_of(rc->t_b[j], B[j]);
   }
@@ -216,7 +241,7 @@ void rns_constants(const std::vector<u64>& Q, const std::vector<u64>& B, u64 t, 
   for (size_t i = 0; i < k; ++i) {
     for (size_t j = 0; j < kb; ++j) {
       rc->bq[i][j] = B[j] % Q[i];
-      rc->bqs[i][j] = shoup_of(rc->bq[i][j], Q[i]);
+      rc->bqs[i][j] = comp(rc->bq[i][j], Q[i]);
     }
     rc->bmodq[i] = prod_mod(B, kb, Q[i]);
   }

@@ -71,8 +71,12 @@ void launch_unpack_planes(const DevView& V, const PlaneTab& P, int ell, int l0, 
 // Request words [ell][2][k][N] (reduced, or split format) to byte planes, steps [ks0, ks1) (-1: all).
 void launch_pack_request(const DevView& V, const u64* words, bool split, int ell, u32* C, cudaStream_t st, int ks0 = 0,
                          int ks1 = -1);
-// Shared-memory limits of the kernels above (called by kernels_init).
+// Shared-memory limits of each source file's kernels (called by kernels_init).
 cudaError_t mac_planes_init();
+cudaError_t transforms_init();
+cudaError_t tensor_init();
+cudaError_t relin_init();
+cudaError_t client_init(int N);
 
 // Fused ct x pt multiply-accumulate of a regenerated chunk: H[l][c][p][n] = sum_j C[j][c][p][n] *
 // P[l][j][p][n] mod q_p.  C a prepared request (split operand format and half sums), P [L][ell][k][N] in the

@@ -1052,15 +1052,16 @@ int pepsi_setup(const pepsi_params* params, uint64_t key_seed, pepsi_ctx** out) 
   // auxiliary base B: primes with log2 B >= log2(t N Q G) + 3, G the
   // longest run of layers whose exact products are summed before rounding
   // (and, for the value modes, N t / 2 times more: the product with a value
-  // plaintext of centred coefficients).  57-bit primes (folding products), or
-  // 59-bit ones (forward transforms without the per-stage reduction), where as
-  // few of them cover the bound as of 61-bit ones, else 61-bit primes.
+  // plaintext of centred coefficients).  57-bit primes (folding products) where
+  // they are at most one more than 61-bit ones would be, else 59-bit ones (forward
+  // transforms without the per-stage reduction) where as few, else 61-bit.
   c->value_margin = params->server_values != 0 && c->rescale_cap > 1;
   const double needB = std::log2((double)c->t) + c->logN + lq + std::ceil(std::log2((double)c->rescale_cap)) + 3.0 +
                        (c->value_margin ? std::ceil(c->logN + std::log2((double)c->t) - 1.0) : 0.0);
-  int bbits = 61;
-  for (int b : {59, 57})
-    if (std::ceil(needB / (b - 0.1)) <= std::ceil(needB / 60.9)) bbits = b;
+  const double n61 = std::ceil(needB / 60.9);
+  const int bbits = std::ceil(needB / 56.9) <= n61 + 1 && std::ceil(needB / 56.9) <= PEPSI_MAXB ? 57
+                    : std::ceil(needB / 58.9) <= n61                                            ? 59
+                                                                                                : 61;
   double haveB = 0;
   std::vector<u64> taken = c->Q;
   while (haveB < needB) {
