@@ -119,6 +119,7 @@ __device__ __forceinline__ void encode_block(u64* a, const Load& ld, u32* m, con
 // Block (layer l, j-chunk): bit planes of the layer's codewords, encoded
 // (inverse NTT mod t of the slot vector in bit-reversed order), centred
 // lift into each q_p and forward NTT; stored in the split operand format.
+template <bool PM>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ptgen(DevView V, const uint16_t* __restrict__ pos, int ell, int h, int JC, u64* P) {
   extern __shared__ u64 sm[];
   const int N = V.N, k = V.k;
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ptgen(DevView V, const u
       // centred lift to q_p on the load, split operand format on the store
       const u64 q = V.pr[p].q, sp = V.pr[p].split;
       u64* out = P + (((size_t)l * ell + j) * k + p) * N;
-      ntt_fwd_gg(
+      ntt_fwd_gg<PM>(
           poly,
           [&](int i) -> u64 {
             const u64 m = mbuf[i];
@@ -206,6 +207,7 @@ __device__ __forceinline__ u64 smod_dev(i64 v, u64 q) { return v >= 0 ? (u64)v :
 
 // Block per ciphertext j: encode bit plane j, then for each prime sample
 // a, compute c0 = e - a s + round(Q m / t), c1 = a (coefficient form).
+template <bool PM>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_encrypt(DevView V, const uint16_t* __restrict__ pos, int h, const u64* __restrict__ s_ntt, u64 seed,
                           u64 idx0, u64* cts) {
   extern __shared__ u64 sm[];
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_encrypt(DevView V, const
     const u64* sr = s_ntt + (size_t)p * N;
     // a, its transform times s left in place, and back: every thread's last
     // elements of the first transform are its first of the second
-    ntt_fwd_gg(
+    ntt_fwd_gg<PM>(
         poly,
         [&](int i) {
           const u64 a = sample_mod(key_a, i, pq);
@@ -240,7 +242,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_encrypt(DevView V, const
           return a;
         },
         [&](int i, u64 v) { poly[nsw(i)] = mulmod(v, sr[i], pq); }, V, p);
-    ntt_inv_gg(
+    ntt_inv_gg<PM>(
         poly, [&](int i) { return poly[nsw(i)]; },
         [&](int i, u64 v) {
           const u64 e = smod_dev(sample_cbd21(key_e, i), pq.q);
@@ -467,7 +469,8 @@ void launch_ptgen(const DevView& V, const uint16_t* pos, int L, int ell, int h, 
   if (L <= 0) return;
   const int JC = ptgen_jc(V.N);
   dim3 grid((ell + JC - 1) / JC, L);
-  k_ptgen<<<grid, chain_threads(V.N), ptgen_smem(V.N), st>>>(V, pos, ell, h, JC, P);
+  auto go = [&](auto kernel) { kernel<<<grid, chain_threads(V.N), ptgen_smem(V.N), st>>>(V, pos, ell, h, JC, P); };
+  V.allpm ? go(k_ptgen<true>) : go(k_ptgen<false>);
 }
 
 void launch_valgen(const DevView& V, const u32* vals, int L, u64* VP, cudaStream_t st) {
@@ -478,7 +481,10 @@ void launch_valgen(const DevView& V, const u32* vals, int L, u64* VP, cudaStream
 void launch_encrypt(const DevView& V, const uint16_t* pos, int ell, int h, const u64* s_ntt, u64 seed, u64 idx0,
                     u64* cts, cudaStream_t st) {
   if (ell <= 0) return;
-  k_encrypt<<<ell, chain_threads(V.N), (size_t)V.N * 12, st>>>(V, pos, h, s_ntt, seed, idx0, cts);
+  auto go = [&](auto kernel) {
+    kernel<<<ell, chain_threads(V.N), (size_t)V.N * 12, st>>>(V, pos, h, s_ntt, seed, idx0, cts);
+  };
+  V.allpm ? go(k_encrypt<true>) : go(k_encrypt<false>);
 }
 
 void launch_keygen(const DevView& V, u64 seed, int8_t* s, u64* s_ntt, u64* rlk, cudaStream_t st) {
@@ -512,6 +518,7 @@ cudaError_t client_init(int N) {
   if (e != cudaSuccess) return e;
   // largest request: the plaintext generator at this N
   if ((size_t)optin < ptgen_smem(N) || (size_t)optin < (size_t)N * 12) return cudaErrorInvalidValue;
-  return allow_smem({(const void*)k_ptgen, (const void*)k_valgen, (const void*)k_encrypt, (const void*)k_keygen_sntt,
+  return allow_smem({(const void*)k_ptgen<true>, (const void*)k_ptgen<false>, (const void*)k_valgen,
+                     (const void*)k_encrypt<true>, (const void*)k_encrypt<false>, (const void*)k_keygen_sntt,
                      (const void*)k_keygen_rlk, (const void*)k_dec_z, (const void*)k_dec_slots, (const void*)k_mask});
 }

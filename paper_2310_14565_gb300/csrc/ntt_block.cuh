@@ -510,23 +510,31 @@ __device__ __forceinline__ void ntt_inv_with(typename A::T* a, const Load& ld, c
   ntt_inv_block(a, N, logN, ar, itw, ninv);
   for (int x = threadIdx.x; x < N; x += blockDim.x) st(x, a[nsw(x)]);
 }
-template <class Load, class Store>
+// PM: every prime the kernel meets has folding products (DevView::allpm).  The
+// kernels come in both forms: with the other arithmetics compiled in beside it,
+// the compiler moved so much out of the branches that the inverse kernels spilled
+// (k_tensor_intt 788 bytes).
+template <bool PM = false, class Load, class Store>
 __device__ __forceinline__ void ntt_fwd_gg(u64* a, const Load& ld, const Store& st, const DevView& V, int pi) {
   const ulonglong2* tw = V.twp + (size_t)pi * V.N;
   const DevPrime P = V.pr[pi];
-  if (P.pm)
+  if constexpr (PM)
+    ntt_fwd_with(a, ld, st, nttd::Pm(P), V.N, V.logN, tw);
+  else if (P.pm)
     ntt_fwd_with(a, ld, st, nttd::Pm(P), V.N, V.logN, tw);
   else if (P.q < (1ull << 59))
     ntt_fwd_with(a, ld, st, nttd::Shoup<true>(P), V.N, V.logN, tw);
   else
     ntt_fwd_with(a, ld, st, nttd::Shoup<false>(P), V.N, V.logN, tw);
 }
-template <class Load, class Store>
+template <bool PM = false, class Load, class Store>
 __device__ __forceinline__ void ntt_inv_gg(u64* a, const Load& ld, const Store& st, const DevView& V, int pi) {
   const ulonglong2* itw = V.itwp + (size_t)pi * V.N;
   const DevPrime P = V.pr[pi];
   const ulonglong2 ninv = make_ulonglong2(P.ninv, P.ninvs);
-  if (P.pm)
+  if constexpr (PM)
+    ntt_inv_with(a, ld, st, nttd::Pm(P), V.N, V.logN, itw, ninv);
+  else if (P.pm)
     ntt_inv_with(a, ld, st, nttd::Pm(P), V.N, V.logN, itw, ninv);
   else
     ntt_inv_with(a, ld, st, nttd::Shoup<false>(P), V.N, V.logN, itw, ninv);

@@ -1164,6 +1164,8 @@ int pepsi_setup(const pepsi_params* params, uint64_t key_seed, pepsi_ctx** out) 
   c->V.kb = c->kb;
   c->V.tidx = c->k + c->kb;
   c->V.pr = c->d_pr;
+  c->V.allpm = 1;
+  for (int i = 0; i < c->k + c->kb; ++i) c->V.allpm &= (int)pr[i].pm;
   c->V.twp = c->d_twp;
   c->V.itwp = c->d_itwp;
   c->V.rc = c->d_rc;

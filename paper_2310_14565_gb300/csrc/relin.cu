@@ -15,7 +15,7 @@ constexpr int relin_min_blocks(int MT) { return MT <= 256 ? 3 : 1; }
 // Phase 1, block per row of DG[L][k+2][k][N]: row (l, i, j) holds
 // NTT_{q_j}([d2]_{q_i}) for digits i < k, and NTT_{q_j}(d0), NTT_{q_j}(d1)
 // for i = k, k+1.
-template <int MT>
+template <int MT, bool PM>
 __global__ void __launch_bounds__(MT, relin_min_blocks(MT)) k_relin_ntt(DevView V, const u64* __restrict__ D, u64* __restrict__ DG) {
   extern __shared__ u64 sm[];
   const int N = V.N, k = V.k;
@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(MT, relin_min_blocks(MT)) k_relin_ntt(DevView 
   const DevPrime pj = V.pr[j];
   const u64* row = i < k ? D + ((l * 3 + 2) * k + i) * N : D + ((l * 3 + (i - k)) * k + j) * N;
   u64* out = DG + r * N;
-  ntt_fwd_gg(
+  ntt_fwd_gg<PM>(
       sm,
       [&](int x) {
         const u64 w = row[x];
@@ -64,7 +64,7 @@ __global__ void k_relin_mac(DevView V, const u64* __restrict__ DG, const u64* __
 // and u = R_c + z * H on the load of the inverse NTT of U, stores u and the
 // coefficient-form row.  The same words as k_relin_mac followed by
 // k_axpy_intt, without R in memory.
-template <int MT>
+template <int MT, bool PM>
 __global__ void __launch_bounds__(MT, relin_min_blocks(MT))
     k_relin_axpy_intt(DevView V, const u64* __restrict__ DG, const u64* __restrict__ rlk,
                       const u64* __restrict__ zres, const u64* __restrict__ H, u64* __restrict__ out, u64* coef) {
@@ -76,17 +76,26 @@ __global__ void __launch_bounds__(MT, relin_min_blocks(MT))
   const size_t l = r / ((size_t)2 * k);
   const DevPrime pr = V.pr[p];
   const u64 z = zres[p];
+  const u64 zc = PM ? mulmod(z, 1ull << pr.s, pr) : 0;  // companion of z
   const size_t gs = (size_t)k * N;  // digit row stride
   const u64* g = DG + l * (k + 2) * gs + (size_t)p * N;
   const u64* key = rlk + ((size_t)c * k + p) * N;  // rlk_i[c] at prime p: key + i * 2 * gs
   const u64* hr = H + r * N;
   u64* ur = out + r * N;
-  ntt_inv_gg(
+  ntt_inv_gg<PM>(
       sm,
       [&](int x) {
         u64 lo = g[(size_t)(k + c) * gs + x], hi = 0;
         for (int i = 0; i < k; ++i) mac128(lo, hi, g[(size_t)i * gs + x], __ldg(key + (size_t)i * 2 * gs + x));
-        const u64 u = addmod(reduce128(hi, lo, pr), mulmod(z, hr[x], pr), pr.q);
+        u64 u;
+        if constexpr (PM) {  // z h below 2 q joins the sum before its reduction
+          const u64 zh = PmMul(pr).mul(hr[x], z, zc);
+          lo += zh;
+          hi += lo < zh;
+          u = pm_reduce(hi, lo, PmMul(pr), (int)pr.nbits);
+        } else {
+          u = addmod(reduce128(hi, lo, pr), mulmod(z, hr[x], pr), pr.q);
+        }
         ur[x] = u;
         return u;
       },
@@ -99,10 +108,11 @@ void launch_relin_digits(const DevView& V, const u64* D, u64* DG, int L, cudaStr
   if (L <= 0) return;
   const size_t rows = (size_t)L * (V.k + 2) * V.k;
   const int nt = xform_threads(V, rows);
+  auto go = [&](auto kernel) { kernel<<<(unsigned)rows, nt, (size_t)V.N * 8, st>>>(V, D, DG); };
   if (nt <= 256)
-    k_relin_ntt<256><<<(unsigned)rows, nt, (size_t)V.N * 8, st>>>(V, D, DG);
+    V.allpm ? go(k_relin_ntt<256, true>) : go(k_relin_ntt<256, false>);
   else
-    k_relin_ntt<NTT_MAX_THREADS><<<(unsigned)rows, nt, (size_t)V.N * 8, st>>>(V, D, DG);
+    V.allpm ? go(k_relin_ntt<NTT_MAX_THREADS, true>) : go(k_relin_ntt<NTT_MAX_THREADS, false>);
 }
 
 void launch_relin(const DevView& V, const u64* D, const u64* rlk, u64* DG, u64* R, int L, cudaStream_t st) {
@@ -116,13 +126,19 @@ void launch_relin_axpy_intt(const DevView& V, const u64* DG, const u64* rlk, con
   const size_t rows = (size_t)L * 2 * V.k;
   if (!rows) return;
   const int nt = xform_threads(V, rows);
+  auto go = [&](auto kernel) {
+    kernel<<<(unsigned)rows, nt, (size_t)V.N * 8, st>>>(V, DG, rlk, zres, H, out, coef);
+  };
   if (nt <= 256)
-    k_relin_axpy_intt<256><<<(unsigned)rows, nt, (size_t)V.N * 8, st>>>(V, DG, rlk, zres, H, out, coef);
+    V.allpm ? go(k_relin_axpy_intt<256, true>) : go(k_relin_axpy_intt<256, false>);
   else
-    k_relin_axpy_intt<NTT_MAX_THREADS><<<(unsigned)rows, nt, (size_t)V.N * 8, st>>>(V, DG, rlk, zres, H, out, coef);
+    V.allpm ? go(k_relin_axpy_intt<NTT_MAX_THREADS, true>) : go(k_relin_axpy_intt<NTT_MAX_THREADS, false>);
 }
 
 cudaError_t relin_init() {
-  return allow_smem({(const void*)k_relin_ntt<256>, (const void*)k_relin_ntt<NTT_MAX_THREADS>,
-                     (const void*)k_relin_axpy_intt<256>, (const void*)k_relin_axpy_intt<NTT_MAX_THREADS>});
+  return allow_smem({(const void*)k_relin_ntt<256, true>, (const void*)k_relin_ntt<NTT_MAX_THREADS, true>,
+                     (const void*)k_relin_axpy_intt<256, true>, (const void*)k_relin_axpy_intt<NTT_MAX_THREADS, true>,
+                     (const void*)k_relin_ntt<256, false>, (const void*)k_relin_ntt<NTT_MAX_THREADS, false>,
+                     (const void*)k_relin_axpy_intt<256, false>,
+                     (const void*)k_relin_axpy_intt<NTT_MAX_THREADS, false>});
 }

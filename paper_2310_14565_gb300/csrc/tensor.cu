@@ -5,12 +5,29 @@
 
 namespace {
 
+// a b mod q and a 128-bit sum mod q in the arithmetic of the kernel's primes
+template <bool PM>
+__device__ __forceinline__ u64 reduce_sum(u64 hi, u64 lo, const DevPrime& p) {
+  if constexpr (PM)
+    return pm_reduce(hi, lo, PmMul(p), (int)p.nbits);
+  else
+    return reduce128(hi, lo, p);
+}
+template <bool PM>
+__device__ __forceinline__ u64 prod(u64 a, u64 b, const DevPrime& p) {
+  if constexpr (PM)
+    return pm_reduce(__umul64hi(a, b), a * b, PmMul(p), (int)p.nbits);
+  else
+    return mulmod(a, b, p);
+}
+
 // ------------------------------------------------------------ tensor
 // Tensor product fused with its inverse transform: block per row
 // (l, c, pi) of T3[L][3][k+kb][N] computes component c of the tensor of
 // (A_l, B_l) at prime pi on the load of the inverse NTT, and stores the
 // coefficient-form row: the tensor (a0b0, a0b1 + a1b0, a1b1) and its
 // inverse NTT without a round trip of the NTT-form tensor through memory.
+template <bool PM>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1)
     k_tensor_intt(DevView V, const u64* __restrict__ AQ, const u64* __restrict__ AB, const u64* __restrict__ BQ,
                   const u64* __restrict__ BB, const u64* __restrict__ cstQ, const u64* __restrict__ side,
@@ -46,32 +63,32 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1)
   const RowSt st(T3 + r * N);
   if (square) {
     if (c == 0)
-      ntt_inv_gg(sm, [&](int x) { return mulmod(a0[x], a0[x], pr); }, st, V, pi);
+      ntt_inv_gg<PM>(sm, [&](int x) { return prod<PM>(a0[x], a0[x], pr); }, st, V, pi);
     else if (c == 1)
-      ntt_inv_gg(
+      ntt_inv_gg<PM>(
           sm,
           [&](int x) {
-            const u64 m = mulmod(a0[x], a1[x], pr);
+            const u64 m = prod<PM>(a0[x], a1[x], pr);
             return addmod(m, m, pr.q);
           },
           st, V, pi);
     else
-      ntt_inv_gg(sm, [&](int x) { return mulmod(a1[x], a1[x], pr); }, st, V, pi);
+      ntt_inv_gg<PM>(sm, [&](int x) { return prod<PM>(a1[x], a1[x], pr); }, st, V, pi);
   } else {
     if (c == 0)
-      ntt_inv_gg(sm, [&](int x) { return mulmod(a0[x], addmod(b0[x], cb, pr.q), pr); }, st, V, pi);
+      ntt_inv_gg<PM>(sm, [&](int x) { return prod<PM>(a0[x], addmod(b0[x], cb, pr.q), pr); }, st, V, pi);
     else if (c == 1)
-      ntt_inv_gg(
+      ntt_inv_gg<PM>(
           sm,
           [&](int x) {
             u64 lo = 0, hi = 0;
             mac128(lo, hi, a0[x], b1[x]);
             mac128(lo, hi, a1[x], addmod(b0[x], cb, pr.q));
-            return reduce128(hi, lo, pr);
+            return reduce_sum<PM>(hi, lo, pr);
           },
           st, V, pi);
     else
-      ntt_inv_gg(sm, [&](int x) { return mulmod(a1[x], b1[x], pr); }, st, V, pi);
+      ntt_inv_gg<PM>(sm, [&](int x) { return prod<PM>(a1[x], b1[x], pr); }, st, V, pi);
   }
 }
 
@@ -169,8 +186,11 @@ void launch_tensor_intt(const DevView& V, const u64* AQ, const u64* AB, const u6
                         const u64* cstQ, const u64* side, u64* T3, int L, bool square, cudaStream_t st) {
   const size_t rows = (size_t)L * 3 * (V.k + V.kb);
   if (!rows) return;
-  k_tensor_intt<<<(unsigned)rows, xform_threads(V, rows), (size_t)V.N * 8, st>>>(V, AQ, AB, BQ, BB, cstQ, side, T3,
+  auto go = [&](auto kernel) {
+    kernel<<<(unsigned)rows, xform_threads(V, rows), (size_t)V.N * 8, st>>>(V, AQ, AB, BQ, BB, cstQ, side, T3,
                                                                           square ? 1 : 0);
+  };
+  V.allpm ? go(k_tensor_intt<true>) : go(k_tensor_intt<false>);
 }
 
 void launch_tensor_sum(const DevView& V, const u64* AQ, const u64* AB, const u64* BQ, const u64* BB,
@@ -181,4 +201,4 @@ void launch_tensor_sum(const DevView& V, const u64* AQ, const u64* AB, const u64
                                                                           square ? 1 : 0, init ? 1 : 0);
 }
 
-cudaError_t tensor_init() { return allow_smem({(const void*)k_tensor_intt}); }
+cudaError_t tensor_init() { return allow_smem({(const void*)k_tensor_intt<true>, (const void*)k_tensor_intt<false>}); }

@@ -8,7 +8,7 @@ namespace {
 // ------------------------------------------------------------------ NTT
 // SPLIT: store the result in the split operand format of the
 // multiply-accumulate (the request's forward transform).
-template <bool FWD, bool SPLIT = false>
+template <bool PM, bool FWD, bool SPLIT = false>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ntt(DevView V, const u64* __restrict__ src, u64* dst, int np, int p0, size_t src_os,
                       size_t dst_os, u32* sums) {
   extern __shared__ u64 sm[];
@@ -21,11 +21,11 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ntt(DevView V, const u64
   const RowLd ld(s);
   if (FWD) {
     if (SPLIT)
-      ntt_fwd_gg(sm, ld, SplitSumSt(d, sums + o * dst_os + (size_t)pl * N, V.pr[p0 + pl].split), V, p0 + pl);
+      ntt_fwd_gg<PM>(sm, ld, SplitSumSt(d, sums + o * dst_os + (size_t)pl * N, V.pr[p0 + pl].split), V, p0 + pl);
     else
-      ntt_fwd_gg(sm, ld, RowSt(d), V, p0 + pl);
+      ntt_fwd_gg<PM>(sm, ld, RowSt(d), V, p0 + pl);
   } else {
-    ntt_inv_gg(sm, ld, RowSt(d), V, p0 + pl);
+    ntt_inv_gg<PM>(sm, ld, RowSt(d), V, p0 + pl);
   }
 }
 
@@ -34,6 +34,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ntt(DevView V, const u64
 // row on the transform's load and also stores it (each element is loaded
 // once).  coef may alias b: a block reads its row of b before it writes
 // that row of coef.
+template <bool PM>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1)
     k_axpy_intt(DevView V, const u64* __restrict__ a, const u64* __restrict__ zres, const u64* b, u64* __restrict__ out,
                 u64* coef) {
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1)
   const u64* br = b + r * N;
   u64* ur = out + r * N;
   u64* cr = coef + r * N;
-  ntt_inv_gg(
+  ntt_inv_gg<PM>(
       sm,
       [&](int x) {
         const u64 u = addmod(ar[x], mulmod(z, br[x], pr), pr.q);
@@ -63,23 +64,31 @@ void launch_ntt(const DevView& V, bool fwd, const u64* src, u64* dst, size_t out
                 size_t dst_os, cudaStream_t st, bool split_out, u32* sums) {
   const size_t rows = outer * (size_t)np;
   if (!rows) return;
-  const size_t smem = (size_t)V.N * sizeof(u64);
+  auto go = [&](auto kernel) {
+    kernel<<<(unsigned)rows, xform_threads(V, rows), (size_t)V.N * sizeof(u64), st>>>(V, src, dst, np, p0, src_os, dst_os,
+                                                                                    sums);
+  };
   if (fwd && split_out)
-    k_ntt<true, true><<<(unsigned)rows, xform_threads(V, rows), smem, st>>>(V, src, dst, np, p0, src_os, dst_os, sums);
+    V.allpm ? go(k_ntt<true, true, true>) : go(k_ntt<false, true, true>);
   else if (fwd)
-    k_ntt<true><<<(unsigned)rows, xform_threads(V, rows), smem, st>>>(V, src, dst, np, p0, src_os, dst_os, nullptr);
+    V.allpm ? go(k_ntt<true, true>) : go(k_ntt<false, true>);
   else
-    k_ntt<false><<<(unsigned)rows, xform_threads(V, rows), smem, st>>>(V, src, dst, np, p0, src_os, dst_os, nullptr);
+    V.allpm ? go(k_ntt<true, false>) : go(k_ntt<false, false>);
 }
 
 void launch_axpy_intt(const DevView& V, const u64* a, const u64* zres, const u64* b, u64* out, u64* coef,
                       size_t groups, cudaStream_t st) {
   const size_t rows = groups * V.k;
   if (!rows) return;
-  k_axpy_intt<<<(unsigned)rows, xform_threads(V, rows), (size_t)V.N * 8, st>>>(V, a, zres, b, out, coef);
+  auto go = [&](auto kernel) {
+    kernel<<<(unsigned)rows, xform_threads(V, rows), (size_t)V.N * 8, st>>>(V, a, zres, b, out, coef);
+  };
+  V.allpm ? go(k_axpy_intt<true>) : go(k_axpy_intt<false>);
 }
 
 cudaError_t transforms_init() {
-  return allow_smem({(const void*)k_ntt<true>, (const void*)k_ntt<false>, (const void*)k_ntt<true, true>,
-                     (const void*)k_axpy_intt});
+  return allow_smem({(const void*)k_ntt<true, true>, (const void*)k_ntt<true, false>,
+                     (const void*)k_ntt<true, true, true>, (const void*)k_ntt<false, true>,
+                     (const void*)k_ntt<false, false>, (const void*)k_ntt<false, true, true>,
+                     (const void*)k_axpy_intt<true>, (const void*)k_axpy_intt<false>});
 }
