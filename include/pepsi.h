@@ -111,9 +111,9 @@ typedef struct {
                               PEPSI_E_PARAM).  The storage is the same for all of them: byte
                               planes of ceil(bits(q_i) / 8) bytes per word (at least 4; 7 for
                               55-bit primes) with the code bits padded to a multiple of 16,
-                              or 64-bit words for codes so short that the padding would make
-                              the planes more than an eighth larger than words.  Results do
-                              not depend on it */
+                              or 64-bit words for codes so short (below about 80 bits with 7
+                              bytes, 43 with 5) that planes would be slower.  Results do not
+                              depend on it */
   uint32_t gamma;          /* client maximum bin load (Table 2, Section 4): 0 or 1 = cuckoo
                               hashing with one item per bin (the paper's evaluation); 2..16 =
                               bins of gamma slots, so up to gamma * b client items.  The client

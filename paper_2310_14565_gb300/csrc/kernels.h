@@ -51,13 +51,17 @@ struct PlaneTab {
 };
 inline int plane_steps(int ell) { return (ell + 15) / 16; }
 inline size_t plane_layer_bytes(int ell, size_t kN, int npl) { return (size_t)plane_steps(ell) * kN * 16 * npl; }
-// Whether a resident table is kept in byte planes, else as 64-bit words: the
-// planes' steps of 16 bits make a short code's table larger (24 bits in 7 planes:
-// 224 bytes per point and layer against 192), and its few bits do not pay for
-// the sums and reductions of an item.  The line allows planes an eighth more
-// bytes.  At 24 bits, 526 layers, N = 8192, k = 4
-// the multiply-accumulate took 1.22 ms on planes and 0.77 ms on words.
-inline bool table_in_planes(int ell, int npl) { return 8 * (size_t)plane_steps(ell) * 16 * npl <= 9 * (size_t)ell * 8; }
+// Whether a resident table is kept in byte planes, else as 64-bit words: short
+// codes do not pay for the padding to steps of 16 bits and for the sums and
+// reductions of an item (a point and 16 layers), about the time of 16 bits.
+// Multiply-accumulate of 512 layers, planes against words: 7 planes, N = 8192, k = 4:
+// 32 bits 1.17 and 0.87 ms, 48 bits 1.30 and 1.15, 64 bits 1.39 and 1.43, 80 bits
+// 1.69 and 1.72, 96 bits 1.78 and 2.01, 128 bits 2.41 and 2.66; 5 planes, N = 4096,
+// k = 3: 32 bits 0.375 and 0.337, 48 bits 0.41 and 0.45, 128 bits 0.64 and 1.00.
+// Four requests and 128 layers cross at the same lengths (48 bits 1.25 and 1.04, 80
+// bits 1.53 and 1.59 ms; 5 planes: 32 bits 0.35 and 0.30, 48 bits 0.39 and 0.41).
+// Beyond, planes may take an eighth more bytes (8 planes): several requests gain.
+inline bool table_in_planes(int ell, int npl) { return plane_steps(ell) * 16 * npl <= 9 * (ell - 16); }
 // 64-bit words of a request in byte planes
 inline size_t request_plane_words(int ell, size_t kN) { return (size_t)plane_steps(ell) * kN * 32; }
 // H[q][l][c][p][n] = sum_j C[q][j][c][p][n] * P[l0 + l][j][p][n] mod q_p for nl layers of the table

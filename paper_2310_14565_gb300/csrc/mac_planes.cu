@@ -43,8 +43,11 @@ __host__ __device__ constexpr int threads(bool brief) { return (consumers(brief)
 // only disorders the DRAM (10.4 ms at the paper shape; three stages 11.4, stages
 // of 3, 5 or 6 steps 10.9, 10.5, 10.9).  Several requests are bound by the consumer
 // warps, which longer stages free of waits (four requests, 48 layers: 2.76, 2.60,
-// 2.46 ms at 4, 6, 8 steps).
-constexpr int KS_SHORT = 2, KS_ONE = 4, KS_MANY = 8;
+// 2.46 ms at 4, 6, 8 steps).  Codes of at most 128 bits: a stage costs its producer
+// warp, which serves three teams, about as much as two steps cost a consumer, so
+// stages of 4 steps as well (512 layers of 128 bits at N = 8192, 7 planes: 2.41 ms,
+// 2.88 with stages of 2; N = 4096, 5 planes: 0.64, 1.05).
+constexpr int KS_ONE = 4, KS_MANY = 8;
 constexpr int MAX_STAGES = 16;
 constexpr int DRAIN = 8;           // steps between moves to the integer sums: 128 code bits
 constexpr u32 BIAS = 0x33000000u;  // 2^23 in units of 2^-48, as f32
@@ -525,8 +528,8 @@ template <int NPL>
 cudaError_t init_npl() {
   using namespace macp;
   cudaError_t e = cudaSuccess;
-  for (const void* f : {(const void*)k_mac_planes<NPL, KS_ONE, false>, (const void*)k_mac_planes<NPL, KS_SHORT, true>,
-                        (const void*)k_mac_planes<NPL, KS_MANY, false>, (const void*)k_mac_planes<NPL, KS_ONE, true>})
+  for (const void* f : {(const void*)k_mac_planes<NPL, KS_ONE, false>, (const void*)k_mac_planes<NPL, KS_ONE, true>,
+                        (const void*)k_mac_planes<NPL, KS_MANY, false>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute((const void*)k_pack_planes<NPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -580,9 +583,8 @@ void launch_mac_planes(const DevView& V, int nq, const u32* const* C, const Plan
     A.C[q] = C[std::min(q, nq - 1)];
     A.H[q] = H[std::min(q, nq - 1)];
   }
-  // short codes: stages of 2 steps (one request) hold whole items of the shortest codes
   const bool brief = ks1 - ks0 <= DRAIN;
-  const int ks = nq > 1 ? (brief ? KS_ONE : KS_MANY) : brief ? KS_SHORT : KS_ONE;
+  const int ks = nq > 1 && !brief ? KS_MANY : KS_ONE;
   const int teams = consumers(brief) / nq, sb = stage_bytes(P.npl, ks, nq);
   const int room = nq == 1 ? 160 * 1024 : SMEM_BUDGET - teams * 2 * MAX_STAGES * 8;
   A.nst = std::max(2, std::min(MAX_STAGES, room / (teams * sb)));
@@ -590,12 +592,10 @@ void launch_mac_planes(const DevView& V, int nq, const u32* const* C, const Plan
   const u32 ntile = ((u32)(l0 + nl + 15) >> 4) - ((u32)l0 >> 4);
   const size_t items = (size_t)V.k * V.N * ntile;
   const unsigned grid = (unsigned)std::min<size_t>((size_t)sm_count(), (items + teams - 1) / teams);
-  const int kind = (nq == 1 ? 0 : 2) + (brief ? 1 : 0);
 #define GO(n)                                                                                            \
-  if (kind == 0) k_mac_planes<n, KS_ONE, false><<<grid, threads(false), smem, st>>>(V, A);               \
-  else if (kind == 1) k_mac_planes<n, KS_SHORT, true><<<grid, threads(true), smem, st>>>(V, A);          \
-  else if (kind == 2) k_mac_planes<n, KS_MANY, false><<<grid, threads(false), smem, st>>>(V, A);         \
-  else k_mac_planes<n, KS_ONE, true><<<grid, threads(true), smem, st>>>(V, A)
+  if (brief) k_mac_planes<n, KS_ONE, true><<<grid, threads(true), smem, st>>>(V, A);                     \
+  else if (nq > 1) k_mac_planes<n, KS_MANY, false><<<grid, threads(false), smem, st>>>(V, A);            \
+  else k_mac_planes<n, KS_ONE, false><<<grid, threads(false), smem, st>>>(V, A)
   PEPSI_NPL_DISPATCH(P.npl, GO)
 #undef GO
 }

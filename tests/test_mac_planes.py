@@ -26,13 +26,19 @@ def test_byte_products_are_exact_in_f32_from_the_bias():
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("bits,ell,mu", [
-    ([30, 31], 16, 17),        # 4 planes, one step, one layer beyond a tile
-    ([36, 36, 37], 17, 16),    # a table kept in words (planes would be larger)
-    ([36, 36, 37], 32, 16),    # 5 planes, one whole tile
+    ([30, 31], 16, 17),        # tables kept in words
+    ([36, 36, 37], 17, 16),
+    ([36, 36, 37], 32, 16),
+    ([30, 31], 32, 17),        # 4 planes, two steps, one layer beyond a tile
+    ([36, 36, 37], 42, 16),    # the last length of 5 planes in words and the first in planes
+    ([36, 36, 37], 43, 33),
+    ([55, 54], 79, 16),        # the same with 7 planes
+    ([55, 54], 80, 17),
     ([45, 46], 129, 15),       # 6 planes, one bit beyond the run of 128
     ([55, 54], 128, 33),       # 7 planes, whole runs
     ([55, 54], 300, 18),
-    ([60, 60], 127, 16),       # 8 planes
+    ([60, 60], 127, 16),       # words
+    ([58, 57], 144, 16),       # 8 planes
     ([59], 257, 9),
 ])
 def test_planes_match_the_oracle(bits, ell, mu):
