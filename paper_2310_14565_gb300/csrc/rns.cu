@@ -5,12 +5,50 @@
 
 namespace {
 
+// side[layer][j]: the lift of (x + cst) mod Q less the lift of x, mod p_j, at
+// coefficient 0 of component 0.
 template <int K, int KB, bool PM>
-__global__ void k_lift(const __grid_constant__ RnsArgs A, const u64* __restrict__ src, u64* __restrict__ dstB,
-                       int L) {
+__device__ __forceinline__ void lift_side(const RnsArgs& A, const u64* __restrict__ src, int layer,
+                                          const u64* __restrict__ cst, u64* side) {
+  constexpr int MQ = K ? K : PEPSI_MAXQ;
+  const int N = A.N, k = K ? K : A.k, kb = KB ? KB : A.kb;
+#pragma unroll 1
+  for (int plain = 0; plain < 2; ++plain) {
+    u64 x[MQ], v[MQ];
+#pragma unroll
+    for (int i = 0; i < MQ; ++i)
+      if (K || i < k) {
+        x[i] = src[((size_t)layer * 2 * k + i) * N];
+        if (!plain) x[i] = addmod(x[i], cst[i], A.pr[i].q);
+      }
+    garner_q<K, PM>(A, x, v);
+    const bool neg = digits_greater<MQ>(v, A.rc.qhalf_dig, k);
+#pragma unroll 1
+    for (int j = 0; j < kb; ++j) {
+      const u64 w = q_digits_mod_b<K, PM>(A, v, neg, j);
+      u64& s = side[(size_t)layer * kb + j];
+      s = plain ? submod(s, w, A.pr[k + j].q) : w;
+    }
+  }
+}
+// Q -> B extension, thread per coefficient; the first `ns` blocks, a thread per
+// layer, make side[] beside the others (in a launch of its own it cost small
+// evaluations 4 to 10 us a lift; in every thread of coefficient 0 its second set of
+// digits cost registers, 232 at k = kb = 8).  The run-time generic form keeps ns = 0
+// and k_lift_side: with both loops it took 200 registers instead of 34.
+template <int K, int KB, bool PM>
+__global__ void __launch_bounds__(128, K == 0 ? 1 : K < 8 ? 16 : 12) k_lift(const __grid_constant__ RnsArgs A, const u64* __restrict__ src, u64* __restrict__ dstB,
+                       int L, u32 ns, const u64* __restrict__ cst, u64* side) {
+  if constexpr (K > 0) {
+    if (blockIdx.x < ns) {
+      const int layer = blockIdx.x * blockDim.x + threadIdx.x;
+      if (layer < L) lift_side<K, KB, PM>(A, src, layer, cst, side);
+      return;
+    }
+  }
   constexpr int MQ = K ? K : PEPSI_MAXQ, MB = KB ? KB : PEPSI_MAXB;
   const int N = A.N, k = K ? K : A.k, kb = KB ? KB : A.kb;
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // over L*2*N
+  const size_t idx = (size_t)(blockIdx.x - ns) * blockDim.x + threadIdx.x;  // over L*2*N
   if (idx >= (size_t)L * 2 * N) return;
   const int n = (int)(idx % N);
   const size_t lc = idx / N;  // layer*2 + comp
@@ -24,28 +62,19 @@ __global__ void k_lift(const __grid_constant__ RnsArgs A, const u64* __restrict_
   for (int j = 0; j < MB; ++j)
     if (KB || j < kb) dstB[(lc * kb + j) * N + n] = q_digits_mod_b<K, PM>(A, v, neg, j);
 }
-// side[layer][j]: the lift of (x + cst) mod Q less the lift of x, mod p_j, at
-// coefficient 0 of component 0 (a kernel of its own: inside k_lift its second
-// set of digits cost registers, 232 at k = kb = 8).
-template <int K, int KB, bool PM>
-__global__ void k_lift_side(const __grid_constant__ RnsArgs A, const u64* __restrict__ src,
-                            const u64* __restrict__ dstB, int L, const u64* __restrict__ cst, u64* __restrict__ side) {
-  constexpr int MQ = K ? K : PEPSI_MAXQ;
-  const int N = A.N, k = K ? K : A.k, kb = KB ? KB : A.kb;
+
+template <bool PM>
+__global__ void k_lift_side(const __grid_constant__ RnsArgs A, const u64* __restrict__ src, int L,
+                            const u64* __restrict__ cst, u64* side) {
   const int layer = blockIdx.x * blockDim.x + threadIdx.x;
-  if (layer >= L) return;
-  u64 x[MQ], v[MQ];
-#pragma unroll
-  for (int i = 0; i < MQ; ++i)
-    if (K || i < k) x[i] = addmod(src[((size_t)layer * 2 * k + i) * N], cst[i], A.pr[i].q);
-  garner_q<K, PM>(A, x, v);
-  const bool neg = digits_greater<MQ>(v, A.rc.qhalf_dig, k);
-  for (int j = 0; j < kb; ++j)
-    side[(size_t)layer * kb + j] =
-        submod(q_digits_mod_b<K, PM>(A, v, neg, j), dstB[((size_t)layer * 2 * kb + j) * N], A.pr[k + j].q);
+  if (layer < L) lift_side<0, 0, PM>(A, src, layer, cst, side);
 }
 
 // ------------------------------------------------------ scale and round
+// Bound by the heavy multiply-add pipe (k_lift too): a thread per coefficient holds
+// its digits in registers, and with folding products the Garner and Horner steps
+// stay unreduced.  A paper-shaped evaluation's scale-and-round 1.07 -> 0.72 ms, lift
+// 0.61 -> 0.47 ms against Shoup and Barrett steps.
 // y = round(t x / Q) exactly: z = t x + (Q-1)/2, [z]_Q from the Q residues
 // by Garner, y = (z - [z]_Q) / Q computed in B, y centred in B and mapped
 // back to Q by Garner over B.
@@ -105,6 +134,7 @@ __global__ void k_scale_round(const __grid_constant__ RnsArgs A, const u64* __re
 #define PEPSI_RNS_COUNTS(V, LAUNCH, PM)               \
   switch ((V).k * 16 + (V).kb) {                      \
     case 3 * 16 + 3: LAUNCH(3, 3, PM); break;         \
+    case 3 * 16 + 4: LAUNCH(3, 4, PM); break;         \
     case 4 * 16 + 4: LAUNCH(4, 4, PM); break;         \
     case 4 * 16 + 5: LAUNCH(4, 5, PM); break;         \
     case 4 * 16 + 6: LAUNCH(4, 6, PM); break;         \
@@ -124,9 +154,9 @@ void launch_lift(const DevView& V, const u64* src, u64* dstB, int L, const u64* 
   if (!total) return;
 #define LIFT(KQ, KBB, PM)                                                                               \
   {                                                                                                     \
-    k_lift<KQ, KBB, PM><<<grid_for(total, 128), 128, 0, st>>>(*V.host_args, src, dstB, L);              \
-    if (cst)                                                                                            \
-      k_lift_side<KQ, KBB, PM><<<grid_for(L, 32), 32, 0, st>>>(*V.host_args, src, dstB, L, cst, side);  \
+    const unsigned ns = cst && KQ ? grid_for(L, 128) : 0;                                               \
+    k_lift<KQ, KBB, PM><<<ns + grid_for(total, 128), 128, 0, st>>>(*V.host_args, src, dstB, L, ns, cst, side); \
+    if (cst && !KQ) k_lift_side<PM><<<grid_for(L, 32), 32, 0, st>>>(*V.host_args, src, L, cst, side);    \
   }
   PEPSI_RNS_DISPATCH(V, LIFT)
 #undef LIFT
