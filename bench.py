@@ -407,7 +407,7 @@ LARGE_RESERVE_GB = 70
 def leg_large(pepsi, torch, steps=3, chunk=128, reserve_gb=None):
     """Configuration 4 (large) in the default line: N = 16384, eight primes,
     h = 8, ell = 128, mu = 3487, 4096 client x 2^24 server items; the
-    resident prefix of the 468 GB table in 7-byte words, the rest
+    resident prefix of the 468 GB table in byte planes (7 per word), the rest
     regenerated per chunk.  A few steps after one warm-up.  reserve_gb: HBM
     left free of resident plaintexts for the evaluation's scratch (None: the
     library's default budget, 0.6 of the free memory)."""
@@ -473,7 +473,7 @@ def leg_large(pepsi, torch, steps=3, chunk=128, reserve_gb=None):
     batch_ms = e0.elapsed_time(e1)
     same = all(torch.equal(bout[i], sout[i]) for i in range(4))
     res = {"workload": "N=16384, 8 primes (55x6, 54x2), h=8, ell=128, mu=3487, 4096 client x 2^24 server items, "
-                       "41 planted; 7-byte resident prefix, the rest regenerated per chunk",
+                       "41 planted; resident prefix in byte planes (7 per word), the rest regenerated per chunk",
            "ms_per_step": round(ms, 1), "steps": steps, "layer_chunk": chunk,
            "resident_layers": resident_layers, "resident_gb": round(resident_layers * layer_bytes / 1e9, 1),
            "batched": {"requests": 4, "ms_per_request": round(batch_ms / 4, 1),
@@ -515,7 +515,7 @@ def run_ours(args):
                         rescale_group=RESCALE["all"], response_primes=RESPONSE_PRIMES,
                         plaintext_bytes=args.plaintext_bytes or (7 if args.case == "large" else 8))
     ctx.set_rescale_group(RESCALE[args.rescale])
-    pbytes = ctx.plaintext_bytes
+    in_planes, pbytes, layer_bytes = table_form(WL["prime_bits"], WL["ell"], N)
     sets = make_sets(WL["m"], WL["n"], WL["planted"], bits=WL.get("bits", 64))
     t0 = time.perf_counter()
     sid = ctx.server_load(sets.server)
@@ -576,16 +576,16 @@ def run_ours(args):
     ctx.profile(False)
     mac_launches, mac_ms = prof["mac"]
     mac_launches_per_eval = mac_launches / psteps
-    # algorithmic bytes of the MAC per evaluation: the plaintext table (mu*ell*k*N words of
-    # pbytes = 7 or 8 bytes), the prepared request (ell*2*k*N words of 8 bytes and their
-    # 4-byte half sums, read once by each launch) and h' (mu*2*k*N words of 8 bytes)
+    # algorithmic bytes of the MAC per evaluation: the resident table, the prepared request
+    # (read once by each launch: its byte planes, 8 bytes per word of whole steps of 16 code
+    # bits, or the word kernel's 8-byte words and 4-byte half sums) and h' (mu*2*k*N words)
     mu, ell = WL["mu"], WL["ell"]
-    mac_bytes_eval = (pbytes * mu * ell * k * N + 12 * mac_launches_per_eval * ell * 2 * k * N +
-                      8 * mu * 2 * k * N)
+    request_bytes = 16 * ((ell + 15) // 16) * 2 * k * N * 8 if in_planes else 12 * ell * 2 * k * N
+    mac_bytes_eval = mu * layer_bytes + mac_launches_per_eval * request_bytes + 8 * mu * 2 * k * N
     mac_launch_ms = mac_ms / mac_launches
     achieved = mac_bytes_eval / mac_launches_per_eval / (mac_launch_ms * 1e-3) / 1e9
     peak, peak_kind = measured_peaks()
-    traffic = stored_traffic() if args.case == "paper" and pbytes == 8 else None
+    traffic = stored_traffic() if args.case == "paper" and in_planes else None
 
     # end to end through the C ABI with host buffers (pinned), copies inside the timed region
     for _ in range(2):
@@ -641,7 +641,7 @@ def run_ours(args):
                            "l2": ("inputs larger than L2 (plaintext chunks of %.1f GB)" % (chunk * 0.134)
                                   if args.case == "large" else
                                   "inputs larger than L2: the %.1f GB resident plaintext table is read every step"
-                                  % (WL["mu"] * WL["ell"] * k * N * pbytes / 1e9)),
+                                  % (WL["mu"] * layer_bytes / 1e9)),
                            "plaintext_bytes_per_word": pbytes},
                 "e2e": {"value": round(e2e_ms, 3), "unit": "ms", "h2d_bytes_per_step": int(cts_np.nbytes),
                         "d2h_bytes_per_step": int(out_pinned.numel() * 8)},
@@ -726,18 +726,20 @@ def run_ours(args):
     ntt_ms = e0.elapsed_time(e1) / 10
     ntt_gbs = 2 * 8 * N * k * count / (ntt_ms * 1e-3) / 1e9
 
-    # integer-pipe peaks (measured here, multipliers that change every step) and the
-    # MAC's use of the wide multiply-add: 2 components x 3 Karatsuba split products
-    # per plaintext word and request
+    # integer-pipe peaks (measured here, multipliers that change every step) and, where the
+    # table is in words, the MAC's use of the wide multiply-add: 2 components x 3 Karatsuba
+    # split products per plaintext word and request
     wide_peak = pepsi.int_peak(pepsi.INT_MAD_WIDE)
     mul_peak = pepsi.int_peak(pepsi.INT_MUL_WIDE)
     mad32_peak = pepsi.int_peak(pepsi.INT_MAD_LO)
-    mac_wide_rate = 6.0 * mu * ell * k * N / (mac_launch_ms * 1e-3)
+    mac_wide_rate = 6.0 * mu * ell * k * N / (mac_ms / psteps * 1e-3)
     bmac_ms = batched["kernel_ms_per_call"].get("mac", 0.0)
     bmac_rate = 6.0 * nbq * mu * ell * k * N / (bmac_ms * 1e-3) if bmac_ms else 0.0
+    # on byte planes: one m16n8k16 per plane, component, request, point, 16 layers and 16 bits
+    mma = 2 * pbytes * ((mu + 15) // 16) * ((ell + 15) // 16) * k * N
     # the circuit kernels' share of the heavy multiply-add pipe: busy SM-cycles per
     # evaluation (full-size ncu counters) over this run's CUDA-event time of the class
-    cyc = stored_pipe_cycles() if pbytes == 8 and args.rescale == "all" else None
+    cyc = stored_pipe_cycles() if in_planes and args.rescale == "all" else None
     circuits = None
     if cyc:
         clock_hz = (clk.get("sm_mhz") or 2070.0) * 1e6
@@ -750,11 +752,14 @@ def run_ours(args):
                 circuits[cls] = round(cyc[cls] / (per_eval_s * clock_hz * sms), 3)
     int_pipe = {"mad_wide_u32_per_s": round(wide_peak / 1e12, 3), "mul_wide_u32_per_s": round(mul_peak / 1e12, 3),
                 "mad_u32_per_s": round(mad32_peak / 1e12, 3), "unit": "T ops/s",
-                "mac_mad_wide_frac": round(mac_wide_rate / wide_peak, 4),
-                "batched_mac_mad_wide_frac": round(bmac_rate / wide_peak, 4),
+                "mac_mad_wide_frac": None if in_planes else round(mac_wide_rate / wide_peak, 4),
+                "batched_mac_mad_wide_frac": None if in_planes else round(bmac_rate / wide_peak, 4),
+                "mac_mma_tflops": round(4096 * mma / (mac_ms / psteps * 1e-3) / 1e12, 1) if in_planes else None,
+                "batched_mac_mma_tflops": (round(4096 * nbq * mma / (bmac_ms * 1e-3) / 1e12, 1)
+                                           if in_planes and bmac_ms else None),
                 "circuits_heavy_pipe_busy": circuits,
-                "note": "the MACs issue 6 mad.wide.u32 per plaintext word and request (2 components x 3 Karatsuba "
-                        "split products); peaks measured with multipliers that change every step; "
+                "note": "MAC on words: 6 mad.wide.u32 per plaintext word and request (2 components x 3 Karatsuba "
+                        "split products); MAC on byte planes: f16 mma.sync.m16n8k16 on exact byte products; peaks measured with multipliers that change every step; "
                         "circuits_heavy_pipe_busy: fraction of the SMs' heavy multiply-add pipe cycles each kernel "
                         "class keeps busy (profiles/circuit_pipes_paper.md counters / this run's event times)"}
 
@@ -762,8 +767,8 @@ def run_ours(args):
         "metric": METRIC, "value": round(ms, 3), "unit": "ms", "n_gpus": args.gpus, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(ms, 3), "higher_is_better": False, "scaling": "weak",
         "vs_baseline": None, "dtype": "u64", "data": "synthetic",
-        "config": {"workload": WORKLOAD_NAME, "l2": L2_NOTE % (mu * ell * k * N * pbytes / 1e9), "parallelism": "replicas" if ws > 1 else "1 GPU",
-                   "resident_plaintexts_gb": round(mu * ell * k * N * pbytes / 1e9, 1),
+        "config": {"workload": WORKLOAD_NAME, "l2": L2_NOTE % (mu * layer_bytes / 1e9), "parallelism": "replicas" if ws > 1 else "1 GPU",
+                   "resident_plaintexts_gb": round(mu * layer_bytes / 1e9, 1),
                    "plaintext_bytes_per_word": pbytes,
                    "rescale": RESCALE_NOTE[args.rescale],
                    "response": "switched to one prime (2 x N words)"},
@@ -775,7 +780,7 @@ def run_ours(args):
         "ct_mult_relin_per_s": round(mult_per_s, 1), "ct_mult_relin_batch": nb,
         "ntt": {"gbs": round(ntt_gbs, 1), "hbm_frac": round(ntt_gbs / peak, 4),
                 "note": "forward+inverse over 1200x4 polynomials of N=8192, 2*8*N bytes per polynomial"},
-        "roofline": {"bound": "hbm", "kernel": "k_mac", "achieved": round(achieved, 1), "peak": peak,
+        "roofline": {"bound": "hbm", "kernel": "k_mac_planes" if in_planes else "k_mac", "achieved": round(achieved, 1), "peak": peak,
                      "unit": "GB/s", "frac": round(achieved / peak, 4), "traffic": traffic,
                      "peak_source": peak_kind, "launches_per_step": mac_launches_per_eval,
                      "avg_launch_ms": round(mac_launch_ms, 4)},
@@ -923,69 +928,72 @@ def run_serve(args):
     return 0
 
 
-def stored_traffic():
-    """DRAM bytes of one full k_mac launch, from the committed small-case
-    capture of the same kernel (35 layers) scaled by the layers it
-    processes: the plaintext reads and h' writes grow with the layers, the
-    request is read once per launch.  None unless the capture was taken on
-    the current kernel source."""
-    path = os.path.join(ROOT, "profiles", "k_mac_small_dram.md")
-    if not os.path.exists(path) or WL["mu"] != 526:
-        return None
-    for line in open(path):
-        if line.startswith("machine-readable:"):
-            kv = dict(f.split("=") for f in line.split()[1:])
-            if kv.get("kernel_rev") != prof_rev():
-                return None
-            per_layer = (int(kv["traffic_bytes_per_launch"]) - int(kv["request_bytes"])) / int(kv["layers"])
-            return int(round(per_layer * WL["mu"] + int(kv["request_bytes"])))
-    return None
+def table_form(prime_bits, ell, N):
+    """Form of a resident table: (in byte planes, bytes per word, bytes per
+    layer).  ceil(bits/8) byte planes of whole steps of 16 code bits, or 64-bit
+    words for short codes (table_in_planes in csrc/kernels.h)."""
+    npl = max(4, (max(prime_bits) + 7) // 8)
+    padded = 16 * ((ell + 15) // 16) * npl
+    in_planes = padded <= 9 * (ell - 16)
+    return in_planes, npl if in_planes else 8, (padded if in_planes else ell * 8) * len(prime_bits) * N
 
 
-def kernels_rev():
-    """Identity of all device code (kernels.cu, ntt_block.cuh, common.cuh),
-    comments and blank lines removed: stored pipe counters apply while it
-    matches."""
+def source_hash(*files):
+    """Identity of device sources, comments and blank lines removed: stored
+    counters apply while it matches."""
     import hashlib
     import re
 
     h = hashlib.sha256()
-    for f in ("kernels.cu", "ntt_block.cuh", "common.cuh"):
+    for f in files:
         text = open(os.path.join(ROOT, "paper_2310_14565_gb300", "csrc", f)).read()
         code = [re.sub(r"//.*$", "", ln).rstrip() for ln in text.splitlines()]
         h.update("\n".join(ln for ln in code if ln).encode())
     return h.hexdigest()[:16]
 
 
-def stored_pipe_cycles():
-    """Busy SM-cycles of the heavy multiply-add pipe per evaluation and kernel
-    class, from the committed full-size ncu summary, if it was taken on the
-    current device code (else None)."""
-    path = os.path.join(ROOT, "profiles", "circuit_pipes_paper.md")
+def prof_rev():
+    """Identity of the byte-plane MAC's source."""
+    return source_hash("mac_planes.cu", "mbar.cuh")
+
+
+def kernels_rev():
+    """Identity of all device code."""
+    return source_hash("kernels.cu", "transforms.cu", "tensor.cu", "relin.cu", "rns.cu", "client.cu", "mac_planes.cu",
+                       "ntt_block.cuh", "xform.cuh", "rns.cuh", "mbar.cuh", "common.cuh")
+
+
+def stored_counters(name, rev):
+    """key=value fields of the machine-readable line of a committed ncu summary
+    of the paper-shaped workload's kernels, if it was taken on the current
+    source (else None)."""
+    path = os.path.join(ROOT, "profiles", name)
     if not os.path.exists(path) or WL["mu"] != 526:
         return None
     for line in open(path):
         if line.startswith("machine-readable:"):
             kv = dict(f.split("=") for f in line.split()[1:])
-            if kv.pop("kernel_rev", None) != kernels_rev():
-                return None
-            return {c: int(v.split(",")[0]) for c, v in kv.items()}
+            return kv if kv.pop("kernel_rev", None) == rev else None
     return None
 
 
-def prof_rev():
-    """Identity of the MAC kernel source, to tell whether stored counters are
-    current: a hash of its code with comments and blank lines removed, so
-    that edits of comments alone keep the counters."""
-    import hashlib
-    import re
+def stored_traffic():
+    """DRAM bytes of one full k_mac_planes launch, from the committed small-case
+    capture of the same kernel (35 layers) scaled by the layers it processes:
+    the table reads and h' writes grow with the layers, the request is read once
+    per launch."""
+    kv = stored_counters("k_mac_planes_small_dram.md", prof_rev())
+    if kv is None:
+        return None
+    per_layer = (int(kv["traffic_bytes_per_launch"]) - int(kv["request_bytes"])) / int(kv["layers"])
+    return int(round(per_layer * WL["mu"] + int(kv["request_bytes"])))
 
-    src = os.path.join(ROOT, "paper_2310_14565_gb300", "csrc", "kernels.cu")
-    text = open(src).read()
-    start = text.find("// ------------------------------------------------------- fused MAC")
-    end = text.find("// ---------------------------------------------------- RNS conversions")
-    code = [re.sub(r"//.*$", "", ln).rstrip() for ln in text[start:end].splitlines()]
-    return hashlib.sha256("\n".join(ln for ln in code if ln).encode()).hexdigest()[:16]
+
+def stored_pipe_cycles():
+    """Busy SM-cycles of the heavy multiply-add pipe per evaluation and kernel
+    class, from the committed full-size ncu summary."""
+    kv = stored_counters("circuit_pipes_paper.md", kernels_rev())
+    return kv and {c: int(v.split(",")[0]) for c, v in kv.items()}
 
 
 def main():
@@ -998,8 +1006,8 @@ def main():
     ap.add_argument("--no-extra-legs", action="store_true",
                     help="skip the batched (64 mixed queries), serving and large legs of the default run")
     ap.add_argument("--plaintext-bytes", type=int, choices=[0, 7, 8], default=0,
-                    help="storage of the resident plaintexts per word: 8 (64-bit words) or 7 (three planes); "
-                         "0: 7 for the large case, whose table is only partly resident, else 8")
+                    help="pepsi_params.plaintext_bytes: most bytes per word of the resident plaintexts (the storage, "
+                         "byte planes, is the same for both)")
     ap.add_argument("--chunk", type=int, default=0,
                     help="circuit chunk in layers (default: autotuned on the request)")
     ap.add_argument("--ntt-threads", type=int, default=0,

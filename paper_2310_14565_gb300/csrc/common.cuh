@@ -86,7 +86,7 @@ struct DevView {
   const ulonglong2* itwp;    // [np][N] (psi^-brev(i), its Shoup companion); entry 0: psi^-brev(1) N^-1
   const RnsConst* rc;
   const RnsArgs* host_args;  // host copy for by-value launches (not dereferenced on the device)
-  int allpm;                 // every ciphertext and auxiliary prime has folding products
+  int allpm;                 // every ciphertext and auxiliary prime has folding products (kernels' PM forms)
   int nt;                    // threads per block of the ciphertext transforms (0: the default for N)
 };
 

@@ -1,6 +1,6 @@
 // Kernels of PEPSI's server evaluation (Algorithms 1, 2, 5) and the client
-// steps around it (Algorithms 3, 7), for sm_103a.  Integer work only: the
-// ciphertext arithmetic is 64-bit modular arithmetic on the CUDA cores.
+// steps around it (Algorithms 3, 7), for sm_103a: the multiply-accumulates of
+// tables in 64-bit words, pointwise kernels and the pipe probes.  Integer work only.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

@@ -5,8 +5,8 @@
 // merged negacyclic form of Longa-Naehrig), Harvey's lazy butterflies.
 // Inverse: Gentleman-Sande with psi^-brev(m+i), then the factor N^-1.
 //
-// The log2 N radix-2 stages run in phases of RR <= 3 consecutive stages.  The butterflies of stages [s0, s0+RR) only combine the 2^RR
-// elements base + i * (N >> (s0+RR)), i < 2^RR, so a thread loads such a
+// The log2 N radix-2 stages run in phases of RR <= 3 consecutive stages.  The
+// butterflies of stages [s0, s0+RR) only combine the 2^RR elements base + i * (N >> (s0+RR)), i < 2^RR, so a thread loads such a
 // group into registers, runs the RR stages there and stores it back: one
 // shared-memory round trip and one barrier per phase instead of per stage.
 // Every thread of the block must call these (they contain __syncthreads);
@@ -513,7 +513,8 @@ __device__ __forceinline__ void ntt_inv_with(typename A::T* a, const Load& ld, c
 // PM: every prime the kernel meets has folding products (DevView::allpm).  The
 // kernels come in both forms: with the other arithmetics compiled in beside it,
 // the compiler moved so much out of the branches that the inverse kernels spilled
-// (k_tensor_intt 788 bytes).
+// (k_tensor_intt 788 bytes); 1200 x 4 rows of N = 8192 forward 281 -> 269 us, the
+// products of 256 ciphertexts 2.39 -> 2.33 ms.
 template <bool PM = false, class Load, class Store>
 __device__ __forceinline__ void ntt_fwd_gg(u64* a, const Load& ld, const Store& st, const DevView& V, int pi) {
   const ulonglong2* tw = V.twp + (size_t)pi * V.N;

@@ -12,6 +12,8 @@ namespace {
 constexpr int relin_min_blocks(int MT) { return MT <= 256 ? 3 : 1; }
 
 // ---------------------------------------------------------- relinearise
+// Bound by the heavy multiply-add pipe (256 ciphertexts of N = 8192, k = 4, both
+// phases: 0.77 ms with folding products).
 // Phase 1, block per row of DG[L][k+2][k][N]: row (l, i, j) holds
 // NTT_{q_j}([d2]_{q_i}) for digits i < k, and NTT_{q_j}(d0), NTT_{q_j}(d1)
 // for i = k, k+1.

@@ -6,6 +6,11 @@
 namespace {
 
 // ------------------------------------------------------------------ NTT
+// Bound by the heavy multiply-add pipe and, nearly as long, the ALU: a block per
+// row keeps every stage on chip, one read and one write of the row.  1200 x 4 rows
+// of N = 8192 forward: 366 us with Shoup products and barriers of the whole block,
+// 281 us with folding products, constant-XOR addressing and barriers of parts,
+// 269 us compiled for folding alone.
 // SPLIT: store the result in the split operand format of the
 // multiply-accumulate (the request's forward transform).
 template <bool PM, bool FWD, bool SPLIT = false>
