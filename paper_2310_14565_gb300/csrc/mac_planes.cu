@@ -354,7 +354,14 @@ __global__ void __launch_bounds__(macp::threads(SHORT), 1) k_mac_planes(DevView 
       if (!__all_sync(0xffffffffu, mbar_try_wait(full(team, slot), parity)) && ok)
         ok = __all_sync(0xffffffffu, mbar_wait_bounded(full(team, slot), parity));
     };
+    // The stage is refilled by an asynchronous copy, which a generic read is ordered
+    // before only through a proxy fence: without it the copy of the stage after next
+    // overwrote rows still being read (stages of one to three steps, where a stage's
+    // reads are few and its refill comes soon: a handful of wrong items in 11 million).
+    // Every lane fences its own reads, which keeps the producer warp, the bound of
+    // short codes, free of it; no case's time changes by more than its runs differ.
     auto leave = [&]() {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();  // every lane has read the stage
       if (lane == 0) mbar_arrive(empty(team, slot));
       if (++slot == nst) {
