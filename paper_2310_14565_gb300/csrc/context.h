@@ -237,9 +237,10 @@ struct LazyRun {
 void ntt(pepsi_ctx* c, bool fwd, const u64* src, u64* dst, size_t outer, int np, int p0, size_t sos, size_t dos,
          cudaStream_t st);
 // Arith-CW-Eq (Algorithm 1) on L layers whose h' is in b.H, up to its last
-// ciphertext product (returned); and the whole circuit with per-layer rounding.
-LastMult eq_circuit_front(pepsi_ctx* c, EvalBufs& b, int L, cudaStream_t st);
-void eq_circuit(pepsi_ctx* c, EvalBufs& b, int L, cudaStream_t st);
+// ciphertext product (its operands to m); and the whole circuit with per-layer
+// rounding.  An error is that of an allocation: the words are then not made.
+cudaError_t eq_circuit_front(pepsi_ctx* c, EvalBufs& b, int L, LastMult& m, cudaStream_t st);
+cudaError_t eq_circuit(pepsi_ctx* c, EvalBufs& b, int L, cudaStream_t st);
 // Lazy rescaling: add the chunk's last products to the run sums, rounding runs as they complete.
 void lazy_chunk(pepsi_ctx* c, EvalBufs& b, const LastMult& m, const u64* VP, int L, bool end, LazyRun& r,
                 cudaStream_t st);

@@ -241,10 +241,13 @@ int enqueue_step(Lane& L, Step& step, bool capturing = false) {
     const bool last = T.done + n == L.mu;
     L.b.H = T.H;
     if (T.lr.G > 1) {
-      const LastMult m = eq_circuit_front(c, L.b, nl, st);
+      LastMult m;
+      const cudaError_t ce = eq_circuit_front(c, L.b, nl, m, st);
+      if (ce != cudaSuccess) return cuda_status(ce);
       lazy_chunk(c, L.b, m, VP, nl, last, T.lr, st);
     } else {
-      eq_circuit(c, L.b, nl, st);
+      const cudaError_t ce = eq_circuit(c, L.b, nl, st);
+      if (ce != cudaSuccess) return cuda_status(ce);
       if (valued) {
         ntt(c, true, L.b.D, L.b.D, (size_t)nl * 3, c->k, 0, kN, kN, st);
         Prof p(c, PC_POINTWISE, st);

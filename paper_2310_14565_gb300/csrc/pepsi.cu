@@ -111,8 +111,8 @@ void extend(pepsi_ctx* c, const u64* src_ntt, u64* coef, u64* Bpart, int L, cons
 // relin(D) + z * H -> out, then extend(out): the key-switching sum and the
 // affine step on the load of the inverse NTT (the relinearised product
 // itself is not stored).
-void relin_axpy_extend(pepsi_ctx* c, const u64* D, const u64* z, const u64* H, u64* out, u64* coef, u64* Bpart,
-                       int L, const u64* cstv, u64* side, u64* Rtmp, cudaStream_t st);
+cudaError_t relin_axpy_extend(pepsi_ctx* c, const u64* D, const u64* z, const u64* H, u64* out, u64* coef, u64* Bpart,
+                              int L, const u64* cstv, u64* side, u64* Rtmp, cudaStream_t st);
 
 // out = a + z * b, then extend(out) as above, the axpy on the load of the
 // inverse NTT (coef may alias b).
@@ -143,25 +143,26 @@ void mult_tail(pepsi_ctx* c, const u64* AQ, const u64* AB, const u64* BQ, const 
 
 // scratch id of the relinearisation digits (declared with the others below)
 constexpr int kScratchDG = 40;
-void relin(pepsi_ctx* c, const u64* D, u64* R, int L, cudaStream_t st) {
+cudaError_t relin(pepsi_ctx* c, const u64* D, u64* R, int L, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   u64* DG = (u64*)scratch(c, kScratchDG, (size_t)L * (c->k + 2) * c->k * c->N * 8, &e);
-  if (!DG) return;  // the allocation error resurfaces through cudaGetLastError
+  if (!DG) return e;
   Prof p(c, PC_RELIN, st, 2);
   launch_relin(c->V, D, c->d_rlk, DG, R, L, st);
+  return cudaSuccess;
 }
 
-void relin_axpy_extend(pepsi_ctx* c, const u64* D, const u64* z, const u64* H, u64* out, u64* coef, u64* Bpart,
-                       int L, const u64* cstv, u64* side, u64* Rtmp, cudaStream_t st) {
+cudaError_t relin_axpy_extend(pepsi_ctx* c, const u64* D, const u64* z, const u64* H, u64* out, u64* coef, u64* Bpart,
+                              int L, const u64* cstv, u64* side, u64* Rtmp, cudaStream_t st) {
   if (!c->relin_fused) {  // the schedule's unfused form: R stored in Rtmp, then the affine step
-    relin(c, D, Rtmp, L, st);
+    CK(relin(c, D, Rtmp, L, st));
     axpy_extend(c, Rtmp, z, H, out, coef, Bpart, L, cstv, side, st);
-    return;
+    return cudaSuccess;
   }
   const size_t kbN = (size_t)c->kb * c->N;
   cudaError_t e = cudaSuccess;
   u64* DG = (u64*)scratch(c, kScratchDG, (size_t)L * (c->k + 2) * c->k * c->N * 8, &e);
-  if (!DG) return;  // the allocation error resurfaces through cudaGetLastError
+  if (!DG) return e;
   {
     Prof p(c, PC_RELIN, st, 2);
     launch_relin_digits(c->V, D, DG, L, st);
@@ -172,6 +173,7 @@ void relin_axpy_extend(pepsi_ctx* c, const u64* D, const u64* z, const u64* H, u
     launch_lift(c->V, coef, Bpart, L, cstv, side, st);
   }
   ntt(c, true, Bpart, Bpart, (size_t)L * 2, c->kb, c->k, kbN, kbN, st);
+  return cudaSuccess;
 }
 
 
@@ -211,12 +213,12 @@ cudaError_t eval_bufs(pepsi_ctx* c, int Lc, bool need_pc, EvalBufs* b) {
 
 
 // Arith-CW-Eq (Algorithm 1) on L layers whose h' is in H (NTT form), up to
-// its last ciphertext product, whose operands are returned (h >= 2).  For
+// its last ciphertext product, whose operands go to m (h >= 2).  For
 // h = 1 there is no product: D <- h' directly.  Hc <- h' in coefficient form.
-LastMult eq_circuit_front(pepsi_ctx* c, EvalBufs& b, int L, cudaStream_t st) {
+cudaError_t eq_circuit_front(pepsi_ctx* c, EvalBufs& b, int L, LastMult& m, cudaStream_t st) {
   const size_t k = c->k, N = c->N;
   const size_t ct2 = 2 * k * N;
-  LastMult m;
+  m = LastMult{};
   auto last = [&](const u64* AQ, const u64* AB, const u64* BQ, const u64* BB, const u64* cQ, const u64* side,
                   bool square) {
     m.AQ = AQ;
@@ -244,30 +246,32 @@ LastMult eq_circuit_front(pepsi_ctx* c, EvalBufs& b, int L, cudaStream_t st) {
     case 4: {  // u = R(h'^2) - 3h';  E = Mult(u, u + 2)
       extend(c, b.H, b.Hc, b.XB, L, nullptr, nullptr, st);
       mult_tail(c, b.H, b.XB, b.H, b.XB, nullptr, nullptr, true, b.T3, b.D, L, st);
-      relin_axpy_extend(c, b.D, cst(c, CS_M3), b.H, b.U, b.X, b.YB, L, cst(c, CS_D_2), b.side, b.R, st);
+      CK(relin_axpy_extend(c, b.D, cst(c, CS_M3), b.H, b.U, b.X, b.YB, L, cst(c, CS_D_2), b.side, b.R, st));
       last(b.U, b.YB, b.U, b.YB, cst(c, CS_D_2), b.side, false);
       break;
     }
     case 8: {  // u = R(h'^2) - 7h'; w = R(u^2); E = Mult(w + 12u, w + 16u + 60)
       extend(c, b.H, b.Hc, b.XB, L, nullptr, nullptr, st);
       mult_tail(c, b.H, b.XB, b.H, b.XB, nullptr, nullptr, true, b.T3, b.D, L, st);
-      relin_axpy_extend(c, b.D, cst(c, CS_M7), b.H, b.U, b.X, b.XB, L, nullptr, nullptr, b.R, st);
+      CK(relin_axpy_extend(c, b.D, cst(c, CS_M7), b.H, b.U, b.X, b.XB, L, nullptr, nullptr, b.R, st));
       mult_tail(c, b.U, b.XB, b.U, b.XB, nullptr, nullptr, true, b.T3, b.D, L, st);
-      relin(c, b.D, b.W, L, st);
+      CK(relin(c, b.D, b.W, L, st));
       axpy_extend(c, b.W, cst(c, CS_P12), b.U, b.X, b.R, b.XB, L, nullptr, nullptr, st);
       axpy_extend(c, b.W, cst(c, CS_P16), b.U, b.Y, b.U, b.YB, L, cst(c, CS_D_60), b.side, st);
       last(b.X, b.XB, b.Y, b.YB, cst(c, CS_D_60), b.side, false);
       break;
     }
   }
-  return m;
+  return cudaSuccess;
 }
 
 // The whole circuit with per-layer rounding: D <- prod_{i<h}(h' - i) as
 // un-relinearised 3-component ciphertexts (coefficient form).
-void eq_circuit(pepsi_ctx* c, EvalBufs& b, int L, cudaStream_t st) {
-  const LastMult m = eq_circuit_front(c, b, L, st);
+cudaError_t eq_circuit(pepsi_ctx* c, EvalBufs& b, int L, cudaStream_t st) {
+  LastMult m;
+  CK(eq_circuit_front(c, b, L, m, st));
   if (m.AQ) mult_tail(c, m.AQ, m.AB, m.BQ, m.BB, m.cQ, m.side, m.square, b.T3, b.D, L, st);
+  return cudaSuccess;
 }
 
 
@@ -405,7 +409,7 @@ cudaError_t finish_request(pepsi_ctx* c, EvalBufs& b, u64* acc, bool acc_ntt, in
                            cudaStream_t st) {
   const size_t kN = (size_t)c->k * c->N;
   if (acc_ntt) ntt(c, false, acc, acc, 3, c->k, 0, kN, kN, st);  // value-weighted sum, NTT form
-  relin(c, acc, b.R, 1, st);
+  CK(relin(c, acc, b.R, 1, st));
   axpy(c, b.zero, cst(c, CS_ZINV), b.R, b.R, 2, st);
   ntt(c, false, b.R, b.out, 2, c->k, 0, kN, kN, st);
   if (mode == PEPSI_MODE_CARDINALITY || mode == PEPSI_MODE_SUM) {
@@ -549,10 +553,11 @@ int eval_core(pepsi_ctx* c, int set_id, const u64* cts, u32 layer0, u32 nl, int 
     }
     const u64* VP = valued ? S.dVP + (size_t)l0 * vstride : nullptr;
     if (G > 1) {  // a6 + a7 with lazy rescaling
-      const LastMult m = eq_circuit_front(c, b, L, st);
+      LastMult m;
+      CKS(eq_circuit_front(c, b, L, m, st));
       lazy_chunk(c, b, m, VP, L, l0 + L == end, lr, st);
     } else {
-      eq_circuit(c, b, L, st);  // a6
+      CKS(eq_circuit(c, b, L, st));  // a6
       if (e_out) CKS(copy_any(e_out + (size_t)(l0 - layer0) * ct3, b.D, (size_t)L * ct3 * 8, st));
       if (valued) {  // a7, Algorithms 4-5: sum of val_s[i'] * E_{i'} in NTT form
         ntt(c, true, b.D, b.D, (size_t)L * 3, c->k, 0, k * N, k * N, st);
@@ -714,11 +719,12 @@ int eval_batch_core(pepsi_ctx* c, int nq, const int* set_ids, const u64* const* 
         b.H = HB + (size_t)g * hq + (res ? (size_t)l0 * ct2 : 0);
         const u64* VP = gmode[g] >= PEPSI_MODE_LABELS ? S.dVP + (size_t)l0 * vstride : nullptr;
         if (lr[g].G > 1) {
-          const LastMult m = eq_circuit_front(c, b, L, st);
+          LastMult m;
+          CKS(eq_circuit_front(c, b, L, m, st));
           lazy_chunk(c, b, m, VP, L, l0 + L == mu, lr[g], st);
           continue;
         }
-        eq_circuit(c, b, L, st);
+        CKS(eq_circuit(c, b, L, st));
         if (VP) {
           ntt(c, true, b.D, b.D, (size_t)L * 3, c->k, 0, kN, kN, st);
           Prof p(c, PC_POINTWISE, st);
@@ -1933,7 +1939,7 @@ int pepsi_ct_mult(pepsi_ctx* c, const uint64_t* a, const uint64_t* b, size_t n, 
     launch_relin_digits(c->V, D, DG, L, st);
     launch_relin_axpy_intt(c->V, DG, c->d_rlk, zero, D, R, out, L, st);
   } else if (relin_flag) {
-    relin(c, D, R, L, st);
+    CKS(relin(c, D, R, L, st));
     ntt(c, false, R, out, n * 2, c->k, 0, kN, kN, st);
   } else {
     CKS(cudaMemcpyAsync(out, D, n * 3 * kN * 8, cudaMemcpyDeviceToDevice, st));
@@ -1950,7 +1956,7 @@ int pepsi_relin(pepsi_ctx* c, const uint64_t* in, size_t n, uint64_t* out, void*
   cudaError_t e = cudaSuccess;
   u64* R = (u64*)scratch(c, S_R, n * 2 * kN * 8, &e);
   if (!R) return cuda_status(e);
-  relin(c, in, R, (int)n, st);
+  CKS(relin(c, in, R, (int)n, st));
   ntt(c, false, R, out, n * 2, c->k, 0, kN, kN, st);
   return cuda_status(cudaGetLastError());
 }
