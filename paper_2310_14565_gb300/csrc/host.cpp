@@ -178,12 +178,11 @@ static bool folds_below(const DevPrime& p, u128 x) {
          ((u128)1 << p.nbits) + top * p.d < 2 * (u128)p.q && (x >> p.nbits) * p.d < ((u128)1 << 31);
 }
 
-void rns_constants(const std::vector<u64>& Q, const std::vector<u64>& B, u64 t, RnsConst* rc) {
-  const size_t k = Q.size(), kb = B.size();
-  *rc = RnsConst{};
-  // folding products throughout when every intermediate value of the conversions
-  // fits: Garner steps below 3 q_i + 4 q_i (digits of other primes below 4 q_i),
-  // Horner sums below 2 p + a digit, t x below 2^(n+32)
+// Folding products throughout when every intermediate value of the conversions
+// fits: Garner steps below 3 q_i + 4 q_i (digits of other primes below 4 q_i),
+// Horner sums below 2 p + a digit, t x below 2^(n+32).
+bool folding_conversions(const std::vector<u64>& Q, const std::vector<u64>& B, u64 t) {
+  const size_t k = Q.size();
   std::vector<u64> all = Q;
   all.insert(all.end(), B.begin(), B.end());
   const u64 qmax = *std::max_element(Q.begin(), Q.end()), bmax = *std::max_element(B.begin(), B.end());
@@ -194,6 +193,13 @@ void rns_constants(const std::vector<u64>& Q, const std::vector<u64>& B, u64 t, 
     pm = folds_below(p, 8 * (u128)p.q) && folds_below(p, 2 * (u128)p.q + other) && own < 4 * p.q &&
          (i < k || other < 2 * p.q) && ((u128)1 << p.nbits) + (u128)(t + 1) * p.d < 2 * (u128)p.q;
   }
+  return pm;
+}
+
+void rns_constants(const std::vector<u64>& Q, const std::vector<u64>& B, u64 t, RnsConst* rc) {
+  const size_t k = Q.size(), kb = B.size();
+  *rc = RnsConst{};
+  const bool pm = folding_conversions(Q, B, t);
   rc->pm = pm ? 1 : 0;
   auto comp = [&](u64 w, u64 q) { return pm ? companion(w, make_prime(q, 1)) : shoup_of(w, q); };
   for (size_t i = 0; i < k; ++i)

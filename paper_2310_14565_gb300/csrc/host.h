@@ -23,6 +23,8 @@ DevPrime make_prime(u64 q, u32 N);
 u64 companion(u64 w, const DevPrime& p);
 // twiddles psi^brev(i) (fwd) and psi^-brev(i) (inv) with their companions
 void twiddles(const DevPrime& p, u64 psi, u32 N, u64* tw, u64* tws, u64* itw, u64* itws);
+// whether the conversions between Q and B can use folding products throughout
+bool folding_conversions(const std::vector<u64>& Q, const std::vector<u64>& B, u64 t);
 // constants of the exact RNS conversions
 void rns_constants(const std::vector<u64>& Qp, const std::vector<u64>& Bp, u64 t, RnsConst* rc);
 // round(Q v / t) mod q_i for v in [0, t)

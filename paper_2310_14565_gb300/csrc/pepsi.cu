@@ -1058,27 +1058,29 @@ int pepsi_setup(const pepsi_params* params, uint64_t key_seed, pepsi_ctx** out) 
   // auxiliary base B: primes with log2 B >= log2(t N Q G) + 3, G the
   // longest run of layers whose exact products are summed before rounding
   // (and, for the value modes, N t / 2 times more: the product with a value
-  // plaintext of centred coefficients).  57-bit primes (folding products) where
-  // they are at most one more than 61-bit ones would be, else 59-bit ones (forward
-  // transforms without the per-stage reduction) where as few, else 61-bit.
+  // plaintext of centred coefficients).  57-bit primes (folding products) where as
+  // few as of 61 bits, or one more where the conversions fold with them (five 50-bit
+  // primes at N = 16384 do not: the sixth prime only added work); else 59-bit ones
+  // (forward transforms without the per-stage reduction) where as few, else 61-bit.
   c->value_margin = params->server_values != 0 && c->rescale_cap > 1;
   const double needB = std::log2((double)c->t) + c->logN + lq + std::ceil(std::log2((double)c->rescale_cap)) + 3.0 +
                        (c->value_margin ? std::ceil(c->logN + std::log2((double)c->t) - 1.0) : 0.0);
-  const double n61 = std::ceil(needB / 60.9);
-  const int bbits = std::ceil(needB / 56.9) <= n61 + 1 && std::ceil(needB / 56.9) <= PEPSI_MAXB ? 57
-                    : std::ceil(needB / 58.9) <= n61                                            ? 59
-                                                                                                : 61;
-  double haveB = 0;
-  std::vector<u64> taken = c->Q;
-  while (haveB < needB) {
-    if ((int)c->B.size() >= PEPSI_MAXB) {
-      delete c;
-      return PEPSI_E_PARAM;
+  auto base = [&](int bits) {  // empty: more than PEPSI_MAXB primes
+    std::vector<u64> B, taken = c->Q;
+    for (double have = 0; have < needB; have += std::log2((double)B.back())) {
+      if (B.size() >= PEPSI_MAXB) return std::vector<u64>();
+      B.push_back(hostmath::find_prime(bits, c->N, taken));
+      taken.push_back(B.back());
     }
-    u64 p = hostmath::find_prime(bbits, c->N, taken);
-    taken.push_back(p);
-    c->B.push_back(p);
-    haveB += std::log2((double)p);
+    return B;
+  };
+  c->B = base(57);
+  const double n61 = std::ceil(needB / 60.9);
+  if (c->B.empty() || (double)c->B.size() > n61 + (hostmath::folding_conversions(c->Q, c->B, c->t) ? 1 : 0))
+    c->B = base(std::ceil(needB / 58.9) <= n61 ? 59 : 61);
+  if (c->B.empty()) {
+    delete c;
+    return PEPSI_E_PARAM;
   }
   c->kb = (int)c->B.size();
   // MAC partial sums (Karatsuba form, S0 = sum cl xl, S2 = sum ch xh and
