@@ -131,6 +131,7 @@ __global__ void k_scale_round(const __grid_constant__ RnsArgs A, const u64* __re
 }  // namespace
 
 // instantiate F<K, KB, PM> for the prime counts in use, else the run-time generic version
+// (labelled N = 16384, 8 + 10 primes, h = 8 and 100 layers: 14.35 ms an evaluation, 15.17 generic)
 #define PEPSI_RNS_COUNTS(V, LAUNCH, PM)               \
   switch ((V).k * 16 + (V).kb) {                      \
     case 3 * 16 + 3: LAUNCH(3, 3, PM); break;         \
@@ -140,6 +141,7 @@ __global__ void k_scale_round(const __grid_constant__ RnsArgs A, const u64* __re
     case 4 * 16 + 6: LAUNCH(4, 6, PM); break;         \
     case 8 * 16 + 8: LAUNCH(8, 8, PM); break;         \
     case 8 * 16 + 9: LAUNCH(8, 9, PM); break;         \
+    case 8 * 16 + 10: LAUNCH(8, 10, PM); break;       \
     default: LAUNCH(0, 0, PM); break;                 \
   }
 #define PEPSI_RNS_DISPATCH(V, LAUNCH)       \

@@ -1,7 +1,9 @@
-"""The auxiliary base of the exact products: how many primes a context takes."""
+"""The auxiliary base of the exact products: how many primes a context takes, and the
+words of the conversions at the largest counts in use."""
+import numpy as np
 import pytest
 
-from gpu_helpers import torch_cuda
+from gpu_helpers import T, torch_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -26,3 +28,30 @@ def test_auxiliary_primes(kw, kb):
     gc = pepsi.Context(**kw)
     assert gc.kb == kb
     gc.close()
+
+
+def test_ten_auxiliary_primes_match_oracle():
+    """Eight 56-bit primes, values, runs of up to 40000 layers: ten auxiliary
+    primes, the conversions' largest instantiated form.  Labels and masked sum
+    against the oracle word for word."""
+    torch_cuda()
+    import oracle
+    import paper_2310_14565_gb300 as pepsi
+    from paper_2310_14565_gb300.workload import make_sets
+
+    N, bits, h, lb, mu = 256, [56] * 8, 4, 10, 8
+    sets = make_sets(20, 70, 5, bits=32)
+    values = np.arange(1, 71, dtype=np.uint32)
+    oc = oracle.Ctx(N=N, t=T, prime_bits=bits, h=h, lambda_bar=lb, mu=mu, hash_key=0x5EED)
+    gc = pepsi.Context(N=N, t=T, prime_bits=bits, h=h, lambda_bar=lb, mu=mu, hash_key=0x5EED, key_seed=3,
+                       rescale_group=40000, server_values=1)
+    assert gc.kb == 10
+    s, rlk = oc.keygen(3)
+    rc, Ts, V, _ = oc.server_table_values(sets.server, values)
+    assert rc == 0
+    sid = gc.server_load_values(sets.server, values)
+    cts, _ = gc.query(sets.client, 4)
+    for mode in (2, 3):
+        want = oc.eval(rlk, cts, Ts, mode=mode, mask_seed=7, V=V, group=mu)
+        assert np.array_equal(gc.eval(sid, cts, mode=mode, mask_seed=7), want), mode
+    assert np.array_equal(gc.eval(sid, cts), oc.eval(rlk, cts, Ts, group=mu))
