@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "context.h"
+#include "xform.cuh"
 
 using hostmath::u128;
 
@@ -1684,9 +1685,9 @@ int pepsi_autotune(pepsi_ctx* c, int set_id, const uint64_t* cts, void* stream, 
     if ((u32)chunk >= G->mu) break;  // one chunk holds every layer
   }
   c->chunk = best_chunk;
-  // 2: threads per transform block (the default, half and twice it)
+  // 2: threads per transform block (the default, timed above, against half and twice it)
   if (!rc) {
-    const int def = c->N >= 16384 ? 1024 : std::max(32, std::min(256, c->N / 8));
+    const int def = ntt_threads(c->N);
     int best_nt = 0;
     for (int nt : {def / 2, def * 2}) {
       if (nt < 64 || nt > 1024) continue;
