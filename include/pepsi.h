@@ -106,14 +106,17 @@ typedef struct {
                               ciphertexts [B][ell][2][k][N], every server layer one block of
                               plaintexts per request block, and the response B ciphertexts
                               [B][2][r][N], block j answering bins j*N .. j*N + N - 1 */
-  uint32_t plaintext_bytes;/* most bytes per word the caller allows for the resident server
-                              plaintexts (NTT form): 0 or 8, or 7 (every q_i < 2^56, else
-                              PEPSI_E_PARAM).  The storage is the same for all of them: byte
-                              planes of ceil(bits(q_i) / 8) bytes per word (at least 4; 7 for
-                              55-bit primes) with the code bits padded to a multiple of 16,
-                              or 64-bit words for codes so short (below about 80 bits with 7
-                              bytes, 43 with 5) that planes would be slower.  Results do not
-                              depend on it */
+  uint32_t plaintext_bytes;/* form of the resident server plaintexts (NTT form).  A table of ell
+                              code bits takes per prime and point either 64-bit words, 8 ell
+                              bytes, or byte planes, 16 ceil(ell / 16) n bytes with n =
+                              ceil(bits(q_i) / 8) of the widest prime, at least 4 (7 for 55-bit
+                              primes).  0 or 8: the faster form, which is planes where
+                              16 ceil(ell / 16) n <= 9 (ell - 16); the smaller one where the
+                              budget does not hold every layer in the faster.  7 (every q_i <
+                              2^56, else PEPSI_E_PARAM): the smaller form throughout.  It is 7
+                              bytes per word for whole steps of 16 bits and 56-bit primes, less
+                              for narrower ones, and at most 8, which short codes take whose
+                              last step is mostly padding.  Results do not depend on it */
   uint32_t gamma;          /* client maximum bin load (Table 2, Section 4): 0 or 1 = cuckoo
                               hashing with one item per bin (the paper's evaluation); 2..16 =
                               bins of gamma slots, so up to gamma * b client items.  The client

@@ -1295,8 +1295,9 @@ int pepsi_set_schedule(pepsi_ctx* c, const pepsi_schedule* s) {
 namespace {
 // Device side of one block: its table [mu][N] (and values) to codeword
 // positions, value plaintexts, and the resident prefix of mu_res layers of
-// NTT-form plaintexts.
-int load_block(pepsi_ctx* c, std::vector<u64>&& hT, std::vector<uint32_t>* hV, u32 mu, u32 mu_res, int* internal) {
+// NTT-form plaintexts, as words or in byte planes.
+int load_block(pepsi_ctx* c, std::vector<u64>&& hT, std::vector<uint32_t>* hV, u32 mu, u32 mu_res, bool words,
+               int* internal) {
   ServerSet S;
   S.mu = mu;
   S.hT = std::move(hT);
@@ -1331,7 +1332,7 @@ int load_block(pepsi_ctx* c, std::vector<u64>&& hT, std::vector<uint32_t>* hV, u
     }
   }
   S.mu_res = mu_res;
-  S.words = !table_in_planes(c->ell, c->npl);
+  S.words = words;
   if (S.mu_res && S.words) {
     e = cudaMalloc((void**)&S.dP, (size_t)S.mu_res * c->ell * k * N * 8);
     if (e != cudaSuccess) {
@@ -1410,13 +1411,19 @@ int server_load_impl(pepsi_ctx* c, const uint64_t* items, bool with_values, cons
   if (rc) return rc;
   // resident NTT-form plaintexts: the longest prefix of layers the budget
   // holds for every block
-  const size_t per_layer = (table_in_planes(c->ell, c->npl) ? plane_layer_bytes(c->ell, c->k * N, c->npl)
-                                                             : (size_t)c->ell * c->k * N * 8) * c->blocks;
+  const size_t in_planes = plane_layer_bytes(c->ell, c->k * N, c->npl) * c->blocks;
+  const size_t in_words = (size_t)c->ell * c->k * N * 8 * c->blocks;
   size_t freeb = 0, totalb = 0;
   cudaMemGetInfo(&freeb, &totalb);
   const u64 cap = c->prm.resident_bytes;
   const size_t budget = cap == 0 ? (size_t)(0.6 * (double)freeb) : (cap == UINT64_MAX ? 0 : (size_t)cap);
-  const u32 mu_res = (u32)std::min<size_t>(mu, budget / per_layer);
+  // The faster form, or the smaller one (more layers resident) where it does not
+  // hold them all, or where the caller asks for at most 7 bytes per word: a
+  // regenerated layer costs several times what the slower form does.
+  bool words = !table_in_planes(c->ell, c->npl);
+  if (in_words != in_planes && (c->plaintext_bytes == 7 || budget / (words ? in_words : in_planes) < mu))
+    words = in_words < in_planes;
+  const u32 mu_res = (u32)std::min<size_t>(mu, budget / (words ? in_words : in_planes));
   for (u32 b = 0; b < c->blocks; ++b) {
     std::vector<u64> T((size_t)mu * N);
     std::vector<uint32_t> V(with_values ? (size_t)mu * N : 0);
@@ -1425,7 +1432,7 @@ int server_load_impl(pepsi_ctx* c, const uint64_t* items, bool with_values, cons
       if (with_values) memcpy(&V[(size_t)l * N], &G.hV[(size_t)l * bins + (size_t)b * N], N * 4);
     }
     int id = -1;
-    rc = load_block(c, std::move(T), with_values ? &V : nullptr, mu, mu_res, &id);
+    rc = load_block(c, std::move(T), with_values ? &V : nullptr, mu, mu_res, words, &id);
     if (rc) {
       for (int i : G.blk) free_set(c->sets[i]);
       return rc;
