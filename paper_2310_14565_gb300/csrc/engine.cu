@@ -52,7 +52,8 @@ struct Slot {
   int mode = 0;
   u64 mask_seed = 0;
   u64* out = nullptr;
-  u64* C = nullptr;    // [ell][2][k][N] request, NTT form, split operand format
+  u64* C = nullptr;    // request, NTT form, split operand words and half sums; null on a lane without word chunks
+  u64* P = nullptr;    // request, NTT form, byte planes; null on a lane without resident byte planes
   u64* H = nullptr;    // [Lc][2][k][N] h' of the current chunk
   u64* acc = nullptr;  // [3][k][N] layer sum
   u64* X = nullptr;    // [3][k+kb][N] run sum of the exact products (lazy rescaling)
@@ -116,20 +117,19 @@ struct pepsi_graph {
 
 namespace {
 
-// A lane of a wholly resident set keeps its requests in byte planes; one with
-// regenerated layers keeps them as split words (and makes the byte planes of a
-// resident chunk in the lane's scratch).
-bool in_planes(const Lane& L) { return L.mu_res == L.mu && !L.c->sets[L.set].words; }
-size_t prepared_words(const Lane& L) {
-  const size_t kN = (size_t)L.c->k * L.c->N;
-  return in_planes(L) ? request_plane_words(L.c->ell, kN) : request_prepared_words(L.c->ell, kN);
-}
+// The formats of a lane's requests: byte planes where layers are resident in
+// planes, split words where chunks are words (tables of short codes, regenerated
+// layers); a partly resident set in planes takes both.
+bool reads_planes(const Lane& L) { return L.mu_res > 0 && !L.c->sets[L.set].words; }
+bool reads_words(const Lane& L) { return L.mu_res < L.mu || L.c->sets[L.set].words; }
 
 // Bytes of a request's device state on a lane (lazy: with its run sum).
 size_t request_bytes(const Lane& L, bool lazy) {
   const pepsi_ctx* c = L.c;
   const size_t kN = (size_t)c->k * c->N;
-  size_t w = prepared_words(L) + (size_t)L.Lc * 2 * kN + 3 * kN;
+  size_t w = (size_t)L.Lc * 2 * kN + 3 * kN;
+  if (reads_words(L)) w += request_prepared_words(c->ell, kN);
+  if (reads_planes(L)) w += request_plane_words(c->ell, kN);
   if (lazy) w += (size_t)3 * (c->k + c->kb) * c->N;
   return w * 8;
 }
@@ -157,12 +157,13 @@ int admit(pepsi_engine* e, Lane& L, int s, u64 ticket, const Request& r, size_t 
   S.out = r.out;
   S.bytes = bytes;
   const u32 G = rescale_run(c, L.mu, r.mode);
-  cudaError_t err = pool_alloc(e, &S.C, prepared_words(L), st);
+  cudaError_t err = cudaSuccess;
+  if (reads_words(L)) err = pool_alloc(e, &S.C, request_prepared_words(c->ell, kN), st);
+  if (err == cudaSuccess && reads_planes(L)) err = pool_alloc(e, &S.P, request_plane_words(c->ell, kN), st);
   if (err == cudaSuccess) err = pool_alloc(e, &S.H, (size_t)L.Lc * 2 * kN, st);
   if (err == cudaSuccess) err = pool_alloc(e, &S.acc, 3 * kN, st);
   if (err == cudaSuccess && G > 1) err = pool_alloc(e, &S.X, (size_t)3 * (c->k + c->kb) * c->N, st);
-  if (err == cudaSuccess)
-    err = in_planes(L) ? prepare_request(c, r.cts, nullptr, S.C, st) : prepare_request(c, r.cts, S.C, nullptr, st);
+  if (err == cudaSuccess) err = prepare_request(c, r.cts, S.C, S.P, st);
   if (err != cudaSuccess) return cuda_status(err);
   if (G > 1) {
     S.lr.X = S.X;
@@ -174,9 +175,9 @@ int admit(pepsi_engine* e, Lane& L, int s, u64 ticket, const Request& r, size_t 
 }
 
 void release(Slot& S, cudaStream_t st) {
-  for (u64* p : {S.C, S.H, S.acc, S.X})
+  for (u64* p : {S.C, S.P, S.H, S.acc, S.X})
     if (p) cudaFreeAsync(p, st);
-  S.C = S.H = S.acc = S.X = nullptr;
+  S.C = S.P = S.H = S.acc = S.X = nullptr;
   S.busy = false;
 }
 
@@ -192,30 +193,22 @@ int enqueue_step(Lane& L, Step& step, bool capturing = false) {
   if (L.pos < L.mu_res) n = std::min<u32>(n, L.mu_res - L.pos);
   const int nl = (int)n;
   const u64* Cs[kMaxSlots];
+  const u32* planes[kMaxSlots];
   u64* Hs[kMaxSlots];
   int act[kMaxSlots], na = 0;
   for (int s = 0; s < L.nslots; ++s)
     if (L.slot[s].busy) {
       Cs[na] = L.slot[s].C;
+      planes[na] = reinterpret_cast<const u32*>(L.slot[s].P);
       Hs[na] = L.slot[s].H;
       act[na++] = s;
     }
   if (!na) return PEPSI_OK;
-  if (L.pos < L.mu_res && in_planes(L)) {
+  if (L.pos < L.mu_res && !S.words) {
     for (int q0 = 0; q0 < na; q0 += c->batch_requests) {  // launches of at most batch_requests requests
       Prof p(c, PC_MAC, st);
-      const u32* planes[kMaxSlots];
-      const int nq = std::min(c->batch_requests, na - q0);
-      for (int q = 0; q < nq; ++q) planes[q] = reinterpret_cast<const u32*>(Cs[q0 + q]);
-      launch_mac_planes(c->V, nq, planes, S.planes(c->npl), Hs + q0, c->ell, (int)L.pos, nl, c->d_err, st);
-    }
-  } else if (L.pos < L.mu_res && !S.words) {  // split words: byte planes of one request at a time
-    for (int q = 0; q < na; ++q) {
-      Prof p(c, PC_MAC, st, 2);
-      u32* planes = reinterpret_cast<u32*>(c->scratch[S_CP].p);
-      launch_pack_request(c->V, Cs[q], true, c->ell, planes, st);
-      const u32* pc = planes;
-      launch_mac_planes(c->V, 1, &pc, S.planes(c->npl), Hs + q, c->ell, (int)L.pos, nl, c->d_err, st);
+      launch_mac_planes(c->V, std::min(c->batch_requests, na - q0), planes + q0, S.planes(c->npl), Hs + q0, c->ell,
+                        (int)L.pos, nl, c->d_err, st);
     }
   } else {
     const u64* P = L.b.Pc;
@@ -466,13 +459,8 @@ int pepsi_engine_create(const pepsi_lane* lanes, int nlanes, uint64_t hbm_budget
     L.nslots = (int)lanes[i].slots;
     L.Lc = balanced_chunk(L.c->chunk, L.mu);
     err = eval_bufs(L.c, L.Lc, L.mu_res < L.mu, &L.b);
-    {  // scratch of the request's preparation, before any capture: NTT words, or byte planes
-      const size_t kN = (size_t)L.c->k * L.c->N;
-      if (in_planes(L))
-        scratch(L.c, S_CW, (size_t)L.c->ell * 2 * kN * 8, &err);
-      else if (L.mu_res && !S.words)
-        scratch(L.c, S_CP, request_plane_words(L.c->ell, kN) * 8, &err);
-    }
+    if (!reads_words(L))  // the NTT words that byte planes are made from, before any capture
+      scratch(L.c, S_CW, (size_t)L.c->ell * 2 * L.c->k * L.c->N * 8, &err);
     if (err == cudaSuccess) err = cudaHostAlloc((void**)&L.err_ring, (kStepsAhead + 1) * sizeof(int), 0);
     if (err == cudaSuccess) memset(L.err_ring, 0, (kStepsAhead + 1) * sizeof(int));
     if (err != cudaSuccess) rc = cuda_status(err);
