@@ -279,11 +279,16 @@ int pepsi_query(pepsi_ctx* ctx, const uint64_t* items, size_t m, uint64_t enc_se
  * the response is switched); ciphertext (j, i) of the response answers
  * client batch i of request block j, its mask drawn from
  * mask_seed + j * gamma + i.  With gamma > 1 the batches of a block are
- * evaluated as by pepsi_eval_batch (shared multiply-accumulates).  A host request of 128 code bits or more is uploaded in two pieces of its
- * bits (the first short), the copy of the second overlapping the first piece's
- * transform and multiply-accumulate; the words do not depend on it.  Device
- * buffers need 8-byte alignment (16-byte aligned rows take wider accesses).
- * Errors: PEPSI_E_PARAM (bad set/mode), PEPSI_E_NOMEM, PEPSI_E_CUDA. */
+ * evaluated as by pepsi_eval_batch (shared multiply-accumulates).  A host
+ * request of 128 code bits or more against a table in byte planes is uploaded
+ * in two pieces of its bits (the first short), the copy of the second overlapping
+ * the first piece's transform and multiply-accumulate; the words do not depend
+ * on it.  Device buffers need 8-byte alignment (16-byte aligned rows take wider
+ * accesses).  With device outputs the call returns before its work is done: a
+ * bounded wait that expires then is reported by the context's next evaluation
+ * with host outputs, or by pepsi_wait_probe(ctx, 1) once the work is done.
+ * Errors: PEPSI_E_PARAM (bad set/mode), PEPSI_E_NOMEM, PEPSI_E_CUDA,
+ * PEPSI_E_TIMEOUT. */
 int pepsi_eval(pepsi_ctx* ctx, int set_id, const uint64_t* cts, int mode, uint64_t mask_seed, uint64_t* out_ct,
                void* stream);
 
