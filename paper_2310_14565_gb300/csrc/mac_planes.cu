@@ -183,8 +183,8 @@ struct Tile {
 // about 560 cycles of serial address work: one request took 12.1 ms instead of
 // 11.1 ms at the paper shape, four requests and 48 layers 3.1 ms instead of 2.7.)
 // Every wait is bounded (about one second); on expiry the warp goes on to
-// where it can stop, waits, again bounded, for its copies in flight, sets *err
-// and returns.
+// where it can stop, sets *err and returns.  The producers wait, again bounded, for
+// the last copies of their teams before they return.
 // SHORT: at most DRAIN steps, so the integer sums are read once.
 template <int NPL, int KS, bool SHORT>
 __global__ void __launch_bounds__(macp::threads(SHORT), 1) k_mac_planes(DevView V, const __grid_constant__ PlaneArgs A) {
@@ -285,16 +285,15 @@ __global__ void __launch_bounds__(macp::threads(SHORT), 1) k_mac_planes(DevView 
         ++round;
       }
     }
-    if (!ok) {
-      // copies still in flight are among the last nst stages issued to each team
+    // Copies still in flight are among the last nst stages issued to each team: none
+    // may land after the block has ended, also where a consumer's wait expired.
 #pragma unroll
-      for (int u = 0; u < TEAMS_PER_PRODUCER; ++u)
-        for (int b = 0; b < filled[u]; ++b) {
-          const int n = last_slot[u] - b;
-          mbar_wait_bounded(full(p + u * PRODUCERS, n % nst), (u32)(n / nst) & 1);
-        }
-      if (lane == 0) atomicExch(A.err, 1);
-    }
+    for (int u = 0; u < TEAMS_PER_PRODUCER; ++u)
+      for (int b = 0; b < filled[u]; ++b) {
+        const int n = last_slot[u] - b;
+        ok &= mbar_wait_bounded(full(p + u * PRODUCERS, n % nst), (u32)(n / nst) & 1);
+      }
+    if (!ok && lane == 0) atomicExch(A.err, 1);
     return;
   }
 
