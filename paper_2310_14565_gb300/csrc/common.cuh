@@ -134,7 +134,8 @@ struct PmMul {
     const u64 L = (u64)(u32)x * c, M = (u64)(u32)(x >> 32) * c + (L >> 32);
     return (u64)(u32)(M >> n32) * d + ((u64)((u32)M & nmask) << 32 | (u32)L);
   }
-  // x < 2^(n+5) -> [0, 2^n + 2^29) with x = x1 2^n + x0: x0 + x1 d
+  // x < 2^(n+5) -> [0, 2^n + 2^32) with x = x1 2^n + x0: x0 + x1 d, x1 < 32, d < 2^27
+  // (and x1 d < q, so one subtraction reduces it)
   __device__ __forceinline__ u64 fold(u64 x) const {
     const u32 h = (u32)(x >> 32);
     return ((u64)(h & nmask) << 32 | (u32)x) + (h >> n32) * d;
@@ -174,8 +175,9 @@ __device__ __forceinline__ u64 addmod(u64 a, u64 b, u64 q) {
 }
 __device__ __forceinline__ u64 submod(u64 a, u64 b, u64 q) { return a >= b ? a - b : a + q - b; }
 // (hi:lo) < 2^(2n+5) mod q = 2^n - d (a sum of up to 32 products of residues): two
-// folds, three wide products against the six or so of Barrett's.  d < 2^(n/2 - 4)
-// (the condition of pm), so the second fold's product stays below 2^(n-3).
+// folds, three wide products against the six or so of Barrett's.  The condition of
+// pm, 2^(s+1) d < 2^n with s >= (n + 5) / 2, gives d < 2^((n-7)/2), so the second fold's
+// product, below 2^5 d^2, stays below 2^(n-2).
 __device__ __forceinline__ u64 pm_reduce(u64 hi, u64 lo, const PmMul& m, int n) {
   const u64 h = hi << (64 - n) | lo >> n;
   const u64 low = (u64)((u32)(lo >> 32) & m.nmask) << 32 | (u32)lo;

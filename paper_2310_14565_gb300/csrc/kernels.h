@@ -51,7 +51,7 @@ struct PlaneTab {
 };
 inline int plane_steps(int ell) { return (ell + 15) / 16; }
 inline size_t plane_layer_bytes(int ell, size_t kN, int npl) { return (size_t)plane_steps(ell) * kN * 16 * npl; }
-// Whether a resident table is kept in byte planes, else as 64-bit words: short
+// Whether a resident table is faster in byte planes than as 64-bit words: short
 // codes do not pay for the padding to steps of 16 bits and for the sums and
 // reductions of an item (a point and 16 layers), about the time of 16 bits.
 // Multiply-accumulate of 512 layers, planes against words: 7 planes, N = 8192, k = 4:

@@ -6,9 +6,11 @@
 
 // Threads of a block running the register-blocked NTT: one per two groups of 8
 // elements from N = 4096 on (N = 4096, 1200 x 3 rows: 137 us with 256 threads, 147
-// us with 128 or 512; N = 16384, 256 x 8 rows: 301 us with 1024, 321 us with 512; N =
-// 8192 alone is as fast with 256 as with 512, but the relinearisation's transforms
-// of 59 layers took 3.43 ms an evaluation with 256 and 3.25 ms with 512).
+// us with 128 or 512; N = 16384, 256 x 8 rows: 301 us with 1024, 321 us with 512).  N =
+// 8192 takes 512 as the better one over the set sizes (h = 8, 526 layers: 12.28 ms an
+// evaluation, 12.48 with 256; 74 layers: even), although 256 wins where much of the
+// time is relinearisation of full launches (256 products: 2.37 ms, 2.44; the paper
+// shape 15.91, 16.02), which the autotuner finds.
 constexpr int NTT_MAX_THREADS = 1024;
 inline int ntt_threads(int N) {
   return N >= 4096 ? N / 16 : std::max(32, N / 8);
