@@ -89,6 +89,15 @@ struct DevView {
   int allpm;                 // every ciphertext and auxiliary prime has folding products (kernels' PM forms)
   int nt;                    // threads per block of the ciphertext transforms (0: the default for N)
 };
+// The rings a transform kernel is compiled for: all, or those below N = 4096 alone.
+// The named barriers of the fused forms (N = 4096, 8192, 16384) reserve all sixteen of
+// a block's barriers, which limits the small blocks of small rings: 1500 x 4 rows of N
+// = 256 took 34 us in the kernels with the fused forms and 16 us without, N = 1024 66
+// and 51 us.  Kernels for 4096 and up alone, without the generic form, were slower by
+// up to 1 % (they spilled more).
+enum Ring { RING_ANY, RING_SMALL };
+constexpr int FUSED_LOGN = 12;
+
 
 // ---------------------------------------------------------------- arithmetic
 __device__ __forceinline__ u64 shoup_lazy(u64 x, u64 w, u64 ws, u64 q) {

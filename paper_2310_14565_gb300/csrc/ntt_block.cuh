@@ -36,6 +36,15 @@ __device__ __forceinline__ T& at(T* a, u32 nb, int c) {
   return *reinterpret_cast<T*>(reinterpret_cast<char*>(a) + (nb ^ (u32)(low * (int)sizeof(T))) + high * (int)sizeof(T));
 }
 
+// The same where c is not a constant: nsw of the sum is the shorter form.
+template <bool FIXED, class T>
+__device__ __forceinline__ T& at_phase(T* a, int base, u32 nb, int c) {
+  if constexpr (FIXED)
+    return at(a, nb, c);
+  else
+    return a[nsw(base + c)];
+}
+
 namespace nttd {
 
 // Arithmetic of a transform's modulus.  mul(x, t) multiplies by a table entry
@@ -198,7 +207,8 @@ __device__ __forceinline__ void inv_group_last(typename A::T (&x)[8], int base, 
   }
 }
 
-template <int RR, class A>
+// FIXED: N, logN and s0 are constants of the instance (at_phase).
+template <int RR, bool FIXED, class A>
 __device__ __forceinline__ void fwd_phase(u64* a, int N, int logN, int s0, const A& ar,
                                           const ulonglong2* __restrict__ tw, bool last) {
   constexpr int E = 1 << RR;
@@ -209,15 +219,15 @@ __device__ __forceinline__ void fwd_phase(u64* a, int N, int logN, int s0, const
     const u32 nb = (u32)nsw(base) * 8;
     u64 x[E];
 #pragma unroll
-    for (int i = 0; i < E; ++i) x[i] = at(a, nb, i << slog);
+    for (int i = 0; i < E; ++i) x[i] = at_phase<FIXED>(a, base, nb, i << slog);
     fwd_group<RR>(x, base, logN, s0, ar, tw);
     if (last) fwd_final<E>(x, ar);
 #pragma unroll
-    for (int i = 0; i < E; ++i) at(a, nb, i << slog) = x[i];
+    for (int i = 0; i < E; ++i) at_phase<FIXED>(a, base, nb, i << slog) = x[i];
   }
 }
 
-template <int RR, class A>
+template <int RR, bool FIXED, class A>
 __device__ __forceinline__ void inv_phase(typename A::T* a, int N, int logN, int s0, const A& ar,
                                           const ulonglong2* __restrict__ itw, bool last, const ulonglong2& ninv) {
   typedef typename A::T T;
@@ -229,11 +239,11 @@ __device__ __forceinline__ void inv_phase(typename A::T* a, int N, int logN, int
     const u32 nb = (u32)nsw(base) * (u32)sizeof(T);
     T x[E];
 #pragma unroll
-    for (int i = 0; i < E; ++i) x[i] = at(a, nb, i << slog);
+    for (int i = 0; i < E; ++i) x[i] = at_phase<FIXED>(a, base, nb, i << slog);
     inv_group<RR>(x, base, logN, s0, ar, itw);
     if (last) inv_final<E>(x, ar, ninv);
 #pragma unroll
-    for (int i = 0; i < E; ++i) at(a, nb, i << slog) = x[i];
+    for (int i = 0; i < E; ++i) at_phase<FIXED>(a, base, nb, i << slog) = x[i];
   }
 }
 
@@ -245,12 +255,12 @@ template <class A>
 __device__ __forceinline__ void ntt_fwd_block(u64* a, int N, int logN, const A& ar, const ulonglong2* __restrict__ tw) {
   int s0 = 0;
   for (; s0 + 3 <= logN; s0 += 3) {
-    nttd::fwd_phase<3>(a, N, logN, s0, ar, tw, s0 + 3 == logN);
+    nttd::fwd_phase<3, false>(a, N, logN, s0, ar, tw, s0 + 3 == logN);
     __syncthreads();
   }
   const int rem = logN - s0;
-  if (rem == 2) nttd::fwd_phase<2>(a, N, logN, s0, ar, tw, true);
-  if (rem == 1) nttd::fwd_phase<1>(a, N, logN, s0, ar, tw, true);
+  if (rem == 2) nttd::fwd_phase<2, false>(a, N, logN, s0, ar, tw, true);
+  if (rem == 1) nttd::fwd_phase<1, false>(a, N, logN, s0, ar, tw, true);
   if (rem) __syncthreads();
 }
 
@@ -261,11 +271,11 @@ __device__ __forceinline__ void ntt_inv_block(typename A::T* a, int N, int logN,
                                               const ulonglong2* __restrict__ itw, const ulonglong2& ninv) {
   const int rem = logN % 3;
   int s0 = logN - rem;
-  if (rem == 2) nttd::inv_phase<2>(a, N, logN, s0, ar, itw, s0 == 0, ninv);
-  if (rem == 1) nttd::inv_phase<1>(a, N, logN, s0, ar, itw, s0 == 0, ninv);
+  if (rem == 2) nttd::inv_phase<2, false>(a, N, logN, s0, ar, itw, s0 == 0, ninv);
+  if (rem == 1) nttd::inv_phase<1, false>(a, N, logN, s0, ar, itw, s0 == 0, ninv);
   if (rem) __syncthreads();
   for (s0 -= 3; s0 >= 0; s0 -= 3) {
-    nttd::inv_phase<3>(a, N, logN, s0, ar, itw, s0 == 0, ninv);
+    nttd::inv_phase<3, false>(a, N, logN, s0, ar, itw, s0 == 0, ninv);
     __syncthreads();
   }
 }
@@ -420,7 +430,7 @@ __device__ __forceinline__ void ntt_fwd_fused(u64* a, const Load& ld, const Stor
   __syncthreads();
 #pragma unroll
   for (int m = 0; m < M; ++m) {
-    nttd::fwd_phase<3>(a, N, LOGN, 3 + 3 * m, ar, tw, false);
+    nttd::fwd_phase<3, true>(a, N, LOGN, 3 + 3 * m, ar, tw, false);
     if (m == 0)
       part_sync<LOGN>();
     else
@@ -460,7 +470,7 @@ __device__ __forceinline__ void ntt_inv_fused(typename A::T* a, const Load& ld, 
   __syncwarp();
 #pragma unroll
   for (int m = M - 1; m >= 0; --m) {
-    nttd::inv_phase<3>(a, N, LOGN, 3 + 3 * m, ar, itw, false, ninv);
+    nttd::inv_phase<3, true>(a, N, LOGN, 3 + 3 * m, ar, itw, false, ninv);
     if (m > 1)
       __syncwarp();
     else if (m == 1)
@@ -482,28 +492,32 @@ __device__ __forceinline__ void ntt_inv_fused(typename A::T* a, const Load& ld, 
 // Global-to-global transforms of row pi with the fused forms for the ring
 // sizes of the workloads (N = 4096, 8192, 16384), else load, block
 // transform and store; each in the arithmetic of the row's prime.
-template <class A, class Load, class Store>
+template <int RING, class A, class Load, class Store>
 __device__ __forceinline__ void ntt_fwd_with(u64* a, const Load& ld, const Store& st, const A& ar, int N, int logN,
                                              const ulonglong2* __restrict__ tw) {
-  switch (logN) {
-    case 12: ntt_fwd_fused<12>(a, ld, st, ar, tw); return;
-    case 13: ntt_fwd_fused<13>(a, ld, st, ar, tw); return;
-    case 14: ntt_fwd_fused<14>(a, ld, st, ar, tw); return;
-    default: break;
+  if constexpr (RING != RING_SMALL) {
+    switch (logN) {
+      case 12: ntt_fwd_fused<12>(a, ld, st, ar, tw); return;
+      case 13: ntt_fwd_fused<13>(a, ld, st, ar, tw); return;
+      case 14: ntt_fwd_fused<14>(a, ld, st, ar, tw); return;
+      default: break;
+    }
   }
   for (int x = threadIdx.x; x < N; x += blockDim.x) a[nsw(x)] = ld(x);
   __syncthreads();
   ntt_fwd_block(a, N, logN, ar, tw);
   for (int x = threadIdx.x; x < N; x += blockDim.x) st(x, a[nsw(x)]);
 }
-template <class A, class Load, class Store>
+template <int RING, class A, class Load, class Store>
 __device__ __forceinline__ void ntt_inv_with(typename A::T* a, const Load& ld, const Store& st, const A& ar, int N,
                                              int logN, const ulonglong2* __restrict__ itw, const ulonglong2& ninv) {
-  switch (logN) {
-    case 12: ntt_inv_fused<12>(a, ld, st, ar, itw, ninv); return;
-    case 13: ntt_inv_fused<13>(a, ld, st, ar, itw, ninv); return;
-    case 14: ntt_inv_fused<14>(a, ld, st, ar, itw, ninv); return;
-    default: break;
+  if constexpr (RING != RING_SMALL) {
+    switch (logN) {
+      case 12: ntt_inv_fused<12>(a, ld, st, ar, itw, ninv); return;
+      case 13: ntt_inv_fused<13>(a, ld, st, ar, itw, ninv); return;
+      case 14: ntt_inv_fused<14>(a, ld, st, ar, itw, ninv); return;
+      default: break;
+    }
   }
   for (int x = threadIdx.x; x < N; x += blockDim.x) a[nsw(x)] = ld(x);
   __syncthreads();
@@ -513,32 +527,33 @@ __device__ __forceinline__ void ntt_inv_with(typename A::T* a, const Load& ld, c
 // PM: every prime the kernel meets has folding products (DevView::allpm).  The
 // kernels come in both forms: with the other arithmetics compiled in beside it,
 // the compiler moved so much out of the branches that the inverse kernels spilled
-// (k_tensor_intt 788 bytes); 1200 x 4 rows of N = 8192 forward 281 -> 269 us, the
+// more (k_tensor_intt 788 bytes against 664, k_relin_axpy_intt 420 against 296,
+// k_axpy_intt 140 against 72); 1200 x 4 rows of N = 8192 forward 281 -> 269 us, the
 // products of 256 ciphertexts 2.39 -> 2.33 ms.
-template <bool PM = false, class Load, class Store>
+template <bool PM = false, int RING = RING_ANY, class Load, class Store>
 __device__ __forceinline__ void ntt_fwd_gg(u64* a, const Load& ld, const Store& st, const DevView& V, int pi) {
   const ulonglong2* tw = V.twp + (size_t)pi * V.N;
   const DevPrime P = V.pr[pi];
   if constexpr (PM)
-    ntt_fwd_with(a, ld, st, nttd::Pm(P), V.N, V.logN, tw);
+    ntt_fwd_with<RING>(a, ld, st, nttd::Pm(P), V.N, V.logN, tw);
   else if (P.pm)
-    ntt_fwd_with(a, ld, st, nttd::Pm(P), V.N, V.logN, tw);
+    ntt_fwd_with<RING>(a, ld, st, nttd::Pm(P), V.N, V.logN, tw);
   else if (P.q < (1ull << 59))
-    ntt_fwd_with(a, ld, st, nttd::Shoup<true>(P), V.N, V.logN, tw);
+    ntt_fwd_with<RING>(a, ld, st, nttd::Shoup<true>(P), V.N, V.logN, tw);
   else
-    ntt_fwd_with(a, ld, st, nttd::Shoup<false>(P), V.N, V.logN, tw);
+    ntt_fwd_with<RING>(a, ld, st, nttd::Shoup<false>(P), V.N, V.logN, tw);
 }
-template <bool PM = false, class Load, class Store>
+template <bool PM = false, int RING = RING_ANY, class Load, class Store>
 __device__ __forceinline__ void ntt_inv_gg(u64* a, const Load& ld, const Store& st, const DevView& V, int pi) {
   const ulonglong2* itw = V.itwp + (size_t)pi * V.N;
   const DevPrime P = V.pr[pi];
   const ulonglong2 ninv = make_ulonglong2(P.ninv, P.ninvs);
   if constexpr (PM)
-    ntt_inv_with(a, ld, st, nttd::Pm(P), V.N, V.logN, itw, ninv);
+    ntt_inv_with<RING>(a, ld, st, nttd::Pm(P), V.N, V.logN, itw, ninv);
   else if (P.pm)
-    ntt_inv_with(a, ld, st, nttd::Pm(P), V.N, V.logN, itw, ninv);
+    ntt_inv_with<RING>(a, ld, st, nttd::Pm(P), V.N, V.logN, itw, ninv);
   else
-    ntt_inv_with(a, ld, st, nttd::Shoup<false>(P), V.N, V.logN, itw, ninv);
+    ntt_inv_with<RING>(a, ld, st, nttd::Shoup<false>(P), V.N, V.logN, itw, ninv);
 }
 
 // ntt_inv_gg for a modulus q_pi below 2^30 (the plaintext modulus) in 32-bit
@@ -547,5 +562,5 @@ __device__ __forceinline__ void ntt_inv_gg(u64* a, const Load& ld, const Store& 
 template <class Load, class Store>
 __device__ __forceinline__ void ntt_inv_gg_small(u32* a, const Load& ld, const Store& st, const DevView& V, int pi) {
   const DevPrime P = V.pr[pi];
-  ntt_inv_with(a, ld, st, nttd::Small(P), V.N, V.logN, V.itwp + (size_t)pi * V.N, make_ulonglong2(P.ninv, P.ninvs));
+  ntt_inv_with<RING_ANY>(a, ld, st, nttd::Small(P), V.N, V.logN, V.itwp + (size_t)pi * V.N, make_ulonglong2(P.ninv, P.ninvs));
 }

@@ -20,7 +20,7 @@ constexpr int relin_min_blocks(int MT) { return MT <= 256 ? 3 : 1; }
 // Phase 1, block per row of DG[L][k+2][k][N]: row (l, i, j) holds
 // NTT_{q_j}([d2]_{q_i}) for digits i < k, and NTT_{q_j}(d0), NTT_{q_j}(d1)
 // for i = k, k+1.
-template <int MT, bool PM>
+template <int MT, bool PM, int RING>
 __global__ void __launch_bounds__(MT, relin_min_blocks(MT)) k_relin_ntt(DevView V, const u64* __restrict__ D, u64* __restrict__ DG) {
   extern __shared__ u64 sm[];
   const int N = V.N, k = V.k;
@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(MT, relin_min_blocks(MT)) k_relin_ntt(DevView 
   const DevPrime pj = V.pr[j];
   const u64* row = i < k ? D + ((l * 3 + 2) * k + i) * N : D + ((l * 3 + (i - k)) * k + j) * N;
   u64* out = DG + r * N;
-  ntt_fwd_gg<PM>(
+  ntt_fwd_gg<PM, RING>(
       sm,
       [&](int x) {
         const u64 w = row[x];
@@ -69,7 +69,7 @@ __global__ void k_relin_mac(DevView V, const u64* __restrict__ DG, const u64* __
 // and u = R_c + z * H on the load of the inverse NTT of U, stores u and the
 // coefficient-form row.  The same words as k_relin_mac followed by
 // k_axpy_intt, without R in memory.
-template <int MT, bool PM>
+template <int MT, bool PM, int RING>
 __global__ void __launch_bounds__(MT, relin_min_blocks(MT))
     k_relin_axpy_intt(DevView V, const u64* __restrict__ DG, const u64* __restrict__ rlk,
                       const u64* __restrict__ zres, const u64* __restrict__ H, u64* __restrict__ out, u64* coef) {
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(MT, relin_min_blocks(MT))
   const u64* key = rlk + ((size_t)c * k + p) * N;  // rlk_i[c] at prime p: key + i * 2 * gs
   const u64* hr = H + r * N;
   u64* ur = out + r * N;
-  ntt_inv_gg<PM>(
+  ntt_inv_gg<PM, RING>(
       sm,
       [&](int x) {
         u64 lo = g[(size_t)(k + c) * gs + x], hi = 0;
@@ -114,10 +114,14 @@ void launch_relin_digits(const DevView& V, const u64* D, u64* DG, int L, cudaStr
   const size_t rows = (size_t)L * (V.k + 2) * V.k;
   const int nt = xform_threads(V, rows);
   auto go = [&](auto kernel) { kernel<<<(unsigned)rows, nt, (size_t)V.N * 8, st>>>(V, D, DG); };
-  if (nt <= 256)
-    V.allpm ? go(k_relin_ntt<256, true>) : go(k_relin_ntt<256, false>);
-  else
-    V.allpm ? go(k_relin_ntt<NTT_MAX_THREADS, true>) : go(k_relin_ntt<NTT_MAX_THREADS, false>);
+  in_form(V, [&](auto pm, auto ring) {
+    constexpr bool PM = decltype(pm)::value;
+    constexpr int RING = decltype(ring)::value;
+    if (nt <= 256)
+      go(k_relin_ntt<256, PM, RING>);
+    else
+      go(k_relin_ntt<NTT_MAX_THREADS, PM, RING>);
+  });
 }
 
 void launch_relin(const DevView& V, const u64* D, const u64* rlk, u64* DG, u64* R, int L, cudaStream_t st) {
@@ -134,16 +138,23 @@ void launch_relin_axpy_intt(const DevView& V, const u64* DG, const u64* rlk, con
   auto go = [&](auto kernel) {
     kernel<<<(unsigned)rows, nt, (size_t)V.N * 8, st>>>(V, DG, rlk, zres, H, out, coef);
   };
-  if (nt <= 256)
-    V.allpm ? go(k_relin_axpy_intt<256, true>) : go(k_relin_axpy_intt<256, false>);
-  else
-    V.allpm ? go(k_relin_axpy_intt<NTT_MAX_THREADS, true>) : go(k_relin_axpy_intt<NTT_MAX_THREADS, false>);
+  in_form(V, [&](auto pm, auto ring) {
+    constexpr bool PM = decltype(pm)::value;
+    constexpr int RING = decltype(ring)::value;
+    if (nt <= 256)
+      go(k_relin_axpy_intt<256, PM, RING>);
+    else
+      go(k_relin_axpy_intt<NTT_MAX_THREADS, PM, RING>);
+  });
 }
 
 cudaError_t relin_init() {
-  return allow_smem({(const void*)k_relin_ntt<256, true>, (const void*)k_relin_ntt<NTT_MAX_THREADS, true>,
-                     (const void*)k_relin_axpy_intt<256, true>, (const void*)k_relin_axpy_intt<NTT_MAX_THREADS, true>,
-                     (const void*)k_relin_ntt<256, false>, (const void*)k_relin_ntt<NTT_MAX_THREADS, false>,
-                     (const void*)k_relin_axpy_intt<256, false>,
-                     (const void*)k_relin_axpy_intt<NTT_MAX_THREADS, false>});
+  return allow_smem({(const void*)k_relin_ntt<256, true, RING_ANY>,
+                     (const void*)k_relin_ntt<NTT_MAX_THREADS, true, RING_ANY>,
+                     (const void*)k_relin_axpy_intt<256, true, RING_ANY>,
+                     (const void*)k_relin_axpy_intt<NTT_MAX_THREADS, true, RING_ANY>,
+                     (const void*)k_relin_ntt<256, false, RING_ANY>,
+                     (const void*)k_relin_ntt<NTT_MAX_THREADS, false, RING_ANY>,
+                     (const void*)k_relin_axpy_intt<256, false, RING_ANY>,
+                     (const void*)k_relin_axpy_intt<NTT_MAX_THREADS, false, RING_ANY>});
 }

@@ -27,9 +27,10 @@ __device__ __forceinline__ u64 prod(u64 a, u64 b, const DevPrime& p) {
 // (A_l, B_l) at prime pi on the load of the inverse NTT, and stores the
 // coefficient-form row: the tensor (a0b0, a0b1 + a1b0, a1b1) and its
 // inverse NTT without a round trip of the NTT-form tensor through memory.
-// Bound by the heavy multiply-add pipe; compiled for folding primes alone the
-// inverse stages do not spill (256 ciphertexts of N = 8192, k = 4: 0.56 ms).
-template <bool PM>
+// Bound by the heavy multiply-add pipe (256 ciphertexts of N = 8192, k = 4: 0.56 ms).
+// Its six loads beside the transforms of four ring forms spill at 64 registers: 664
+// bytes compiled for folding primes alone, 788 with the other arithmetics in it.
+template <bool PM, int RING>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1)
     k_tensor_intt(DevView V, const u64* __restrict__ AQ, const u64* __restrict__ AB, const u64* __restrict__ BQ,
                   const u64* __restrict__ BB, const u64* __restrict__ cstQ, const u64* __restrict__ side,
@@ -65,9 +66,9 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1)
   const RowSt st(T3 + r * N);
   if (square) {
     if (c == 0)
-      ntt_inv_gg<PM>(sm, [&](int x) { return prod<PM>(a0[x], a0[x], pr); }, st, V, pi);
+      ntt_inv_gg<PM, RING>(sm, [&](int x) { return prod<PM>(a0[x], a0[x], pr); }, st, V, pi);
     else if (c == 1)
-      ntt_inv_gg<PM>(
+      ntt_inv_gg<PM, RING>(
           sm,
           [&](int x) {
             const u64 m = prod<PM>(a0[x], a1[x], pr);
@@ -75,12 +76,12 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1)
           },
           st, V, pi);
     else
-      ntt_inv_gg<PM>(sm, [&](int x) { return prod<PM>(a1[x], a1[x], pr); }, st, V, pi);
+      ntt_inv_gg<PM, RING>(sm, [&](int x) { return prod<PM>(a1[x], a1[x], pr); }, st, V, pi);
   } else {
     if (c == 0)
-      ntt_inv_gg<PM>(sm, [&](int x) { return prod<PM>(a0[x], addmod(b0[x], cb, pr.q), pr); }, st, V, pi);
+      ntt_inv_gg<PM, RING>(sm, [&](int x) { return prod<PM>(a0[x], addmod(b0[x], cb, pr.q), pr); }, st, V, pi);
     else if (c == 1)
-      ntt_inv_gg<PM>(
+      ntt_inv_gg<PM, RING>(
           sm,
           [&](int x) {
             u64 lo = 0, hi = 0;
@@ -90,7 +91,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1)
           },
           st, V, pi);
     else
-      ntt_inv_gg<PM>(sm, [&](int x) { return prod<PM>(a1[x], b1[x], pr); }, st, V, pi);
+      ntt_inv_gg<PM, RING>(sm, [&](int x) { return prod<PM>(a1[x], b1[x], pr); }, st, V, pi);
   }
 }
 
@@ -192,7 +193,7 @@ void launch_tensor_intt(const DevView& V, const u64* AQ, const u64* AB, const u6
     kernel<<<(unsigned)rows, xform_threads(V, rows), (size_t)V.N * 8, st>>>(V, AQ, AB, BQ, BB, cstQ, side, T3,
                                                                           square ? 1 : 0);
   };
-  V.allpm ? go(k_tensor_intt<true>) : go(k_tensor_intt<false>);
+  in_form(V, [&](auto pm, auto ring) { go(k_tensor_intt<decltype(pm)::value, decltype(ring)::value>); });
 }
 
 void launch_tensor_sum(const DevView& V, const u64* AQ, const u64* AB, const u64* BQ, const u64* BB,
@@ -203,4 +204,6 @@ void launch_tensor_sum(const DevView& V, const u64* AQ, const u64* AB, const u64
                                                                           square ? 1 : 0, init ? 1 : 0);
 }
 
-cudaError_t tensor_init() { return allow_smem({(const void*)k_tensor_intt<true>, (const void*)k_tensor_intt<false>}); }
+cudaError_t tensor_init() {
+  return allow_smem({(const void*)k_tensor_intt<true, RING_ANY>, (const void*)k_tensor_intt<false, RING_ANY>});
+}

@@ -13,7 +13,7 @@ namespace {
 // 269 us compiled for folding alone.
 // SPLIT: store the result in the split operand format of the
 // multiply-accumulate (the request's forward transform).
-template <bool PM, bool FWD, bool SPLIT = false>
+template <bool PM, int RING, bool FWD, bool SPLIT = false>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ntt(DevView V, const u64* __restrict__ src, u64* dst, int np, int p0, size_t src_os,
                       size_t dst_os, u32* sums) {
   extern __shared__ u64 sm[];
@@ -26,11 +26,11 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ntt(DevView V, const u64
   const RowLd ld(s);
   if (FWD) {
     if (SPLIT)
-      ntt_fwd_gg<PM>(sm, ld, SplitSumSt(d, sums + o * dst_os + (size_t)pl * N, V.pr[p0 + pl].split), V, p0 + pl);
+      ntt_fwd_gg<PM, RING>(sm, ld, SplitSumSt(d, sums + o * dst_os + (size_t)pl * N, V.pr[p0 + pl].split), V, p0 + pl);
     else
-      ntt_fwd_gg<PM>(sm, ld, RowSt(d), V, p0 + pl);
+      ntt_fwd_gg<PM, RING>(sm, ld, RowSt(d), V, p0 + pl);
   } else {
-    ntt_inv_gg<PM>(sm, ld, RowSt(d), V, p0 + pl);
+    ntt_inv_gg<PM, RING>(sm, ld, RowSt(d), V, p0 + pl);
   }
 }
 
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ntt(DevView V, const u64
 // row on the transform's load and also stores it (each element is loaded
 // once).  coef may alias b: a block reads its row of b before it writes
 // that row of coef.
-template <bool PM>
+template <bool PM, int RING>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1)
     k_axpy_intt(DevView V, const u64* __restrict__ a, const u64* __restrict__ zres, const u64* b, u64* __restrict__ out,
                 u64* coef) {
@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1)
   const u64* br = b + r * N;
   u64* ur = out + r * N;
   u64* cr = coef + r * N;
-  ntt_inv_gg<PM>(
+  ntt_inv_gg<PM, RING>(
       sm,
       [&](int x) {
         const u64 u = addmod(ar[x], mulmod(z, br[x], pr), pr.q);
@@ -73,12 +73,16 @@ void launch_ntt(const DevView& V, bool fwd, const u64* src, u64* dst, size_t out
     kernel<<<(unsigned)rows, xform_threads(V, rows), (size_t)V.N * sizeof(u64), st>>>(V, src, dst, np, p0, src_os, dst_os,
                                                                                     sums);
   };
-  if (fwd && split_out)
-    V.allpm ? go(k_ntt<true, true, true>) : go(k_ntt<false, true, true>);
-  else if (fwd)
-    V.allpm ? go(k_ntt<true, true>) : go(k_ntt<false, true>);
-  else
-    V.allpm ? go(k_ntt<true, false>) : go(k_ntt<false, false>);
+  in_form(V, [&](auto pm, auto ring) {
+    constexpr bool PM = decltype(pm)::value;
+    constexpr int RING = decltype(ring)::value;
+    if (fwd && split_out)
+      go(k_ntt<PM, RING, true, true>);
+    else if (fwd)
+      go(k_ntt<PM, RING, true>);
+    else
+      go(k_ntt<PM, RING, false>);
+  });
 }
 
 void launch_axpy_intt(const DevView& V, const u64* a, const u64* zres, const u64* b, u64* out, u64* coef,
@@ -88,12 +92,13 @@ void launch_axpy_intt(const DevView& V, const u64* a, const u64* zres, const u64
   auto go = [&](auto kernel) {
     kernel<<<(unsigned)rows, xform_threads(V, rows), (size_t)V.N * 8, st>>>(V, a, zres, b, out, coef);
   };
-  V.allpm ? go(k_axpy_intt<true>) : go(k_axpy_intt<false>);
+  in_form(V, [&](auto pm, auto ring) { go(k_axpy_intt<decltype(pm)::value, decltype(ring)::value>); });
 }
 
 cudaError_t transforms_init() {
-  return allow_smem({(const void*)k_ntt<true, true>, (const void*)k_ntt<true, false>,
-                     (const void*)k_ntt<true, true, true>, (const void*)k_ntt<false, true>,
-                     (const void*)k_ntt<false, false>, (const void*)k_ntt<false, true, true>,
-                     (const void*)k_axpy_intt<true>, (const void*)k_axpy_intt<false>});
+  // (rings below 4096 stay within the default limit)
+  return allow_smem({(const void*)k_ntt<true, RING_ANY, true>, (const void*)k_ntt<true, RING_ANY, false>,
+                     (const void*)k_ntt<true, RING_ANY, true, true>, (const void*)k_ntt<false, RING_ANY, true>,
+                     (const void*)k_ntt<false, RING_ANY, false>, (const void*)k_ntt<false, RING_ANY, true, true>,
+                     (const void*)k_axpy_intt<true, RING_ANY>, (const void*)k_axpy_intt<false, RING_ANY>});
 }

@@ -1,6 +1,7 @@
 // Launch shapes shared by the transform kernels.
 #pragma once
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -32,6 +33,18 @@ inline int xform_threads(const DevView& V, size_t rows) {
   const int base = xform_threads(V);
   const int wide = latency_threads(V.N);
   return rows <= (size_t)sm_count() && wide > base ? wide : base;
+}
+// A launch in the form for the context's primes and ring: f(PM, RING), as constants.
+template <class F>
+void in_form(const DevView& V, const F& f) {
+  typedef std::bool_constant<true> yes;
+  typedef std::bool_constant<false> no;
+  typedef std::integral_constant<int, RING_ANY> any;
+  typedef std::integral_constant<int, RING_SMALL> small;
+  if (V.logN >= FUSED_LOGN)
+    V.allpm ? f(yes(), any()) : f(no(), any());
+  else
+    V.allpm ? f(yes(), small()) : f(no(), small());
 }
 inline unsigned grid_for(size_t total, int threads) { return (unsigned)((total + threads - 1) / threads); }
 // Let a kernel use all the dynamic shared memory a block may hold beside its static.
