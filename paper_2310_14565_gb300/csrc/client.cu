@@ -106,12 +106,12 @@ __device__ __forceinline__ u64 sample_mod(u64 key, u64 pos, const DevPrime& p) {
 }
 // Encode: inverse transform modulo t of ld (a slot value below t per position)
 // into m[], in 32-bit words for t below 2^30.  a: N words of scratch.
-template <class Load>
+template <int RING, class Load>
 __device__ __forceinline__ void encode_block(u64* a, const Load& ld, u32* m, const DevView& V) {
   if (V.pr[V.tidx].q < (1ull << 30))
-    ntt_inv_gg_small(reinterpret_cast<u32*>(a), ld, [&](int i, u32 v) { m[i] = v; }, V, V.tidx);
+    ntt_inv_gg_small<RING>(reinterpret_cast<u32*>(a), ld, [&](int i, u32 v) { m[i] = v; }, V, V.tidx);
   else
-    ntt_inv_gg(a, [&](int i) -> u64 { return ld(i); }, [&](int i, u64 v) { m[i] = (u32)v; }, V, V.tidx);
+    ntt_inv_gg<false, RING>(a, [&](int i) -> u64 { return ld(i); }, [&](int i, u64 v) { m[i] = (u32)v; }, V, V.tidx);
   __syncthreads();
 }
 
@@ -119,7 +119,7 @@ __device__ __forceinline__ void encode_block(u64* a, const Load& ld, u32* m, con
 // Block (layer l, j-chunk): bit planes of the layer's codewords, encoded
 // (inverse NTT mod t of the slot vector in bit-reversed order), centred
 // lift into each q_p and forward NTT; stored in the split operand format.
-template <bool PM>
+template <bool PM, int RING>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ptgen(DevView V, const uint16_t* __restrict__ pos, int ell, int h, int JC, u64* P) {
   extern __shared__ u64 sm[];
   const int N = V.N, k = V.k;
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ptgen(DevView V, const u
     if (j >= ell) break;
     // Encode: slot s at position brev(s), inverse NTT mod t into mbuf
     const u32* bj = bits + jj * words;
-    encode_block(
+    encode_block<RING>(
         poly,
         [&](int i) -> u32 {
           const u32 s = brev_bits(i, V.logN);
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_ptgen(DevView V, const u
       // centred lift to q_p on the load, split operand format on the store
       const u64 q = V.pr[p].q, sp = V.pr[p].split;
       u64* out = P + (((size_t)l * ell + j) * k + p) * N;
-      ntt_fwd_gg<PM>(
+      ntt_fwd_gg<PM, RING>(
           poly,
           [&](int i) -> u64 {
             const u64 m = mbuf[i];
@@ -207,7 +207,7 @@ __device__ __forceinline__ u64 smod_dev(i64 v, u64 q) { return v >= 0 ? (u64)v :
 
 // Block per ciphertext j: encode bit plane j, then for each prime sample
 // a, compute c0 = e - a s + round(Q m / t), c1 = a (coefficient form).
-template <bool PM>
+template <bool PM, int RING>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_encrypt(DevView V, const uint16_t* __restrict__ pos, int h, const u64* __restrict__ s_ntt, u64 seed,
                           u64 idx0, u64* cts) {
   extern __shared__ u64 sm[];
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_encrypt(DevView V, const
   u64* poly = sm;
   u32* mbuf = reinterpret_cast<u32*>(sm + N);
   const DevPrime t = V.pr[V.tidx];
-  encode_block(
+  encode_block<RING>(
       poly,
       [&](int i) -> u32 {
         const uint16_t* ps = pos + (size_t)brev_bits(i, V.logN) * h;
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_encrypt(DevView V, const
     const u64* sr = s_ntt + (size_t)p * N;
     // a, its transform times s left in place, and back: every thread's last
     // elements of the first transform are its first of the second
-    ntt_fwd_gg<PM>(
+    ntt_fwd_gg<PM, RING>(
         poly,
         [&](int i) {
           const u64 a = sample_mod(key_a, i, pq);
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_encrypt(DevView V, const
           return a;
         },
         [&](int i, u64 v) { poly[nsw(i)] = mulmod(v, sr[i], pq); }, V, p);
-    ntt_inv_gg<PM>(
+    ntt_inv_gg<PM, RING>(
         poly, [&](int i) { return poly[nsw(i)]; },
         [&](int i, u64 v) {
           const u64 e = smod_dev(sample_cbd21(key_e, i), pq.q);
@@ -298,6 +298,7 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_keygen_rlk(DevView V, u6
 }
 
 // Decryption, step 1: z = c0 + c1 s per prime (coefficient form).
+template <int RING>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_dec_z(DevView V, const u64* __restrict__ ct, const u64* __restrict__ s_ntt, u64* z) {
   extern __shared__ u64 sm[];
   const int p = blockIdx.x, N = V.N, k = V.k;
@@ -305,9 +306,9 @@ __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_dec_z(DevView V, const u
   const u64* c1 = ct + ((size_t)k + p) * N;
   const u64 *c0 = ct + (size_t)p * N, *sr = s_ntt + (size_t)p * N;
   u64* zr = z + (size_t)p * N;
-  ntt_fwd_gg(
+  ntt_fwd_gg<false, RING>(
       sm, [&](int i) { return c1[i]; }, [&](int i, u64 v) { sm[nsw(i)] = mulmod(v, sr[i], pq); }, V, p);
-  ntt_inv_gg(
+  ntt_inv_gg<false, RING>(
       sm, [&](int i) { return sm[nsw(i)]; }, [&](int i, u64 v) { zr[i] = addmod(v, c0[i], pq.q); }, V, p);
 }
 __device__ __forceinline__ void garner_any(const RnsArgs& A, const u64* x, u64* v) {
@@ -367,9 +368,10 @@ __global__ void k_dec_coef(const __grid_constant__ RnsArgs A, DevView V, const u
   }
 }
 // Step 3: slots = values of m at psi_t^(2s+1): forward NTT mod t, slot s in position brev(s).
+template <int RING>
 __global__ void __launch_bounds__(NTT_MAX_THREADS, 1) k_dec_slots(DevView V, const u32* __restrict__ m, u32* slots) {
   extern __shared__ u64 sm[];
-  ntt_fwd_gg(
+  ntt_fwd_gg<false, RING>(
       sm, [&](int i) -> u64 { return m[i]; }, [&](int i, u64 v) { slots[brev_bits(i, V.logN)] = (u32)v; }, V, V.tidx);
 }
 
@@ -470,7 +472,7 @@ void launch_ptgen(const DevView& V, const uint16_t* pos, int L, int ell, int h, 
   const int JC = ptgen_jc(V.N);
   dim3 grid((ell + JC - 1) / JC, L);
   auto go = [&](auto kernel) { kernel<<<grid, chain_threads(V.N), ptgen_smem(V.N), st>>>(V, pos, ell, h, JC, P); };
-  V.allpm ? go(k_ptgen<true>) : go(k_ptgen<false>);
+  in_form(V, [&](auto pm, auto ring) { go(k_ptgen<decltype(pm)::value, decltype(ring)::value>); });
 }
 
 void launch_valgen(const DevView& V, const u32* vals, int L, u64* VP, cudaStream_t st) {
@@ -484,7 +486,7 @@ void launch_encrypt(const DevView& V, const uint16_t* pos, int ell, int h, const
   auto go = [&](auto kernel) {
     kernel<<<ell, chain_threads(V.N), (size_t)V.N * 12, st>>>(V, pos, h, s_ntt, seed, idx0, cts);
   };
-  V.allpm ? go(k_encrypt<true>) : go(k_encrypt<false>);
+  in_form(V, [&](auto pm, auto ring) { go(k_encrypt<decltype(pm)::value, decltype(ring)::value>); });
 }
 
 void launch_keygen(const DevView& V, u64 seed, int8_t* s, u64* s_ntt, u64* rlk, cudaStream_t st) {
@@ -502,9 +504,12 @@ void launch_modswitch(const DevView& V, const ModSwitchArgs& M, const u64* in, u
 void launch_decrypt(const DevView& V, const u64* ct, const u64* s_ntt, u64* zbuf, u32* mbuf, u32* slots,
                     unsigned long long* maxr, cudaStream_t st) {
   cudaMemsetAsync(maxr, 0, sizeof(unsigned long long), st);
-  k_dec_z<<<V.k, latency_threads(V.N), (size_t)V.N * 8, st>>>(V, ct, s_ntt, zbuf);
+  const bool small = V.logN < FUSED_LOGN;
+  auto z = small ? k_dec_z<RING_SMALL> : k_dec_z<RING_ANY>;
+  z<<<V.k, latency_threads(V.N), (size_t)V.N * 8, st>>>(V, ct, s_ntt, zbuf);
   k_dec_coef<<<grid_for(V.N, 128), 128, 0, st>>>(*V.host_args, V, zbuf, mbuf, maxr);
-  k_dec_slots<<<1, latency_threads(V.N), (size_t)V.N * 8, st>>>(V, mbuf, slots);
+  auto to_slots = small ? k_dec_slots<RING_SMALL> : k_dec_slots<RING_ANY>;
+  to_slots<<<1, latency_threads(V.N), (size_t)V.N * 8, st>>>(V, mbuf, slots);
 }
 
 void launch_mask(const DevView& V, u64 seed, u64* ct, cudaStream_t st) {
@@ -518,7 +523,9 @@ cudaError_t client_init(int N) {
   if (e != cudaSuccess) return e;
   // largest request: the plaintext generator at this N
   if ((size_t)optin < ptgen_smem(N) || (size_t)optin < (size_t)N * 12) return cudaErrorInvalidValue;
-  return allow_smem({(const void*)k_ptgen<true>, (const void*)k_ptgen<false>, (const void*)k_valgen,
-                     (const void*)k_encrypt<true>, (const void*)k_encrypt<false>, (const void*)k_keygen_sntt,
-                     (const void*)k_keygen_rlk, (const void*)k_dec_z, (const void*)k_dec_slots, (const void*)k_mask});
+  return allow_smem({(const void*)k_ptgen<true, RING_ANY>, (const void*)k_ptgen<false, RING_ANY>,
+                     (const void*)k_ptgen<true, RING_SMALL>, (const void*)k_ptgen<false, RING_SMALL>,
+                     (const void*)k_valgen, (const void*)k_encrypt<true, RING_ANY>,
+                     (const void*)k_encrypt<false, RING_ANY>, (const void*)k_keygen_sntt, (const void*)k_keygen_rlk,
+                     (const void*)k_dec_z<RING_ANY>, (const void*)k_dec_slots<RING_ANY>, (const void*)k_mask});
 }

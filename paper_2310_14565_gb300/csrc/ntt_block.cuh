@@ -527,8 +527,8 @@ __device__ __forceinline__ void ntt_inv_with(typename A::T* a, const Load& ld, c
 // PM: every prime the kernel meets has folding products (DevView::allpm).  The
 // kernels come in both forms: with the other arithmetics compiled in beside it,
 // the compiler moved so much out of the branches that the inverse kernels spilled
-// more (k_tensor_intt 788 bytes against 664, k_relin_axpy_intt 420 against 296,
-// k_axpy_intt 140 against 72); 1200 x 4 rows of N = 8192 forward 281 -> 269 us, the
+// more (k_tensor_intt 788 bytes against 664, k_relin_axpy_intt 400 against 332,
+// k_axpy_intt 136 against 72); 1200 x 4 rows of N = 8192 forward 281 -> 269 us, the
 // products of 256 ciphertexts 2.39 -> 2.33 ms.
 template <bool PM = false, int RING = RING_ANY, class Load, class Store>
 __device__ __forceinline__ void ntt_fwd_gg(u64* a, const Load& ld, const Store& st, const DevView& V, int pi) {
@@ -559,8 +559,8 @@ __device__ __forceinline__ void ntt_inv_gg(u64* a, const Load& ld, const Store& 
 // ntt_inv_gg for a modulus q_pi below 2^30 (the plaintext modulus) in 32-bit
 // words: a[] holds N 32-bit words, ld(x) returns element x in [0, 2q) as
 // u32, st(x, v) receives it reduced.  The same residues as ntt_inv_gg.
-template <class Load, class Store>
+template <int RING = RING_ANY, class Load, class Store>
 __device__ __forceinline__ void ntt_inv_gg_small(u32* a, const Load& ld, const Store& st, const DevView& V, int pi) {
   const DevPrime P = V.pr[pi];
-  ntt_inv_with<RING_ANY>(a, ld, st, nttd::Small(P), V.N, V.logN, V.itwp + (size_t)pi * V.N, make_ulonglong2(P.ninv, P.ninvs));
+  ntt_inv_with<RING>(a, ld, st, nttd::Small(P), V.N, V.logN, V.itwp + (size_t)pi * V.N, make_ulonglong2(P.ninv, P.ninvs));
 }

@@ -9,7 +9,7 @@ namespace {
 // blocks of at most 256 threads, three per SM (80 registers a thread and no spills;
 // at N = 8192 with 256-thread blocks the relinearisation took 1.98 ms against
 // 2.07 ms at 64), and MT = NTT_MAX_THREADS for larger blocks (64 registers; the sum on
-// the inverse's load spills 296 bytes).  N <= 4096 and the schedules that take 256
+// the inverse's load spills 332 bytes).  N <= 4096 and the schedules that take 256
 // threads (the autotuner's at the paper shape) run the first; the default at N = 8192
 // is 512 threads (xform.cuh).
 constexpr int relin_min_blocks(int MT) { return MT <= 256 ? 3 : 1; }
