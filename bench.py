@@ -739,19 +739,6 @@ def run_ours(args):
     bmac_rate = 6.0 * nbq * mu * ell * k * N / (bmac_ms * 1e-3) if bmac_ms else 0.0
     # on byte planes: one m16n8k16 per plane, component, request, point, 16 layers and 16 bits
     mma = 2 * pbytes * ((mu + 15) // 16) * ((ell + 15) // 16) * k * N
-    # the circuit kernels' share of the heavy multiply-add pipe: busy SM-cycles per
-    # evaluation (full-size ncu counters) over this run's CUDA-event time of the class
-    cyc = stored_pipe_cycles() if in_planes and args.rescale == "all" else None
-    circuits = None
-    if cyc:
-        clock_hz = (clk.get("sm_mhz") or 2070.0) * 1e6
-        sms = torch.cuda.get_device_properties(0).multi_processor_count
-        circuits = {}
-        for cls in ("ntt", "lift", "tensor", "scale_round", "relin", "mac"):
-            launches_c, ms_c = prof.get(cls, (0, 0.0))
-            if cls in cyc and ms_c > 0:
-                per_eval_s = ms_c / psteps * 1e-3
-                circuits[cls] = round(cyc[cls] / (per_eval_s * clock_hz * sms), 3)
     int_pipe = {"mad_wide_u32_per_s": round(wide_peak / 1e12, 3), "mul_wide_u32_per_s": round(mul_peak / 1e12, 3),
                 "mad_u32_per_s": round(mad32_peak / 1e12, 3), "unit": "T ops/s",
                 "mac_mad_wide_frac": None if in_planes else round(mac_wide_rate / wide_peak, 4),
@@ -759,11 +746,9 @@ def run_ours(args):
                 "mac_mma_tflops": round(4096 * mma / (mac_ms / psteps * 1e-3) / 1e12, 1) if in_planes else None,
                 "batched_mac_mma_tflops": (round(4096 * nbq * mma / (bmac_ms * 1e-3) / 1e12, 1)
                                            if in_planes and bmac_ms else None),
-                "circuits_heavy_pipe_busy": circuits,
                 "note": "MAC on words: 6 mad.wide.u32 per plaintext word and request (2 components x 3 Karatsuba "
-                        "split products); MAC on byte planes: f16 mma.sync.m16n8k16 on exact byte products; peaks measured with multipliers that change every step; "
-                        "circuits_heavy_pipe_busy: fraction of the SMs' heavy multiply-add pipe cycles each kernel "
-                        "class keeps busy (profiles/circuit_pipes_paper.md counters / this run's event times)"}
+                        "split products); MAC on byte planes: f16 mma.sync.m16n8k16 on exact byte products; peaks "
+                        "measured with multipliers that change every step"}
 
     line = {
         "metric": METRIC, "value": round(ms, 3), "unit": "ms", "n_gpus": args.gpus, "steps": args.steps,
@@ -959,12 +944,6 @@ def prof_rev():
     return source_hash("mac_planes.cu", "mbar.cuh")
 
 
-def kernels_rev():
-    """Identity of all device code."""
-    return source_hash("kernels.cu", "transforms.cu", "tensor.cu", "relin.cu", "rns.cu", "client.cu", "mac_planes.cu",
-                       "ntt_block.cuh", "xform.cuh", "rns.cuh", "mbar.cuh", "common.cuh")
-
-
 def stored_counters(name, rev):
     """key=value fields of the machine-readable line of a committed ncu summary
     of the paper-shaped workload's kernels, if it was taken on the current
@@ -989,13 +968,6 @@ def stored_traffic():
         return None
     per_layer = (int(kv["traffic_bytes_per_launch"]) - int(kv["request_bytes"])) / int(kv["layers"])
     return int(round(per_layer * WL["mu"] + int(kv["request_bytes"])))
-
-
-def stored_pipe_cycles():
-    """Busy SM-cycles of the heavy multiply-add pipe per evaluation and kernel
-    class, from the committed full-size ncu summary."""
-    kv = stored_counters("circuit_pipes_paper.md", kernels_rev())
-    return kv and {c: int(v.split(",")[0]) for c, v in kv.items()}
 
 
 def main():
