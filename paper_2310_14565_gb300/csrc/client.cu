@@ -475,6 +475,27 @@ void launch_ptgen(const DevView& V, const uint16_t* pos, int L, int ell, int h, 
   in_form(V, [&](auto pm, auto ring) { go(k_ptgen<decltype(pm)::value, decltype(ring)::value>); });
 }
 
+int ptgen_layers(const DevView& V, int ell) {
+  const int chunks = (ell + ptgen_jc(V.N) - 1) / ptgen_jc(V.N);  // blocks of a layer
+  int per_sm = 1;
+  in_form(V, [&](auto pm, auto ring) {
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ptgen<decltype(pm)::value, decltype(ring)::value>,
+                                                  chain_threads(V.N), ptgen_smem(V.N));
+  });
+  const int slots = std::max(1, sm_count() * per_sm);
+  int best = 16;
+  double use = 0;
+  for (int L = 16; L <= 64; L += 16) {
+    const int blocks = L * chunks, waves = (blocks + slots - 1) / slots;
+    const double u = (double)blocks / ((double)waves * slots);
+    if (u > use + 0.02) {
+      use = u;
+      best = L;
+    }
+  }
+  return best;
+}
+
 void launch_valgen(const DevView& V, const u32* vals, int L, u64* VP, cudaStream_t st) {
   if (L <= 0) return;
   k_valgen<<<L, chain_threads(V.N), (size_t)V.N * 12, st>>>(V, vals, VP);

@@ -38,6 +38,9 @@ void launch_cw_unrank(const u64* T, size_t count, const u64* binom, int ell, int
 // Server plaintexts pt_s[l][j] in NTT form for L layers: P[L][ell][k][N], split operand format.
 void launch_ptgen(const DevView& V, const uint16_t* pos, int L, int ell, int h, u64* P, cudaStream_t st);
 
+// Layers (whole tiles of 16, at most 64) per launch of the above that leave the least of its last wave empty.
+int ptgen_layers(const DevView& V, int ell);
+
 // SMs of the current device.
 int sm_count();
 

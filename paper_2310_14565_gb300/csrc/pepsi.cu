@@ -1347,11 +1347,13 @@ int load_block(pepsi_ctx* c, std::vector<u64>&& hT, std::vector<uint32_t>* hV, u
                    reinterpret_cast<u64*>(S.dP) + (size_t)l0 * c->ell * k * N, c->stream);
     }
   } else if (S.mu_res) {
-    // the table, and words of up to one tile of layers to pack from (fewer when
-    // memory is short)
+    // the table, and words of some tiles of layers to pack from (fewer when memory
+    // is short): launches of one tile left a third of the generator's last wave
+    // empty at 363 bits and N = 8192 (74 layers: 31.6 ms a load, 28.7 by whole waves;
+    // 128 bits, 187 layers: 61.4 and 52.0 ms)
     const size_t per_layer = (size_t)c->ell * k * N;  // plaintext words of a layer
     u64* tmp = nullptr;
-    int G = (int)std::min<u32>(16, S.mu_res);
+    int G = (int)std::min<u32>(ptgen_layers(c->V, c->ell), S.mu_res);
     e = cudaMalloc((void**)&S.dP, (size_t)S.mu_res * plane_layer_bytes(c->ell, k * N, c->npl));
     if (e == cudaSuccess) {
       e = cudaMalloc((void**)&tmp, (size_t)G * per_layer * 8);
